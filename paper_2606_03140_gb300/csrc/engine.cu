@@ -427,7 +427,7 @@ sedacs_status flush_staged(sedacs_ctx* ctx) {
 sedacs_status build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode, double alpha, double beta,
                        bool b_from_sp2, bool a_from_sp2 = false, int c1 = -1, double g1 = 0.0, int c2 = -1,
                        double g2 = 0.0, bool c_from_sp2 = false, bool sym = false, int ca = 0, int cb = 0,
-                       int cout = 0, int cc1 = 0, int out2 = -1, int cout2 = 0) {
+                       int cout = 0, int cc1 = 0) {
   const Layout& L = ctx->lay;
   std::vector<GemmMat> mats(L.n_sub);
   std::vector<GemmWork> work;
@@ -441,7 +441,6 @@ sedacs_status build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode,
     m.out_off = mptr(ctx, out, i, cout);
     m.outp_off = ctx->f64 ? -1 : pptr_(ctx, out, i, cout);
     m.outp_plane = ctx->slot[out].plane_stride;
-    m.outp2_off = (out2 >= 0 && !ctx->f64) ? pptr_(ctx, out2, i, cout2) : -1;
     m.x_off = (mode == kModeRsp) ? mptr(ctx, kR2, i) : mptr(ctx, kX, i);
     m.c_off = (mode == kModeRsp) ? mptr(ctx, kR1, i) : (c1 >= 0 ? mptr(ctx, c1, i, cc1) : -1);
     m.c2_off = (c2 >= 0) ? mptr(ctx, c2, i) : -1;
@@ -484,16 +483,13 @@ sedacs_status build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode,
   op.n_work = (int)work.size();
   op.same_ab = (a == b && ca == cb && a_from_sp2 == b_from_sp2) ? 1 : 0;
   op.n_addends = (c1 >= 0 ? 1 : 0) + (c2 >= 0 ? 1 : 0);
-  op.dual = out2 >= 0 ? 1 : 0;
   op.alpha = alpha;
   op.beta = beta;
   op.g1 = g1;
   op.g2 = g2;
   op.mode = mode;
   op.sym = sym && !rows_out;
-  op.alpha2 = 0.0;
   op.ops_upper = 0;
-  op.store_upper = 0;
   return SEDACS_OK;
 }
 
@@ -512,11 +508,7 @@ void run_op(sedacs_ctx* ctx, int id, int nsplit_in, int nsplit_out) {
   p.beta = op.beta;
   p.g1 = op.g1;
   p.g2 = op.g2;
-  p.alpha2 = op.alpha2;
   p.ops_upper = op.ops_upper;
-  p.store_upper = op.store_upper;
-  // planes-only results exist in the fp16 two-plane path, whose outputs are read as planes
-  p.no_master = (!ctx->f64 && nsplit_in == kPlanesF16x2 && nsplit_out == kPlanesF16x2) ? op.no_master : 0;
   if (ctx->f64) launch_gemm_f64(p, op.n_work, ctx->stream);
   else launch_gemm_tc(p, op.n_work, nsplit_in, ctx->stream);
   ctx->launches += op.n_work > 0 ? 1 : 0;
@@ -530,21 +522,9 @@ sedacs_status upload_vec(sedacs_ctx* ctx, T** dst, const std::vector<T>& v) {
   return SEDACS_OK;
 }
 
-// Coefficients of the polynomial sum_k c_k X^k of the inverse stage (X in kY0, X^2 in kY1).
-// V^2-stride scheme (degree 2M + 1): T_1 = c_2M+1 X X^2 + c_2M X^2 + c_2M-1 X + c_2M-2 I,
-// T_j = B_{M-j} + X^2 T_{j-1}, B_j = c_2j + c_2j+1 X.  V^3-stride scheme (degree 9): the product
-// X X^2 gives X^3 and T_1 = c_9 X^3 + c_8 X^2 + c_7 X + c_6 I, then T_2 = X^3 T_1 + c_5 X^2 + c_4 X +
-// c_3 I and r = X^3 T_2 + c_2 X^2 + c_1 X + c_0 I.
+// Coefficients of the polynomial sum_k c_k X^k of the inverse stage (X in kY0, X^2 in kY1), degree 2M + 1:
+// T_1 = c_2M+1 X X^2 + c_2M X^2 + c_2M-1 X + c_2M-2 I, T_j = B_{M-j} + X^2 T_{j-1}, B_j = c_2j + c_2j+1 X.
 void set_horner(sedacs_ctx* ctx, const double* c) {
-  if (ctx->fermi_v3) {
-    GemmOp& i3 = ctx->ops[OP_F_I3];
-    i3.alpha = 1.0; i3.alpha2 = c[9]; i3.beta = c[6]; i3.g1 = c[7]; i3.g2 = c[8];
-    GemmOp& i4 = ctx->ops[OP_F_I4];
-    i4.alpha = 1.0; i4.beta = c[3]; i4.g1 = c[4]; i4.g2 = c[5];
-    GemmOp& i5 = ctx->ops[OP_F_I5];
-    i5.alpha = 1.0; i5.beta = c[0]; i5.g1 = c[1]; i5.g2 = c[2];
-    return;
-  }
   const int M = ctx->fermi_m;
   GemmOp& t1 = ctx->ops[OP_F_IT1];
   t1.alpha = c[2 * M + 1];
@@ -565,12 +545,6 @@ void run_fop(sedacs_ctx* ctx, int id, int nin, int nout);
 // The inverse stage: V^2 = V V, then r(V) in the slot horner_slot(M) (kR1 copy 0 in the tensor forms).
 void run_inverse(sedacs_ctx* ctx, int nf) {
   run_fop(ctx, OP_F_V2, nf, nf);
-  if (ctx->fermi_v3) {
-    run_fop(ctx, OP_F_I3, nf, nf);
-    run_fop(ctx, OP_F_I4, nf, nf);
-    run_fop(ctx, OP_F_I5, nf, nf);
-    return;
-  }
   run_fop(ctx, OP_F_IT1, nf, nf);
   for (int j = 2; j <= ctx->fermi_m; ++j) run_fop(ctx, OP_F_IH0 + (j - 2), nf, nf);
 }
@@ -592,36 +566,38 @@ sedacs_status build_fermi_ops(sedacs_ctx* ctx) {
   const double* a = fermi_tanh(ctx);
   const double* c = fermi_inv(ctx);
   const bool T = true, F = false;
-  // start: Z2 = z z, Z4 = Z2 Z2
-  STCHK(build_op(ctx, OP_F_Z2, kP, kP, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
-  STCHK(build_op(ctx, OP_F_Z4, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
-  // q(Z2) = sum_k a_k Z2^k = B_0 + Z4 (B_1 + Z4 (... B_J)), B_j = a_2j + a_2j+1 Z2:
-  // T_1 = B_{J-1} + Z4 B_J = a_2J+1 (Z2 Z4) + a_2J Z4 + a_2J-1 Z2 + a_2J-2 I
-  STCHK(build_op(ctx, OP_F_ST1, kY0, kY1, horner_slot(1), kModeGeneric, a[2 * J + 1], a[2 * J - 2], F, F, kY1,
-                 a[2 * J], kY0, a[2 * J - 1], F, T));
-  // T_j = B_{J-j} + Z4 T_{j-1}
-  for (int j = 2; j <= J; ++j)
-    STCHK(build_op(ctx, OP_F_SH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
-                   a[2 * (J - j)], F, F, kY0, a[2 * (J - j) + 1], -1, 0.0, F, T));
-  // U_0 = z q into either copy of kX
-  for (int cu = 0; cu < 2; ++cu)
-    STCHK(build_op(ctx, OP_F_U0_0 + cu, kP, horner_slot(J), kX, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F,
-                   T, 0, 0, cu));
-  // doubling: V = U U (from either copy), V2 = V V
-  for (int cu = 0; cu < 2; ++cu)
-    STCHK(build_op(ctx, OP_F_V_0 + cu, kX, kX, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T, cu, cu, 0));
-  STCHK(build_op(ctx, OP_F_V2, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
-  // r(V) = sum_k c_k V^k = B_0 + V2 (B_1 + ... V2 B_M), B_j = c_2j + c_2j+1 V:
-  // T_1 = c_2M+1 (V V2) + c_2M V2 + c_2M-1 V + c_2M-2 I, T_j = B_{M-j} + V2 T_{j-1}
-  STCHK(build_op(ctx, OP_F_IT1, kY0, kY1, horner_slot(1), kModeGeneric, c[2 * M + 1], c[2 * M - 2], F, F, kY1,
-                 c[2 * M], kY0, c[2 * M - 1], F, T));
-  for (int j = 2; j <= M; ++j)
-    STCHK(build_op(ctx, OP_F_IH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
-                   c[2 * (M - j)], F, F, kY0, c[2 * (M - j) + 1], -1, 0.0, F, T));
-  // U' = 2 U r(V) into the other copy; the last doubling (from copy 1): F = U r(V) + I / 2
-  for (int cu = 0; cu < 2; ++cu)
-    STCHK(build_op(ctx, OP_F_UP_0 + cu, kX, horner_slot(M), kX, kModeGeneric, 2.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T,
-                   cu, 0, 1 - cu));
+  if (!ctx->chain) {                    // (chains describe their products when they run, see fermi_chain)
+    // start: Z2 = z z, Z4 = Z2 Z2
+    STCHK(build_op(ctx, OP_F_Z2, kP, kP, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
+    STCHK(build_op(ctx, OP_F_Z4, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
+    // q(Z2) = sum_k a_k Z2^k = B_0 + Z4 (B_1 + Z4 (... B_J)), B_j = a_2j + a_2j+1 Z2:
+    // T_1 = B_{J-1} + Z4 B_J = a_2J+1 (Z2 Z4) + a_2J Z4 + a_2J-1 Z2 + a_2J-2 I
+    STCHK(build_op(ctx, OP_F_ST1, kY0, kY1, horner_slot(1), kModeGeneric, a[2 * J + 1], a[2 * J - 2], F, F, kY1,
+                   a[2 * J], kY0, a[2 * J - 1], F, T));
+    // T_j = B_{J-j} + Z4 T_{j-1}
+    for (int j = 2; j <= J; ++j)
+      STCHK(build_op(ctx, OP_F_SH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
+                     a[2 * (J - j)], F, F, kY0, a[2 * (J - j) + 1], -1, 0.0, F, T));
+    // U_0 = z q into either copy of kX
+    for (int cu = 0; cu < 2; ++cu)
+      STCHK(build_op(ctx, OP_F_U0_0 + cu, kP, horner_slot(J), kX, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F,
+                     T, 0, 0, cu));
+    // doubling: V = U U (from either copy), V2 = V V
+    for (int cu = 0; cu < 2; ++cu)
+      STCHK(build_op(ctx, OP_F_V_0 + cu, kX, kX, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T, cu, cu, 0));
+    STCHK(build_op(ctx, OP_F_V2, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
+    // r(V) = sum_k c_k V^k = B_0 + V2 (B_1 + ... V2 B_M), B_j = c_2j + c_2j+1 V:
+    // T_1 = c_2M+1 (V V2) + c_2M V2 + c_2M-1 V + c_2M-2 I, T_j = B_{M-j} + V2 T_{j-1}
+    STCHK(build_op(ctx, OP_F_IT1, kY0, kY1, horner_slot(1), kModeGeneric, c[2 * M + 1], c[2 * M - 2], F, F, kY1,
+                   c[2 * M], kY0, c[2 * M - 1], F, T));
+    for (int j = 2; j <= M; ++j)
+      STCHK(build_op(ctx, OP_F_IH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
+                     c[2 * (M - j)], F, F, kY0, c[2 * (M - j) + 1], -1, 0.0, F, T));
+    // U' = 2 U r(V) into the other copy; the last doubling (from copy 1): F = U r(V) + I / 2
+    for (int cu = 0; cu < 2; ++cu)
+      STCHK(build_op(ctx, OP_F_UP_0 + cu, kX, horner_slot(M), kX, kModeGeneric, 2.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T,
+                     cu, 0, 1 - cu));
+  }
   STCHK(build_op(ctx, OP_F_FIN, kX, horner_slot(M), kX, kModeGeneric, 1.0, 0.5, F, F, -1, 0.0, -1, 0.0, F, T, 1, 0,
                  0));
   // s = F - F^2 without the cancellation of F - F F on the saturated levels: with V = U^2 and
@@ -629,8 +605,9 @@ sedacs_status build_fermi_ops(sedacs_ctx* ctx) {
   // with G = r - V r (small where F is 0 or 1)
   // (G goes to the Horner slot that does not hold r: kT for M even, kR1 copy 0 for M odd)
   const int gslot = horner_slot(M) == kT ? kR1 : kT;
-  STCHK(build_op(ctx, OP_F_G, kY0, horner_slot(M), gslot, kModeGeneric, -1.0, 0.0, F, F, horner_slot(M), 1.0, -1,
-                 0.0, F, T));
+  if (!ctx->chain)
+    STCHK(build_op(ctx, OP_F_G, kY0, horner_slot(M), gslot, kModeGeneric, -1.0, 0.0, F, F, horner_slot(M), 1.0,
+                   -1, 0.0, F, T));
   STCHK(build_op(ctx, OP_F_S, gslot, gslot, kR2, kModeGeneric, 0.25, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
   // core rows of F into the response slots: dT1 = Z_c F = F_c + E_z,c F
   STCHK(build_op(ctx, OP_F_FT1_0, kZ0, kX, kdT1, kModeGeneric, 1.0, 0.0, T, F, kX, 1.0, -1, 0.0, T));
@@ -662,43 +639,46 @@ sedacs_status build_fermi_ops(sedacs_ctx* ctx) {
   STCHK(build_op(ctx, OP_F_DW0, kdT4, kZ0, kdDw, kModeGeneric, 2.0, 0.0, F, F, kdT4, 2.0));
   STCHK(build_op(ctx, OP_F_DW1, kdT4, kZ1, kdDw, kModeGeneric, 2.0, 0.0, F, F, kdT4, 2.0));
   STCHK(build_op(ctx, OP_F_T2W, kdT4, kHt, kT2, kModeGeneric, 1.0, 0.0, F));
+  if (ctx->chain) {
+    // the recursion's last products read its results, kept as upper tiles; F and s are written in full
+    ctx->ops[OP_F_FIN].ops_upper = ctx->ops[OP_F_S].ops_upper = 1;
+    return SEDACS_OK;
+  }
   // mu shift at a saved stage: U' = U Q + tau Q (U in kY0, Q = (I + tau U)^-1 in the Horner slot)
   // into either copy of kX; tau is set in g1 at run time
   for (int cu = 0; cu < 2; ++cu)
     STCHK(build_op(ctx, OP_F_MOB_0 + cu, kY0, horner_slot(M), kX, kModeGeneric, 1.0, 0.0, F, F, horner_slot(M), 0.0,
                    -1, 0.0, F, T, 0, 0, cu));
-  // fp16 two-plane form: the degree-9 inverse in powers of V^3 (V in kY0, V^2 in kY1, V^3 in kT, T_1
-  // in kR1 copy 0, T_2 in kR1 copy 1, r in kR1 copy 0 = horner_slot(4)); coefficients set by
-  // set_horner.  Its two-output product stores upper tiles only, which that form's operands allow.
-  ctx->fermi_v3 = !ctx->f64 && ctx->nsplit_fermi == kPlanesF16x2;
-  if (ctx->fermi_v3) {
-    STCHK(build_op(ctx, OP_F_I3, kY0, kY1, kT, kModeGeneric, 1.0, 0.0, F, F, kY0, 0.0, kY1, 0.0, F, T, 0, 0, 0, 0,
-                   kR1, 0));
-    STCHK(build_op(ctx, OP_F_I4, kT, kR1, kR1, kModeGeneric, 1.0, 0.0, F, F, kY0, 0.0, kY1, 0.0, F, T, 0, 0, 1));
-    STCHK(build_op(ctx, OP_F_I5, kT, kR1, kR1, kModeGeneric, 1.0, 0.0, F, F, kY0, 0.0, kY1, 0.0, F, T, 0, 1, 0));
-  }
-  // fp16 two-plane form: the recursion's symmetric intermediates are stored as their upper tiles
-  // (operands read across the diagonal as transposes); F itself is written in full
-  if (ctx->nsplit_fermi == kPlanesF16x2 && !ctx->f64) {
-    const int ids[] = {OP_F_Z2, OP_F_Z4, OP_F_ST1, OP_F_SH0, OP_F_SH1, OP_F_SH2, OP_F_SH3, OP_F_U0_0, OP_F_U0_1,
-                       OP_F_V_0, OP_F_V_1, OP_F_V2, OP_F_IT1, OP_F_IH0, OP_F_IH1, OP_F_IH2, OP_F_IH3, OP_F_IH4,
-                       OP_F_IH5, OP_F_UP_0, OP_F_UP_1, OP_F_MOB_0, OP_F_MOB_1, OP_F_I3, OP_F_I4, OP_F_I5};
-    for (int id : ids) {
-      ctx->ops[id].ops_upper = 1;
-      ctx->ops[id].store_upper = 1;
-    }
-    ctx->ops[OP_F_FIN].ops_upper = 1;
-    ctx->ops[OP_F_G].ops_upper = ctx->ops[OP_F_G].store_upper = ctx->ops[OP_F_G].no_master = 1;
-    ctx->ops[OP_F_S].ops_upper = 1;                // s itself is written in full, as bf16 planes
-    // results read only as MMA operands keep no FP32 master: the tanh Horner sums and U_0, V^3 and
-    // T_2 of the inverse, and every U but the kept stage.  Masters stay where an epilogue adds the
-    // result: Z2, Z4, V, V^2 (kY0, kY1), the inverse's last sum r (the mu shift adds Q = r as
-    // tau Q) and the kept stage U_j (copied to kY0, whose master the shift's inverse adds).
-    const int pl[] = {OP_F_ST1, OP_F_SH0, OP_F_SH1, OP_F_SH2, OP_F_SH3, OP_F_U0_0, OP_F_U0_1, OP_F_I3, OP_F_I4,
-                      OP_F_UP_0, OP_F_UP_1, OP_F_MOB_0, OP_F_MOB_1};
-    for (int id : pl) ctx->ops[id].no_master = 1;
-  }
   set_horner(ctx, fermi_inv(ctx));
+  return SEDACS_OK;
+}
+
+// Tables of the product chains: upper tiles grouped by subgraph, windows of subgraphs.
+sedacs_status build_chain_tables(sedacs_ctx* ctx) {
+  const Layout& L = ctx->lay;
+  std::vector<ChainTile> tiles;
+  std::vector<int> first(L.n_sub + 1, 0);
+  for (int i = 0; i < L.n_sub; ++i) {
+    const int T = L.n_real[i] > 0 ? L.n_pad[i] / 128 : 0;
+    for (int tm = 0; tm < T; ++tm)
+      for (int tn = tm; tn < T; ++tn)
+        tiles.push_back(ChainTile{L.sq_off[i], i, tm, tn, L.n_pad[i], L.n_real[i], 0});
+    first[i + 1] = (int)tiles.size();
+  }
+  // windows of whole subgraphs with about equal tile counts
+  const int n = (int)tiles.size();
+  const int nw = std::max(1, (n + chain_window_tiles() / 2) / chain_window_tiles());
+  std::vector<int> win(1, 0);
+  for (int i = 0; i < L.n_sub; ++i)
+    if ((int)win.size() < nw && first[i + 1] > win.back() &&
+        (long long)first[i + 1] * nw >= (long long)n * (long long)win.size())
+      win.push_back(first[i + 1]);
+  if (win.back() < n) win.push_back(n);
+  ctx->n_ctiles = n;
+  ctx->n_cwin = (int)win.size() - 1;
+  STCHK(stage_vec(ctx, &ctx->d_ctiles, tiles));
+  STCHK(stage_vec(ctx, &ctx->d_cwin, win));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_cdone), sizeof(unsigned) * std::max(1, L.n_sub)));
   return SEDACS_OK;
 }
 
@@ -818,6 +798,7 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   STCHK(stage_vec(ctx, &ctx->d_n_pad, npad));
   STCHK(stage_vec(ctx, &ctx->d_n_real, nreal));
   STCHK(stage_vec(ctx, &ctx->d_n_diag, ndiag));
+  if (ctx->chain) STCHK(build_chain_tables(ctx));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_glo), sizeof(double) * std::max(1LL, rb)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_ghi), sizeof(double) * std::max(1LL, rb)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_bounds), sizeof(double) * 2 * std::max(1, P)));
@@ -1163,9 +1144,7 @@ void run_fop(sedacs_ctx* ctx, int id, int nin, int nout) {
     const GemmOp& op = ctx->ops[id];
     double bytes = -1.0;
     if (!ctx->f64 && nin == kPlanesF16x2 && op.sym) {
-      const int master = (nout == kPlanesF16x2 && op.no_master) ? 0 : 4;
-      const double per = 4.0 * (op.same_ab ? 1 : 2) + 4.0 * op.n_addends + (nout == 3 ? 6.0 : 4.0) + master +
-                         4.0 * op.dual;
+      const double per = 4.0 * (op.same_ab ? 1 : 2) + 4.0 * op.n_addends + (nout == 3 ? 6.0 : 4.0) + 4.0;
       bytes = per * ctx->sum_tri;
     }
     if ((int)ctx->kev_bytes.size() < (int)ctx->kev.size()) ctx->kev_bytes.resize(ctx->kev.size(), -1.0);
@@ -1228,33 +1207,168 @@ void mobius_coeffs(double tau, int d, double* c) {
   }
 }
 
-// The doublings k0 .. nd-1 from U_k0 in kX copy cu; the last writes F = (I + U) / 2 into copy 0.
-// The stage js (0 <= js < nd; -1: none) is copied into kR2 copy 1 before its doubling.
+// ---- the recursion as chains of products (chain.cu) -----------------------------------------------
+// A square slot's copy as operand or result of a chained product.
+struct SlotRef {
+  int slot, copy;
+};
+long long ref_planes(const sedacs_ctx* ctx, SlotRef r) {
+  const Slot& S = ctx->slot[r.slot];
+  return S.base + r.copy * S.copy_stride + S.master_bytes;
+}
+long long ref_master(const sedacs_ctx* ctx, SlotRef r) {
+  const Slot& S = ctx->slot[r.slot];
+  return S.base + r.copy * S.copy_stride;
+}
+
+struct FermiChain {
+  sedacs_ctx* ctx;
+  std::vector<ChainOp> ops;
+  explicit FermiChain(sedacs_ctx* c) : ctx(c) {}
+  // out = alpha A B (+ beta I); master: its FP32 master is written too (a later product adds it)
+  ChainOp& mul(SlotRef a, SlotRef b, SlotRef out, double alpha, double beta, bool master) {
+    ChainOp o{};
+    o.a = ref_planes(ctx, a);
+    o.b = ref_planes(ctx, b);
+    o.out = ref_planes(ctx, out);
+    o.outm = master ? ref_master(ctx, out) : -1;
+    o.out2 = o.c1 = o.c2 = -1;
+    o.alpha = (float)alpha;
+    o.beta = (float)beta;
+    ops.push_back(o);
+    return ops.back();
+  }
+  void add1(SlotRef c, double g) {
+    ops.back().c1 = ref_master(ctx, c);
+    ops.back().g1 = (float)g;
+  }
+  void add2(SlotRef c, double g) {
+    ops.back().c2 = ref_master(ctx, c);
+    ops.back().g2 = (float)g;
+  }
+  sedacs_status run();
+};
+
+// r(X) = sum_k c_k X^k into kR1 copy 0 (planes and, where later products add it, master), X in x with X^2
+// going to kY1.  Two-plane form, degree 9 in strides of X^3: the product X X^2 gives X^3 (kT) and T_1 = c_9
+// X^3 + c_8 X^2 + c_7 X + c_6 I (kR1 copy 0) in one, then T_2 = X^3 T_1 + c_5 X^2 + c_4 X + c_3 I (kR1 copy 1)
+// and r = X^3 T_2 + c_2 X^2 + c_1 X + c_0 I.  Three-plane form: Horner in X^2 as in set_horner.
+void chain_inverse(FermiChain& ch, SlotRef x, const double* c, bool master) {
+  const SlotRef x2{kY1, 0}, t{kT, 0}, r0{kR1, 0}, r1{kR1, 1};
+  ch.mul(x, x, x2, 1.0, 0.0, true);
+  if (ch.ctx->nsplit_fermi == kPlanesF16x2) {
+    ChainOp& o = ch.mul(x, x2, t, 1.0, c[6], false);
+    o.out2 = ref_planes(ch.ctx, r0);
+    o.alpha2 = (float)c[9];
+    ch.add1(x, c[7]);
+    ch.add2(x2, c[8]);
+    ch.mul(t, r0, r1, 1.0, c[3], false);
+    ch.add1(x, c[4]);
+    ch.add2(x2, c[5]);
+    ch.mul(t, r1, r0, 1.0, c[0], master);
+    ch.add1(x, c[1]);
+    ch.add2(x2, c[2]);
+    return;
+  }
+  const int M = ch.ctx->fermi_m;
+  ch.mul(x, x2, SlotRef{horner_slot(1), 0}, c[2 * M + 1], c[2 * M - 2], false);
+  ch.add1(x2, c[2 * M]);
+  ch.add2(x, c[2 * M - 1]);
+  for (int j = 2; j <= M; ++j) {
+    ch.mul(x2, SlotRef{horner_slot(j - 1), 0}, SlotRef{horner_slot(j), 0}, 1.0, c[2 * (M - j)], j == M && master);
+    ch.add1(x, c[2 * (M - j) + 1]);
+  }
+}
+
+// The doublings k0 .. nd-1 from U_k0 in u, up to r(V) of the last one (F itself is the product after the
+// chain).  U_js goes to kR2 copy 1, where it stays for mu shifts, with the master their inverse adds;
+// the others alternate between the copies of kX so that U_nd-1 is in copy 1.
+SlotRef chain_u_slot(int k, int nd, int js) {
+  if (k == js && k < nd - 1) return SlotRef{kR2, 1};
+  return SlotRef{kX, (nd - 1 - k) & 1 ? 0 : 1};
+}
+
+void chain_doublings(FermiChain& ch, int k0, int nd, int js, SlotRef u) {
+  const SlotRef v{kY0, 0}, r{horner_slot(ch.ctx->fermi_m), 0};
+  for (int k = k0; k < nd; ++k) {
+    ch.mul(u, u, v, 1.0, 0.0, true);
+    chain_inverse(ch, v, fermi_inv(ch.ctx), k == nd - 1);       // (G adds the last r)
+    if (k == nd - 1) break;
+    const SlotRef next = chain_u_slot(k + 1, nd, js);
+    ch.mul(u, r, next, 2.0, 0.0, k + 1 == js);
+    u = next;
+  }
+}
+
+// Launches the products in runs of at most kMaxChain, with the launch's time and work recorded when
+// kernel statistics are on (flops and bytes as in run_fop, summed over the products).
+sedacs_status FermiChain::run() {
+  cudaStream_t s = ctx->stream;
+  const bool f16 = ctx->nsplit_fermi == kPlanesF16x2;
+  ChainParams p{};
+  p.arena = ctx->arena;
+  p.tiles = ctx->d_ctiles;
+  p.win = ctx->d_cwin;
+  p.done = ctx->d_cdone;
+  p.err = ctx->d_err;
+  p.plane = ctx->slot[kX].plane_stride;
+  p.n_win = ctx->n_cwin;
+  for (size_t at = 0; at < ops.size(); at += kMaxChain) {
+    p.n_ops = (int)std::min<size_t>(kMaxChain, ops.size() - at);
+    double bytes = 0.0;
+    for (int k = 0; k < p.n_ops; ++k) {
+      const ChainOp& o = p.op[k] = ops[at + k];
+      const double per = 4.0 * (o.a == o.b ? 1 : 2) + 4.0 * ((o.c1 >= 0) + (o.c2 >= 0)) + 4.0 +
+                         (o.outm >= 0 ? 4.0 : 0.0) + (o.out2 >= 0 ? 4.0 : 0.0);
+      bytes += per * ctx->sum_tri;
+    }
+    const bool rec = ctx->kstats && ctx->kev_used + 2 <= (int)ctx->kev.size();
+    if (rec) cudaEventRecord(ctx->kev[ctx->kev_used], s);
+    CUCHK(launch_chain(p, f16 ? 2 : 3, ctx->n_ctiles, ctx->lay.n_sub, s));
+    ctx->launches += ctx->n_ctiles > 0 ? 1 : 0;
+    if (rec) {
+      cudaEventRecord(ctx->kev[ctx->kev_used + 1], s);
+      if ((int)ctx->kev_bytes.size() < (int)ctx->kev.size()) ctx->kev_bytes.resize(ctx->kev.size(), -1.0);
+      ctx->kev_bytes[ctx->kev_used] = f16 ? bytes : -1.0;
+      ctx->kev_used += 2;
+      ctx->k_flops += p.n_ops * ctx->sum_n3;
+      if (f16) ctx->k16_flops += p.n_ops * ctx->sum_n3;
+    }
+  }
+  ops.clear();
+  return SEDACS_OK;
+}
+
+// The last product F = U r(V) + I / 2 (U in kX copy 1) and the buffer index of F.
+void fermi_finish(sedacs_ctx* ctx) {
+  const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
+  run_fop(ctx, OP_F_FIN, nf, ctx->f64 ? 0 : 3);      // bf16 planes
+  launch_buffer_index(ctx->d_sp2, 0, ctx->lay.n_sub, ctx->stream);
+  ctx->launches += 1;
+}
+
+void copy_u(sedacs_ctx* ctx, int to_slot, int to_copy, int from_slot, int from_copy) {
+  const Slot& T = ctx->slot[to_slot];
+  const Slot& F = ctx->slot[from_slot];
+  cudaMemcpyAsync(ctx->arena + T.base + (long long)to_copy * T.copy_stride,
+                  ctx->arena + F.base + (long long)from_copy * F.copy_stride, (size_t)F.copy_stride,
+                  cudaMemcpyDeviceToDevice, ctx->stream);
+}
+
+// The doublings k0 .. nd-1 from U_k0 in kX copy cu, one launch per product (FP64 and the diagnostic forms);
+// the last writes F = (I + U) / 2 into copy 0.  The stage js (0 <= js < nd; -1: none) is copied into kR2
+// copy 1 before its doubling.
 void fermi_doublings_from(sedacs_ctx* ctx, int k0, int nd, int cu, int js) {
   const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
   for (int k = k0; k < nd; ++k) {
-    if (k == js) {
-      const Slot& X = ctx->slot[kX];
-      const Slot& Sv = ctx->slot[kR2];
-      cudaMemcpyAsync(ctx->arena + Sv.base + Sv.copy_stride, ctx->arena + X.base + (long long)cu * X.copy_stride,
-                      (size_t)X.copy_stride, cudaMemcpyDeviceToDevice, ctx->stream);
-    }
+    if (k == js) copy_u(ctx, kR2, 1, kX, cu);
     run_fop(ctx, OP_F_V_0 + cu, nf, nf);
     run_inverse(ctx, nf);
-    if (k == nd - 1) {
-      run_fop(ctx, OP_F_FIN, nf, ctx->f64 ? 0 : 3);    // cu == 1 here: F = U r(V) + I / 2, bf16 planes
-    } else {
-      // the U that becomes the kept stage carries its FP32 master: the mu shift's inverse adds it
-      GemmOp& up = ctx->ops[OP_F_UP_0 + cu];
-      const int nm = up.no_master;
-      if (k + 1 == js) up.no_master = 0;
-      run_fop(ctx, OP_F_UP_0 + cu, nf, nf);
-      up.no_master = nm;
-      cu = 1 - cu;
-    }
+    if (k == nd - 1) break;                            // cu == 1 here
+    run_fop(ctx, OP_F_UP_0 + cu, nf, nf);
+    cu = 1 - cu;
   }
-  launch_buffer_index(ctx->d_sp2, 0, ctx->lay.n_sub, ctx->stream);
-  ctx->launches += 1;
+  fermi_finish(ctx);
 }
 
 // Doublings redone from the kept stage after a mu shift (see fermi_reentry).
@@ -1262,7 +1376,7 @@ constexpr int kReentryStages = 3;
 
 // One pass: F at (mu, beta) into kX copy 0, every buffer index pointing there; the stage
 // nd - kReentryStages is kept for mu shifts.
-void run_fermi(sedacs_ctx* ctx, double mu, int nd) {
+sedacs_status run_fermi(sedacs_ctx* ctx, double mu, int nd) {
   cudaStream_t s = ctx->stream;
   const Layout& L = ctx->lay;
   const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
@@ -1270,23 +1384,42 @@ void run_fermi(sedacs_ctx* ctx, double mu, int nd) {
   launch_affine_planes(ctx->d_views[kHt], ctx->d_views[kP], -0.5 * b0, 0.5 * b0 * mu, ctx->f64 ? 1 : 0, nf, nullptr,
                        0.0, 0.0, 0, 0, 0, nullptr, L.n_sub, max_rows(ctx), ctx->arena, ctx->f64, s);   // z
   ctx->launches += 1;
-  run_fop(ctx, OP_F_Z2, nf, nf);
-  run_fop(ctx, OP_F_Z4, nf, nf);
-  run_fop(ctx, OP_F_ST1, nf, nf);
-  for (int j = 2; j <= ctx->fermi_j; ++j) run_fop(ctx, OP_F_SH0 + (j - 2), nf, nf);
-  // U_0 goes to the copy from which n doublings end in copy 0
-  const int cu = nd & 1;
   const int js = std::max(0, nd - kReentryStages);
-  GemmOp& u0 = ctx->ops[OP_F_U0_0 + cu];
-  const int nm = u0.no_master;
-  if (js == 0) u0.no_master = 0;                   // U_0 is the kept stage (see fermi_doublings_from)
-  run_fop(ctx, OP_F_U0_0 + cu, nf, nf);
-  u0.no_master = nm;
-  fermi_doublings_from(ctx, 0, nd, cu, js);
+  if (ctx->chain) {
+    FermiChain ch(ctx);
+    const double* a = fermi_tanh(ctx);
+    const int J = ctx->fermi_j;
+    const SlotRef z{kP, 0}, z2{kY0, 0}, z4{kY1, 0};
+    ch.mul(z, z, z2, 1.0, 0.0, true);
+    ch.mul(z2, z2, z4, 1.0, 0.0, true);
+    ch.mul(z2, z4, SlotRef{horner_slot(1), 0}, a[2 * J + 1], a[2 * J - 2], false);
+    ch.add1(z4, a[2 * J]);
+    ch.add2(z2, a[2 * J - 1]);
+    for (int j = 2; j <= J; ++j) {
+      ch.mul(z4, SlotRef{horner_slot(j - 1), 0}, SlotRef{horner_slot(j), 0}, 1.0, a[2 * (J - j)], false);
+      ch.add1(z2, a[2 * (J - j) + 1]);
+    }
+    const SlotRef u0 = chain_u_slot(0, nd, js);
+    ch.mul(z, SlotRef{horner_slot(J), 0}, u0, 1.0, 0.0, js == 0);
+    chain_doublings(ch, 0, nd, js, u0);
+    STCHK(ch.run());
+    if (js == nd - 1) copy_u(ctx, kR2, 1, kX, 1);      // a single doubling: its U is both operand and kept stage
+    fermi_finish(ctx);
+  } else {
+    run_fop(ctx, OP_F_Z2, nf, nf);
+    run_fop(ctx, OP_F_Z4, nf, nf);
+    run_fop(ctx, OP_F_ST1, nf, nf);
+    for (int j = 2; j <= ctx->fermi_j; ++j) run_fop(ctx, OP_F_SH0 + (j - 2), nf, nf);
+    // U_0 goes to the copy from which n doublings end in copy 0
+    const int cu = nd & 1;
+    run_fop(ctx, OP_F_U0_0 + cu, nf, nf);
+    fermi_doublings_from(ctx, 0, nd, cu, js);
+  }
   ctx->fermi_n = nd;
   ctx->fermi_saved_mu = mu;
   ctx->fermi_saved_j = js;
   ctx->fermi_saved_nd = nd;
+  return SEDACS_OK;
 }
 
 // Largest |beta dmu| handled by a shift at the kept stage: |tau| <= 0.2 (0.3 in FP64, whose
@@ -1301,24 +1434,33 @@ double reentry_reach(const sedacs_ctx* ctx) {
 // U_j' = (U_j + tau I)(I + tau U_j)^-1 with tau = tanh(beta_j (mu - mu_s) / 2), the inverse being a
 // polynomial in U_j (Chebyshev interpolant of 1 / (1 + tau u) on [-1, 1]); the remaining doublings
 // then run as in a full pass.
-void fermi_reentry(sedacs_ctx* ctx, double mu) {
+sedacs_status fermi_reentry(sedacs_ctx* ctx, double mu) {
   const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
   const int nd = ctx->fermi_saved_nd, js = ctx->fermi_saved_j, S = nd - js;
   const double tau = std::tanh(0.5 * std::ldexp(beta_of(ctx), -S) * (mu - ctx->fermi_saved_mu));
-  const Slot& Y = ctx->slot[kY0];
-  const Slot& Sv = ctx->slot[kR2];
-  cudaMemcpyAsync(ctx->arena + Y.base, ctx->arena + Sv.base + Sv.copy_stride, (size_t)Y.copy_stride,
-                  cudaMemcpyDeviceToDevice, ctx->stream);
   double c[16];
-  mobius_coeffs(tau, ctx->fermi_v3 ? 9 : 2 * ctx->fermi_m + 1, c);
-  set_horner(ctx, c);
-  run_inverse(ctx, nf);                              // Q = (I + tau U_j)^-1
-  set_horner(ctx, fermi_inv(ctx));
-  const int cu = S & 1;                              // S doublings then end in copy 0
-  ctx->ops[OP_F_MOB_0 + cu].g1 = tau;
-  run_fop(ctx, OP_F_MOB_0 + cu, nf, nf);             // U_j' = U_j Q + tau Q
-  fermi_doublings_from(ctx, js, nd, cu, -1);
+  mobius_coeffs(tau, 2 * ctx->fermi_m + 1, c);
+  if (ctx->chain) {
+    FermiChain ch(ctx);
+    const SlotRef u{kR2, 1}, q{horner_slot(ctx->fermi_m), 0}, u1 = chain_u_slot(js, nd, -1);
+    chain_inverse(ch, u, c, true);                     // Q = (I + tau U_j)^-1
+    ch.mul(u, q, u1, 1.0, 0.0, false);                 // U_j' = U_j Q + tau Q
+    ch.add1(q, tau);
+    chain_doublings(ch, js, nd, -1, u1);
+    STCHK(ch.run());
+    fermi_finish(ctx);
+  } else {
+    copy_u(ctx, kY0, 0, kR2, 1);
+    set_horner(ctx, c);
+    run_inverse(ctx, nf);
+    set_horner(ctx, fermi_inv(ctx));
+    const int cu = S & 1;                              // S doublings then end in copy 0
+    ctx->ops[OP_F_MOB_0 + cu].g1 = tau;
+    run_fop(ctx, OP_F_MOB_0 + cu, nf, nf);
+    fermi_doublings_from(ctx, js, nd, cu, -1);
+  }
   ctx->fermi_n = nd;
+  return SEDACS_OK;
 }
 
 // Populations of the core rows at dc_off (per atom, the FP64 sum over each core atom's orbitals
@@ -1335,13 +1477,22 @@ void core_pops(sedacs_ctx* ctx, const long long* dc_off, double* pop, double* eb
 
 // s = F - F^2 (as G^2 / 4 from the last doubling's V and r, still in kY0 and the Horner slot) and
 // the core rows D_s = 2 Z_c s Z (kdT1 -> kdDc); d/dmu of F is beta s.
-void fermi_s_rows(sedacs_ctx* ctx) {
+sedacs_status fermi_s_rows(sedacs_ctx* ctx) {
   const int ns = ctx->nsplit_ns;
   const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
-  run_fop(ctx, OP_F_G, nf, nf);
+  if (ctx->chain) {
+    FermiChain ch(ctx);
+    const SlotRef v{kY0, 0}, r{horner_slot(ctx->fermi_m), 0};
+    ch.mul(v, r, SlotRef{kT, 0}, -1.0, 0.0, false);
+    ch.add1(r, 1.0);
+    STCHK(ch.run());
+  } else {
+    run_fop(ctx, OP_F_G, nf, nf);
+  }
   run_fop(ctx, OP_F_S, nf, ctx->f64 ? 0 : 3);
   run_op(ctx, ctx->zc == 0 ? OP_DT1_0 : OP_DT1_1, 3, ns);
   run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);
+  return SEDACS_OK;
 }
 
 // t = s (I - 2F) and its core rows D_t = 2 Z_c t Z (kdT2 -> kdDt); d^2 F / dmu^2 is beta^2 t.
@@ -1426,16 +1577,16 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
   while (!done && pass < 80) {
     ++pass;
     if (have_stage && std::fabs(beta * (mu - ctx->fermi_saved_mu)) <= reentry_reach(ctx)) {
-      fermi_reentry(ctx, mu);                                     // shift at the kept stage
+      STCHK(fermi_reentry(ctx, mu));                              // shift at the kept stage
       ctx->fermi_reentries += 1;
     } else {
-      run_fermi(ctx, mu, fermi_doublings(ctx, mu));
+      STCHK(run_fermi(ctx, mu, fermi_doublings(ctx, mu)));
       have_stage = true;
     }
     back_transform(ctx, false);                                   // T1 = Z_c F, D_c
     if (given) { done = true; break; }
     core_pops(ctx, ctx->d_dcoff, ctx->d_pop, ctx->d_eband, 9);     // N(mu)
-    fermi_s_rows(ctx);
+    STCHK(fermi_s_rows(ctx));
     core_pops(ctx, ctx->d_dcoff_d, pop_s, scr, 10);                // sum of D_s populations
     fermi_t_rows(ctx);
     core_pops(ctx, ctx->d_dcoff_t, pop_t, scr, 14);                // sum of D_t populations
@@ -1776,11 +1927,11 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
     ctx->launches += 1;
     gather_hs(ctx, Vp);
     compute_ht(ctx);
-    run_fermi(ctx, ctx->mu, nd);
+    STCHK(run_fermi(ctx, ctx->mu, nd));
     run_op(ctx, ctx->zc == 0 ? OP_F_FT1_0 : OP_F_FT1_1, 3, ns);   // dT1 = Z_c F
     run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);         // 2 dT1 Z
     core_pops(ctx, ctx->d_dcoff_d, q, eb, 9);
-    fermi_s_rows(ctx);
+    STCHK(fermi_s_rows(ctx));
     core_pops(ctx, ctx->d_dcoff_d, ps, eb, 10);
     double sc[2];
     CUCHK(cudaMemcpyAsync(sc, ctx->d_scal + 9, sizeof(sc), cudaMemcpyDeviceToHost, s));
@@ -1990,6 +2141,7 @@ sedacs_status sedacs_create(int32_t n_atoms, const int32_t* species, const doubl
   ctx->nsplit_sp2 = sp2_fmt[params->precision];
   ctx->nsplit_rsp = ctx->nsplit_sp2 == kPlanesF16x2 ? 3 : ctx->nsplit_sp2;
   ctx->nsplit_fermi = ctx->nsplit_sp2;
+  ctx->chain = !ctx->f64 && (ctx->nsplit_fermi == kPlanesF16x2 || ctx->nsplit_fermi == 3);
   if (ctx->f64) ctx->nsplit_sp2 = 3;
   const int N = n_atoms;
   auto fail = [&](sedacs_status st, const char* msg) {
@@ -2039,7 +2191,8 @@ void sedacs_destroy(sedacs_ctx* ctx) {
                   ctx->d_views_x1, ctx->d_hoff, ctx->d_soff, ctx->d_dcoff, ctx->d_wcoff, ctx->d_rowbase,
                   ctx->d_tr_off, ctx->d_n_pad, ctx->d_n_real, ctx->d_n_diag, ctx->d_glo, ctx->d_ghi, ctx->d_bounds,
                   ctx->d_slots, ctx->d_sp2, ctx->d_nactive, ctx->d_dcoff_d, ctx->d_dqpop, ctx->d_dhoff,
-                  ctx->d_steps, ctx->d_rsp, ctx->d_dcoff_t, ctx->d_dcoff_u, ctx->d_dcoff_w};
+                  ctx->d_steps, ctx->d_rsp, ctx->d_dcoff_t, ctx->d_dcoff_u, ctx->d_dcoff_w, ctx->d_ctiles,
+                  ctx->d_cwin, ctx->d_cdone};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto* v : ctx->d_views)

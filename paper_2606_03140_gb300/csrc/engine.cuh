@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/sedacs.h"
+#include "chain.cuh"
 #include "dense.cuh"
 #include "dense_ops.cuh"
 #include "ewald.cuh"
@@ -41,15 +42,12 @@ struct GemmOp {
   GemmMat* mats_d = nullptr;
   GemmWork* work_d = nullptr;
   int n_work = 0;
-  double alpha = 1.0, beta = 0.0, g1 = 0.0, g2 = 0.0, alpha2 = 0.0;
+  double alpha = 1.0, beta = 0.0, g1 = 0.0, g2 = 0.0;
   int mode = kModeGeneric;
   bool sym = false;          // symmetric output: upper tiles only (counted as n^3 flops)
-  int ops_upper = 0;         // operands stored as upper tiles (fp16 two-plane path)
-  int store_upper = 0;       // result stored as upper tiles (no mirror)
-  int no_master = 0;         // fp16 two-plane path: result kept as planes only (no FP32 master)
+  int ops_upper = 0;         // operands stored as upper tiles (results of a chain)
   int same_ab = 0;           // A and B are one matrix (read once)
   int n_addends = 0;         // C1 / C2 added in the epilogue (FP32 masters)
-  int dual = 0;              // second output (planes)
 };
 
 enum OpId : int {
@@ -74,9 +72,6 @@ enum OpId : int {
   OP_F_T, OP_F_TT1_0, OP_F_TT1_1, OP_F_DT0, OP_F_DT1, OP_F_T2T,
   // mu shift at a saved doubling stage: U' = U Q + tau Q, Q ~ (I + tau U)^-1 (U in kY0), into kX
   OP_F_MOB_0, OP_F_MOB_1,
-  // degree-9 inverse in powers of V^3 (fp16 two-plane form): [V^3 | T_1] from one product V V^2 (two
-  // outputs), T_2 = V^3 T_1 + B_1, r = V^3 T_2 + B_0
-  OP_F_I3, OP_F_I4, OP_F_I5,
   // third- and fourth-order mu terms: P = t F (kT), u = t - 2 P - 2 s s (kY0), its core rows
   // (kdT3, kdDu), T2 = kdT3 h~; Q = u F (kT), w = u - 2 Q - 6 s t (kY1), rows (kdT4, kdDw), T2
   OP_F_TF, OP_F_U, OP_F_UT1_0, OP_F_UT1_1, OP_F_DU0, OP_F_DU1, OP_F_T2U,
@@ -135,10 +130,16 @@ struct sedacs_ctx {
   int nsplit_rsp = 3;    // plane format of the first-order SP2 replay (X and dX): fp16 two-plane
                          // SP2 forms replay in three bf16 planes (dX can exceed the fp16 range)
   int nsplit_fermi = 3;  // plane format of the finite-temperature Fermi recursion's products
+  // the recursion's products run as chains (chain.cu) in the fp16 two-plane and three-plane bf16 forms: tables
+  // of the current layout
+  bool chain = false;
+  sedacs::ChainTile* d_ctiles = nullptr;
+  int* d_cwin = nullptr;
+  unsigned* d_cdone = nullptr;
+  int n_ctiles = 0, n_cwin = 0;
   // finite-temperature Fermi operator: degrees of its two polynomials (kTanh*, kInv*), the
   // tanh doublings of the last pass, and the diagnostics of the last density call
   int fermi_j = 3, fermi_m = 4;   // Horner lengths (start: Z4 steps; inverse: V2 steps)
-  bool fermi_v3 = false;          // inverse by the V^3-stride scheme with the two-output product
   int fermi_n = 0;                // doublings of the last pass
   double fermi_count_err = 0.0;   // collected count minus N_e after the mu solve
   double fermi_dndmu = 0.0;       // dN/dmu at the accepted pass (e / Ha)
