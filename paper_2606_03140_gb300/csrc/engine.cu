@@ -2211,7 +2211,7 @@ void sedacs_destroy(sedacs_ctx* ctx) {
   if (ctx->stage_pinned) cudaFreeHost(ctx->stage_pinned);
   GnnState& G = ctx->gnn;
   for (void* p : {(void*)G.P, (void*)G.grad, (void*)G.m, (void*)G.v, (void*)G.act, (void*)G.part, (void*)G.ebas,
-                  (void*)G.gu, (void*)G.u, (void*)G.pX, (void*)G.pV})
+                  (void*)G.gu, (void*)G.u, (void*)G.p64, (void*)G.pX, (void*)G.pV})
     if (p) cudaFree(p);
   delete ctx;
 }
@@ -2925,12 +2925,10 @@ int32_t sedacs_gnn_num_params(void) { return gnn_num_params(); }
 sedacs_status sedacs_gnn_set_params(sedacs_ctx* ctx, const double* p) {
   if (!ctx || !p) return SEDACS_EINVAL;
   CUCHK(gnn_prepare_params(ctx));
-  double* tmp = nullptr;
-  CUCHK(cudaMalloc(&tmp, sizeof(double) * gnn_num_params()));
-  cudaMemcpyAsync(tmp, p, sizeof(double) * gnn_num_params(), cudaMemcpyDefault, ctx->stream);
+  double* tmp = ctx->gnn.p64;
+  CUCHK(cudaMemcpyAsync(tmp, p, sizeof(double) * gnn_num_params(), cudaMemcpyDefault, ctx->stream));
   gnn_set_params_f64(ctx, tmp);
-  cudaStreamSynchronize(ctx->stream);
-  cudaFree(tmp);
+  CUCHK(cudaStreamSynchronize(ctx->stream));
   ctx->gnn.t = 0;
   cudaMemsetAsync(ctx->gnn.m, 0, sizeof(float) * gnn_num_params(), ctx->stream);
   cudaMemsetAsync(ctx->gnn.v, 0, sizeof(float) * gnn_num_params(), ctx->stream);
@@ -2940,12 +2938,10 @@ sedacs_status sedacs_gnn_set_params(sedacs_ctx* ctx, const double* p) {
 sedacs_status sedacs_gnn_get_params(sedacs_ctx* ctx, double* p, int32_t grad) {
   if (!ctx || !p) return SEDACS_EINVAL;
   CUCHK(gnn_prepare_params(ctx));
-  double* tmp = nullptr;
-  CUCHK(cudaMalloc(&tmp, sizeof(double) * gnn_num_params()));
+  double* tmp = ctx->gnn.p64;
   gnn_get_params_f64(ctx, tmp, grad != 0);
-  cudaMemcpyAsync(p, tmp, sizeof(double) * gnn_num_params(), cudaMemcpyDefault, ctx->stream);
-  cudaStreamSynchronize(ctx->stream);
-  cudaFree(tmp);
+  CUCHK(cudaMemcpyAsync(p, tmp, sizeof(double) * gnn_num_params(), cudaMemcpyDefault, ctx->stream));
+  CUCHK(cudaStreamSynchronize(ctx->stream));
   return SEDACS_OK;
 }
 

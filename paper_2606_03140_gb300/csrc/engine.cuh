@@ -88,6 +88,7 @@ struct GnnState {
   int nchunk = 0;
   int t = 0;                 // Adam step count
   double *gu = nullptr, *u = nullptr;
+  double* p64 = nullptr;     // the FP64 parameter or gradient vector at the boundary
   bool collect = false;      // store (J v, v) pairs produced by the Krylov kernel
   double *pX = nullptr, *pV = nullptr;
   int pairs = 0, pair_cap = 0, pair_head = 0;
