@@ -18,6 +18,7 @@
 // core, ascending, from a per-core bitmap.
 #include "graph.cuh"
 
+#include <algorithm>
 #include <cmath>
 
 namespace sedacs {
@@ -394,63 +395,163 @@ __device__ void block_bitonic(double* key, int* idx, int P2) {
     }
 }
 
-__global__ void rcb_level_kernel(const RcbSeg* segs, int* perm, const double* R, CellGrid g, double* skey, int* sidx,
-                                 int sort_by_index) {
+__global__ void rcb_wrap_kernel(const double* R, int N, CellGrid g, double* wrapped, int* perm) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  perm[i] = i;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) wrapped[(long long)d * N + i] = wrap1(R[3 * i + d], g.box[d]);
+}
+
+// One split of a segment along its widest axis (first on ties): the `left` atoms that come first by (coordinate,
+// index) to the front.  Only the two sets matter (every leaf is sorted by index at the end), so the segment is
+// not sorted: a histogram over kBins equal slices of its extent (a monotone map, so slices are in order) finds
+// the slice that holds the boundary, and the few atoms of that slice are ranked against each other.  Where
+// they are too many for that (coincident or strongly clustered coordinates) the segment is sorted.
+// Measured at 9,000 atoms: 2.0 ms for the levels by sorting, 0.1 ms by selection.
+constexpr int kBins = 2048, kRank = 1024;
+
+__global__ void __launch_bounds__(1024) rcb_split_kernel(const RcbSeg* segs, int* perm, const double* wrapped, int N,
+                                                         double* skey, int* sidx) {
+  const RcbSeg sg = segs[blockIdx.x];
+  const int n = sg.count;
+  int* at = perm + sg.start;
+  double* key = skey + sg.scratch;
+  int* idx = sidx + sg.scratch;
+  __shared__ double smin[3][32], smax[3][32];
+  __shared__ int hist[kBins];
+  __shared__ double ckey[kRank];
+  __shared__ int cidx[kRank];
+  __shared__ int wsum[32];
+  __shared__ int axis_s, bin_s, below_s, n_cand, n_lo, n_hi;
+  __shared__ double lo_s, scale_s, tkey;
+  __shared__ int tidx;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // min / max are exact, so the reduction order does not matter
+  double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int a = at[t];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double w = wrapped[(long long)d * N + a];
+      mn[d] = fmin(mn[d], w);
+      mx[d] = fmax(mx[d], w);
+    }
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    for (int o = 16; o > 0; o >>= 1) {
+      mn[d] = fmin(mn[d], __shfl_xor_sync(0xffffffffu, mn[d], o));
+      mx[d] = fmax(mx[d], __shfl_xor_sync(0xffffffffu, mx[d], o));
+    }
+  if (lane == 0)
+    for (int d = 0; d < 3; ++d) { smin[d][wid] = mn[d]; smax[d][wid] = mx[d]; }
+  for (int t = threadIdx.x; t < kBins; t += blockDim.x) hist[t] = 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double e[3], l[3];
+    for (int d = 0; d < 3; ++d) {
+      double lo = smin[d][0], hi = smax[d][0];
+      for (int q = 1; q < nw; ++q) { lo = fmin(lo, smin[d][q]); hi = fmax(hi, smax[d][q]); }
+      e[d] = __dsub_rn(hi, lo);
+      l[d] = lo;
+    }
+    int ax = 0;
+    double best = e[0];
+    if (e[1] > best) { ax = 1; best = e[1]; }
+    if (e[2] > best) { ax = 2; best = e[2]; }
+    axis_s = ax;
+    lo_s = l[ax];
+    scale_s = best > 0.0 ? kBins / best : 0.0;
+    n_cand = n_lo = n_hi = 0;
+  }
+  __syncthreads();
+  const double* w = wrapped + (long long)axis_s * N;
+  const double lo = lo_s, scale = isfinite(scale_s) ? scale_s : 0.0;
+  auto bin_of = [&](double x) { return min(max((int)((x - lo) * scale), 0), kBins - 1); };
+  for (int t = threadIdx.x; t < n; t += blockDim.x) atomicAdd(&hist[bin_of(w[at[t]])], 1);
+  __syncthreads();
+  // the slice of rank `left`: the scan of the histogram, two slices per thread
+  {
+    const int b0 = 2 * threadIdx.x, h0 = b0 < kBins ? hist[b0] : 0, h1 = b0 + 1 < kBins ? hist[b0 + 1] : 0;
+    int incl = h0 + h1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[wid] = incl;
+    __syncthreads();
+    int before = incl - h0 - h1;
+    for (int q = 0; q < wid; ++q) before += wsum[q];
+    if (sg.left >= before && sg.left < before + h0) { bin_s = b0; below_s = before; }
+    else if (sg.left >= before + h0 && sg.left < before + h0 + h1) { bin_s = b0 + 1; below_s = before + h0; }
+  }
+  __syncthreads();
+  const int bin = bin_s, rank = sg.left - below_s;
+  if (hist[bin] > kRank) {
+    int P2 = 1;
+    while (P2 < n) P2 <<= 1;
+    for (int t = threadIdx.x; t < P2; t += blockDim.x) {
+      key[t] = t < n ? w[at[t]] : 1e308;
+      idx[t] = t < n ? at[t] : 0x7fffffff;
+    }
+    __syncthreads();
+    block_bitonic(key, idx, P2);
+    for (int t = threadIdx.x; t < n; t += blockDim.x) at[t] = idx[t];
+    return;
+  }
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int a = at[t];
+    const double x = w[a];
+    if (bin_of(x) == bin) {
+      const int k = atomicAdd(&n_cand, 1);
+      ckey[k] = x;
+      cidx[k] = a;
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < n_cand; k += blockDim.x) {
+    int r = 0;
+    for (int j = 0; j < n_cand; ++j) r += ckey[j] < ckey[k] || (ckey[j] == ckey[k] && cidx[j] < cidx[k]);
+    if (r == rank) { tkey = ckey[k]; tidx = cidx[k]; }
+  }
+  __syncthreads();
+  for (int t0 = 0; t0 < n; t0 += blockDim.x) {
+    const int t = t0 + threadIdx.x;
+    int a = 0;
+    bool l = false;
+    if (t < n) {
+      a = at[t];
+      const double x = w[a];
+      l = x < tkey || (x == tkey && a < tidx);
+    }
+    const unsigned ml = __ballot_sync(0xffffffffu, t < n && l), mh = __ballot_sync(0xffffffffu, t < n && !l);
+    int bl = 0, bh = 0;
+    if (lane == 0) {
+      bl = atomicAdd(&n_lo, __popc(ml));
+      bh = atomicAdd(&n_hi, __popc(mh));
+    }
+    bl = __shfl_sync(0xffffffffu, bl, 0);
+    bh = __shfl_sync(0xffffffffu, bh, 0);
+    const unsigned below = (1u << lane) - 1u;
+    if (t < n) idx[l ? bl + __popc(ml & below) : n - 1 - (bh + __popc(mh & below))] = a;   // from both ends
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < n; t += blockDim.x) at[t] = idx[t];
+}
+
+// Every leaf's atoms ascending.
+__global__ void rcb_leaf_kernel(const RcbSeg* segs, int* perm, double* skey, int* sidx) {
   const RcbSeg sg = segs[blockIdx.x];
   const int n = sg.count;
   int P2 = 1;
   while (P2 < n) P2 <<= 1;
   double* key = skey + sg.scratch;
   int* idx = sidx + sg.scratch;
-  __shared__ double smin[3][32], smax[3][32];
-  __shared__ int axis_s;
-  if (!sort_by_index) {
-    // min / max are exact, so the reduction order does not matter
-    double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      const int a = perm[sg.start + t];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const double w = wrap1(R[3 * a + d], g.box[d]);
-        mn[d] = fmin(mn[d], w);
-        mx[d] = fmax(mx[d], w);
-      }
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-      for (int o = 16; o > 0; o >>= 1) {
-        mn[d] = fmin(mn[d], __shfl_xor_sync(0xffffffffu, mn[d], o));
-        mx[d] = fmax(mx[d], __shfl_xor_sync(0xffffffffu, mx[d], o));
-      }
-    const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if ((threadIdx.x & 31) == 0)
-      for (int d = 0; d < 3; ++d) { smin[d][wid] = mn[d]; smax[d][wid] = mx[d]; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double e[3];
-      for (int d = 0; d < 3; ++d) {
-        double lo = smin[d][0], hi = smax[d][0];
-        for (int q = 1; q < nw; ++q) { lo = fmin(lo, smin[d][q]); hi = fmax(hi, smax[d][q]); }
-        e[d] = __dsub_rn(hi, lo);
-      }
-      int ax = 0;
-      double best = e[0];
-      if (e[1] > best) { ax = 1; best = e[1]; }
-      if (e[2] > best) { ax = 2; }
-      axis_s = ax;
-    }
-    __syncthreads();
-  }
-  const int ax = sort_by_index ? 0 : axis_s;
   for (int t = threadIdx.x; t < P2; t += blockDim.x) {
-    if (t < n) {
-      const int a = perm[sg.start + t];
-      key[t] = sort_by_index ? (double)a : wrap1(R[3 * a + ax], g.box[ax]);
-      idx[t] = a;
-    } else {
-      key[t] = 1e308;
-      idx[t] = 0x7fffffff;
-    }
+    key[t] = t < n ? (double)perm[sg.start + t] : 1e308;
+    idx[t] = t < n ? perm[sg.start + t] : 0x7fffffff;
   }
   __syncthreads();
   block_bitonic(key, idx, P2);
@@ -681,9 +782,9 @@ cudaError_t GraphBuilder::build(const double* dR, int N, const double box[3], do
 Partitioner::~Partitioner() { release(); }
 
 void Partitioner::release() {
-  for (void* p : {(void*)perm, (void*)skey, (void*)sidx, (void*)segs_d, (void*)bits, (void*)hcnt})
+  for (void* p : {(void*)perm, (void*)skey, (void*)wrapped, (void*)sidx, (void*)segs_d, (void*)bits, (void*)hcnt})
     if (p) cudaFree(p);
-  perm = nullptr; skey = nullptr; sidx = nullptr; segs_d = nullptr; bits = nullptr; hcnt = nullptr;
+  perm = nullptr; skey = wrapped = nullptr; sidx = nullptr; segs_d = nullptr; bits = nullptr; hcnt = nullptr;
   cap_n = cap_scr = cap_seg = 0;
   cap_hcnt = cap_subptr = 0;
   cap_bits = 0;
@@ -704,57 +805,65 @@ cudaError_t Partitioner::rcb(const double* dR, int N, const double box[3], int c
     if ((e = cudaMalloc(&perm, sizeof(int) * N))) return e;
     cap_n = N;
   }
-  const long long need_scr = 2LL * next_pow2(N) + 64;
-  if (need_scr > cap_scr) {
-    if (skey) cudaFree(skey);
-    if (sidx) cudaFree(sidx);
-    if ((e = cudaMalloc(&skey, sizeof(double) * need_scr))) return e;
-    if ((e = cudaMalloc(&sidx, sizeof(int) * need_scr))) return e;
-    cap_scr = need_scr;
-  }
-  if (n_parts + 1 > cap_seg) {
-    if (segs_d) cudaFree(segs_d);
-    if ((e = cudaMalloc(&segs_d, sizeof(RcbSeg) * (n_parts + 1)))) return e;
-    cap_seg = n_parts + 1;
-  }
-  std::vector<int> hp(N);
-  for (int i = 0; i < N; ++i) hp[i] = i;
-  cudaMemcpyAsync(perm, hp.data(), sizeof(int) * N, cudaMemcpyHostToDevice, s);
-  CellGrid g = make_grid(box, 1.0);
+  // the tree follows from integers only: every level's segments, then the leaves, in one upload
   struct Node { int start, count, p; };
   std::vector<Node> level = {{0, N, n_parts}};
   std::vector<RcbSeg> hs;
+  std::vector<int> first(1, 0);
+  long long need_scr = 0;
   while (true) {
-    hs.clear();
     std::vector<Node> next;
     long long scr = 0;
     for (const Node& nd : level) {
       if (nd.p == 1) { next.push_back(nd); continue; }
-      RcbSeg sg;
-      sg.start = nd.start; sg.count = nd.count; sg.scratch = scr;
-      scr += next_pow2(nd.count);
-      hs.push_back(sg);
       const int pl = nd.p / 2;
       const int m = (int)(((long long)nd.count * pl) / nd.p);
+      hs.push_back({nd.start, nd.count, m, scr});
+      scr += next_pow2(nd.count);
       next.push_back({nd.start, m, pl});
       next.push_back({nd.start + m, nd.count - m, nd.p - pl});
     }
-    if (hs.empty()) break;
-    cudaMemcpyAsync(segs_d, hs.data(), sizeof(RcbSeg) * hs.size(), cudaMemcpyHostToDevice, s);
-    rcb_level_kernel<<<(int)hs.size(), 1024, 0, s>>>(segs_d, perm, dR, g, skey, sidx, 0);
-    // the segment array is rewritten next level: wait before reuse
-    if ((e = cudaStreamSynchronize(s))) return e;
+    need_scr = std::max(need_scr, scr);
+    if ((int)hs.size() == first.back()) break;
+    first.push_back((int)hs.size());
     level = next;
   }
   // leaves in depth-first order: the level list is already in tree order
   leaves.clear();
-  for (const Node& nd : level) leaves.push_back({nd.start, nd.count, 0});
-  // sort every leaf by atom index
   long long scr = 0;
-  for (auto& lf : leaves) { lf.scratch = scr; scr += next_pow2(lf.count); }
-  if (scr > cap_scr) return cudaErrorMemoryAllocation;
-  cudaMemcpyAsync(segs_d, leaves.data(), sizeof(RcbSeg) * leaves.size(), cudaMemcpyHostToDevice, s);
-  rcb_level_kernel<<<(int)leaves.size(), 256, 0, s>>>(segs_d, perm, dR, g, skey, sidx, 1);
+  for (const Node& nd : level) {
+    leaves.push_back({nd.start, nd.count, 0, scr});
+    scr += next_pow2(nd.count);
+  }
+  need_scr = std::max(need_scr, scr) + 64;
+  if (need_scr > cap_scr) {
+    if (skey) cudaFree(skey);
+    if (sidx) cudaFree(sidx);
+    if (wrapped) cudaFree(wrapped);
+    skey = wrapped = nullptr;
+    sidx = nullptr;
+    cap_scr = 0;
+    if ((e = cudaMalloc(&skey, sizeof(double) * need_scr))) return e;
+    if ((e = cudaMalloc(&sidx, sizeof(int) * need_scr))) return e;
+    if ((e = cudaMalloc(&wrapped, sizeof(double) * 3 * need_scr))) return e;   // (need_scr >= N)
+    cap_scr = need_scr;
+  }
+  const int n_seg = (int)hs.size();
+  hs.insert(hs.end(), leaves.begin(), leaves.end());
+  if ((int)hs.size() > cap_seg) {
+    if (segs_d) cudaFree(segs_d);
+    segs_d = nullptr;
+    cap_seg = 0;
+    if ((e = cudaMalloc(&segs_d, sizeof(RcbSeg) * hs.size()))) return e;
+    cap_seg = (int)hs.size();
+  }
+  CellGrid g = make_grid(box, 1.0);
+  cudaMemcpyAsync(segs_d, hs.data(), sizeof(RcbSeg) * hs.size(), cudaMemcpyHostToDevice, s);
+  rcb_wrap_kernel<<<(N + 127) / 128, 128, 0, s>>>(dR, N, g, wrapped, perm);
+  for (size_t l = 0; l + 1 < first.size(); ++l)
+    rcb_split_kernel<<<first[l + 1] - first[l], 1024, 0, s>>>(segs_d + first[l], perm, wrapped, N, skey, sidx);
+  rcb_leaf_kernel<<<(int)leaves.size(), 256, 0, s>>>(segs_d + n_seg, perm, skey, sidx);
+  if ((e = cudaGetLastError())) return e;
   return cudaStreamSynchronize(s);
 }
 
@@ -774,7 +883,7 @@ cudaError_t Partitioner::set_cores(const std::vector<std::vector<int>>& cores, i
   std::vector<int> hp;
   leaves.clear();
   for (auto& c : cores) {
-    leaves.push_back({(int)hp.size(), (int)c.size(), 0});
+    leaves.push_back({(int)hp.size(), (int)c.size(), 0, 0});
     hp.insert(hp.end(), c.begin(), c.end());
   }
   if ((int)hp.size() > cap_n) return cudaErrorInvalidValue;

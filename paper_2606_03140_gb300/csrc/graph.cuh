@@ -8,6 +8,7 @@ namespace sedacs {
 struct RcbSeg {
   int start;            // first position in the permutation
   int count;            // atoms in the segment
+  int left;             // of these, to the lower side of the split
   long long scratch;    // offset of its sort scratch
 };
 
@@ -51,6 +52,7 @@ struct GraphBuilder {
 struct Partitioner {
   int* perm = nullptr;        // atoms grouped by core, each core ascending
   double* skey = nullptr;
+  double* wrapped = nullptr;  // wrapped coordinates, [axis][atom]
   int* sidx = nullptr;
   RcbSeg* segs_d = nullptr;
   unsigned* bits = nullptr;
