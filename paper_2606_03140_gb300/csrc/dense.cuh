@@ -9,7 +9,7 @@ namespace sedacs {
 //   C = alpha * A * B^T + beta * I + g1 * C1 + g2 * C2      (generic mode)
 // (B^T: B is read by rows, so for the symmetric operands of the method B^T = B; C1, C2 are
 // masters added in the epilogue, so a product with I + E is formed as C + C E exactly).  Offsets are bytes from
-// the arena base.  For the tensor-core path A and B are blocked split planes (bf16, or the
+// the arena base (gemm_mat below forms them for one subgraph).  For the tensor-core path A and B are blocked split planes (bf16, or the
 // two-plane fp16 format) and the master output is fp32 row-major; for the FP64 path every
 // matrix is fp64 row-major.
 struct GemmMat {
@@ -43,6 +43,14 @@ struct GemmWork {
   int mat, tm, tn, pad;
 };
 
+// Place of a subgraph's matrices in every slot: element offsets in square and core-row slots, sizes.  One
+// table per layout serves all products and elementwise passes.
+struct GemmSub {
+  long long sq, rw;              // element offsets
+  long long tr_off;              // SP2 trace partial slots
+  int n_pad, n_real, m_core, m_pad;
+};
+
 // Per-subgraph state of the mu-branch SP2 recursion.
 struct Sp2State {
   double y;          // image of mu under the polynomial so far
@@ -63,7 +71,10 @@ enum GemmMode : int { kModeGeneric = 0, kModeSp2 = 1, kModeRsp = 2 };
 
 struct GemmParams {
   const GemmWork* work;
-  const GemmMat* mats;
+  const GemmSub* subs;
+  GemmMat slot;       // offsets of the slots (subgraph 0), strides and flags
+  int a_rows, b_rows, out_rows, c_rows, c2_rows;   // core-row slots (others are square)
+  int f64;
   uint8_t* arena;
   double* tr_slots;
   Sp2State* sp2;
@@ -76,6 +87,28 @@ struct GemmParams {
   int ops_upper;      // generic mode: A and B are symmetric and may be stored as their upper 128x128 tiles
                       // only (blocks left of the diagonal read as transposes)
 };
+
+#if defined(__CUDACC__)
+// The problem of subgraph i: its offsets in the slots of the product.
+__device__ __forceinline__ GemmMat gemm_mat(const GemmParams& p, int i) {
+  const GemmSub s = p.subs[i];
+  GemmMat m = p.slot;
+  const int ob = p.f64 ? 8 : 2, mb = p.f64 ? 8 : 4;          // bytes an operand / a master element
+  m.a_off += (p.a_rows ? s.rw : s.sq) * ob;
+  m.b_off += (p.b_rows ? s.rw : s.sq) * ob;
+  const long long out = p.out_rows ? s.rw : s.sq;
+  if (m.out_off >= 0) m.out_off += out * mb;
+  if (m.outp_off >= 0) m.outp_off += out * 2;
+  m.x_off += s.sq * mb;
+  if (m.c_off >= 0) m.c_off += (p.c_rows ? s.rw : s.sq) * (m.c_planes ? 2 : mb);
+  if (m.c2_off >= 0) m.c2_off += (p.c2_rows ? s.rw : s.sq) * mb;
+  m.tr_off = s.tr_off;
+  m.n_pad = s.n_pad;
+  m.n_real = m.k_real = s.n_real;
+  m.m_real = p.out_rows ? s.m_core : s.n_real;
+  return m;
+}
+#endif
 
 // Host launchers (dense.cu)
 void launch_gemm_tc(const GemmParams& p, int n_work, int nsplit, cudaStream_t s);

@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_persistent(const GemmPa
       for (int t = blockIdx.x; t < n_work && ok; t += gridDim.x) {
         const GemmWork w = p.work[t];
         if (!tile_live(w)) continue;
-        const GemmMat m = p.mats[w.mat];
+        const GemmMat m = gemm_mat(p, w.mat);
         const int cur = tile_cur(w, m);
         const long long in_shift = stepping ? cur * m.buf_stride : 0;
         const uint8_t* A = p.arena + m.a_off + (stepping ? in_shift : (m.a_from_sp2 ? cur * m.buf_stride : 0));
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_persistent(const GemmPa
       for (int t = blockIdx.x; t < n_work && ok; t += gridDim.x) {
         const GemmWork w = p.work[t];
         if (!tile_live(w)) continue;
-        const GemmMat m = p.mats[w.mat];
+        const GemmMat m = gemm_mat(p, w.mat);
         const int kb_end = (m.k_real + 63) >> 6;
         const uint32_t prev = (uint32_t)((ti - 1) & 1);
         // accumulator parts of the previous tile that the next k-block overwrites (all three at
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_persistent(const GemmPa
     for (int t = blockIdx.x; t < n_work && ok; t += gridDim.x) {
       const GemmWork w = p.work[t];
       if (!tile_live(w)) continue;
-      const GemmMat m = p.mats[w.mat];
+      const GemmMat m = gemm_mat(p, w.mat);
       const int cur = tile_cur(w, m);
       const int branch_sq = stepping ? (p.sp2[w.mat].y >= 0.5) : 0;
       const long long in_shift = stepping ? cur * m.buf_stride : 0;
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) f64_gemm_kernel(const GemmParams p) {
   __shared__ double Bs[16][64 + 1];
   __shared__ double red[2][8];
   const GemmWork w = p.work[blockIdx.x];
-  const GemmMat m = p.mats[w.mat];
+  const GemmMat m = gemm_mat(p, w.mat);
   int cur = 0, branch_sq = 0;
   const bool stepping = (p.mode == kModeSp2 || p.mode == kModeRsp);
   if (stepping) {

@@ -7,7 +7,7 @@ namespace sedacs {
 namespace {
 
 template <typename T>
-__global__ void split_planes_kernel(const SubView* views, uint8_t* arena, int nsplit) {
+__global__ void split_planes_kernel(SlotViews views, uint8_t* arena, int nsplit) {
   const SubView v = views[blockIdx.y];
   const int row = blockIdx.x;
   if (row >= v.rows_pad) return;
@@ -26,14 +26,14 @@ __global__ void split_planes_kernel(const SubView* views, uint8_t* arena, int ns
 // dX0 = -dh~ / (emax - emin), with the spectral bounds of each subgraph.  One warp per row,
 // 8 consecutive columns per lane (one 16-byte granule of each plane).
 struct AffineOut {
-  const SubView* views;   // nullptr: no such output
+  SlotViews views;        // subs nullptr: no such output
   double a, b;
   int master;             // write the row-major master
   int nsplit;             // plane format to write (0: none)
 };
 
 template <typename T>
-__global__ void affine_planes_kernel(const SubView* in_v, AffineOut o1, AffineOut o2, int kind, const double* bounds,
+__global__ void affine_planes_kernel(SlotViews in_v, AffineOut o1, AffineOut o2, int kind, const double* bounds,
                                      uint8_t* arena) {
   const SubView vi = in_v[blockIdx.y];
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -60,7 +60,7 @@ __global__ void affine_planes_kernel(const SubView* in_v, AffineOut o1, AffineOu
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const AffineOut& o = k == 0 ? o1 : o2;
-      if (!o.views) continue;
+      if (!o.views.subs) continue;
       const SubView vo = o.views[blockIdx.y];
       const T a = (T)(k == 0 ? a1 : o.a), b = (T)(k == 0 ? b1 : o.b);
       float yf[8];
@@ -91,14 +91,14 @@ __global__ void affine_planes_kernel(const SubView* in_v, AffineOut o1, AffineOu
 // block, zero elsewhere, each written as master and / or planes.  One warp per row, 8 columns
 // per lane.
 struct PolyOut {
-  const SubView* views;
+  SlotViews views;
   double a, b, c;
   int master;
   int nsplit;
 };
 
 template <typename T>
-__global__ void poly3_kernel(const SubView* e1, const SubView* e2, const SubView* e3, PolyOut o1, PolyOut o2,
+__global__ void poly3_kernel(SlotViews e1, SlotViews e2, SlotViews e3, PolyOut o1, PolyOut o2,
                              uint8_t* arena) {
   const SubView v1 = e1[blockIdx.y], v2 = e2[blockIdx.y], v3 = e3[blockIdx.y];
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -144,7 +144,7 @@ __global__ void poly3_kernel(const SubView* e1, const SubView* e2, const SubView
 // error (k - 1) 2^-24 of a lane's FP32 sum of k = ceil(n / 32) positive terms, so that the disc
 // still contains the exact one.
 template <typename T>
-__global__ void gersh_rows_kernel(const SubView* views, const uint8_t* arena, double* lo, double* hi,
+__global__ void gersh_rows_kernel(SlotViews views, const uint8_t* arena, double* lo, double* hi,
                                   const long long* row_base) {
   const SubView v = views[blockIdx.y];
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -181,7 +181,7 @@ __global__ void gersh_rows_kernel(const SubView* views, const uint8_t* arena, do
   }
 }
 
-__global__ void gersh_reduce_kernel(const SubView* views, const double* lo, const double* hi,
+__global__ void gersh_reduce_kernel(SlotViews views, const double* lo, const double* hi,
                                     const long long* row_base, double* bounds) {
   const SubView v = views[blockIdx.x];
   double mn = 1e300, mx = -1e300;
@@ -284,7 +284,7 @@ __global__ void sp2_advance_kernel(Sp2State* st, const double* slots, const long
 // symmetric iterate, so pass 0 fills each 128x64 block left of the diagonal ((cb / 2) < rb) from
 // the transpose of rows 64 (cb & 1) .. of the stored tile (cb / 2, rb), through shared memory;
 // pass 1 then converts the stored blocks in place.  One CTA per block.
-__global__ void f16x2_to_bf16x3_kernel(const SubView* views, const Sp2State* st, long long copy_stride,
+__global__ void f16x2_to_bf16x3_kernel(SlotViews views, const Sp2State* st, long long copy_stride,
                                        uint8_t* arena, int pass) {
   __shared__ float tr[64][129];
   const SubView v = views[blockIdx.y];
@@ -335,14 +335,14 @@ __global__ void f16x2_to_bf16x3_kernel(const SubView* views, const Sp2State* st,
 
 }  // namespace
 
-void launch_f16x2_to_bf16x3(const SubView* views, const Sp2State* st, long long copy_stride, int n_sub, int max_rows,
+void launch_f16x2_to_bf16x3(SlotViews views, const Sp2State* st, long long copy_stride, int n_sub, int max_rows,
                             uint8_t* arena, cudaStream_t s) {
   if (n_sub <= 0 || max_rows <= 0) return;
   dim3 g((max_rows / 128) * (max_rows / 64), n_sub);
   for (int pass = 0; pass < 2; ++pass) f16x2_to_bf16x3_kernel<<<g, 256, 0, s>>>(views, st, copy_stride, arena, pass);
 }
 
-void launch_split_planes(const SubView* views, int n_sub, int max_rows, uint8_t* arena, int nsplit, bool f64,
+void launch_split_planes(SlotViews views, int n_sub, int max_rows, uint8_t* arena, int nsplit, bool f64,
                          cudaStream_t s) {
   if (n_sub <= 0 || max_rows <= 0) return;
   dim3 g(max_rows, n_sub);
@@ -350,8 +350,8 @@ void launch_split_planes(const SubView* views, int n_sub, int max_rows, uint8_t*
   else split_planes_kernel<float><<<g, 64, 0, s>>>(views, arena, nsplit);
 }
 
-void launch_affine_planes(const SubView* in, const SubView* out1, double a1, double b1, int master1, int nsplit1,
-                          const SubView* out2, double a2, double b2, int master2, int nsplit2, int kind,
+void launch_affine_planes(SlotViews in, SlotViews out1, double a1, double b1, int master1, int nsplit1,
+                          SlotViews out2, double a2, double b2, int master2, int nsplit2, int kind,
                           const double* bounds, int n_sub, int max_rows, uint8_t* arena, bool f64, cudaStream_t s) {
   if (n_sub <= 0 || max_rows <= 0) return;
   dim3 g((max_rows + 7) / 8, n_sub);
@@ -361,8 +361,8 @@ void launch_affine_planes(const SubView* in, const SubView* out1, double a1, dou
   else affine_planes_kernel<float><<<g, 256, 0, s>>>(in, o1, o2, kind, bounds, arena);
 }
 
-void launch_poly3(const SubView* e1, const SubView* e2, const SubView* e3, const SubView* out1, double a1, double b1,
-                  double c1, int master1, int nsplit1, const SubView* out2, double a2, double b2, double c2,
+void launch_poly3(SlotViews e1, SlotViews e2, SlotViews e3, SlotViews out1, double a1, double b1,
+                  double c1, int master1, int nsplit1, SlotViews out2, double a2, double b2, double c2,
                   int master2, int nsplit2, int n_sub, int max_rows, uint8_t* arena, bool f64, cudaStream_t s) {
   if (n_sub <= 0 || max_rows <= 0) return;
   dim3 g((max_rows + 7) / 8, n_sub);
@@ -372,7 +372,7 @@ void launch_poly3(const SubView* e1, const SubView* e2, const SubView* e3, const
   else poly3_kernel<float><<<g, 256, 0, s>>>(e1, e2, e3, o1, o2, arena);
 }
 
-void launch_gershgorin(const SubView* views, int n_sub, int max_rows, const uint8_t* arena, double* lo, double* hi,
+void launch_gershgorin(SlotViews views, int n_sub, int max_rows, const uint8_t* arena, double* lo, double* hi,
                        const long long* row_base, double* bounds, bool f64, cudaStream_t s) {
   if (n_sub <= 0) return;
   dim3 g((max_rows + 7) / 8, n_sub);

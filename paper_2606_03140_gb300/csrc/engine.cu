@@ -361,50 +361,29 @@ long long mptr(const sedacs_ctx* ctx, int sl, int i, int copy = 0) {
   const long long el = S.rows ? ctx->lay.rw_off[i] : ctx->lay.sq_off[i];
   return S.base + copy * S.copy_stride + el * (ctx->f64 ? 8 : 4);
 }
-long long pptr_(const sedacs_ctx* ctx, int sl, int i, int copy = 0) {
-  const Slot& S = ctx->slot[sl];
-  if (!S.planes) return -1;
-  const long long el = S.rows ? ctx->lay.rw_off[i] : ctx->lay.sq_off[i];
-  return S.base + copy * S.copy_stride + S.master_bytes + el * 2;
-}
-
-// C = alpha A B^T + beta I + g1 C1 + g2 C2 over every subgraph (slots a, b, out, c1, c2; -1: none).
-// Staged uploads: the bytes are appended to ctx->stage_host (16-byte aligned) and sent by
-// flush_staged, which copies them once into pinned memory and enqueues one asynchronous copy
-// per destination (no pageable copies, no stream synchronisation per array).
-void stage_bytes(sedacs_ctx* ctx, void* dst, const void* src, size_t bytes) {
-  if (bytes == 0) return;
+// Staged uploads: a layout's tables are appended to ctx->stage_host (16-byte aligned) and sent by
+// flush_staged, which copies them once into pinned memory and from there to one device block with one
+// asynchronous copy, and then points every table at its place in the block.
+void stage_bytes(sedacs_ctx* ctx, void** dst, const void* src, size_t bytes) {
   const size_t off = (ctx->stage_host.size() + 15) & ~size_t(15);
   ctx->stage_host.resize(off + bytes);
-  std::memcpy(ctx->stage_host.data() + off, src, bytes);
-  ctx->stage_recs.emplace_back(dst, off, bytes);
+  if (bytes) std::memcpy(ctx->stage_host.data() + off, src, bytes);
+  ctx->stage_recs.emplace_back(dst, off);
 }
 
 template <typename T>
-sedacs_status stage_vec(sedacs_ctx* ctx, T** dst, const std::vector<T>& v) {
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(dst), sizeof(T) * std::max<size_t>(1, v.size())));
-  stage_bytes(ctx, *dst, v.data(), sizeof(T) * v.size());
-  return SEDACS_OK;
+void stage_vec(sedacs_ctx* ctx, T** dst, const std::vector<T>& v) {
+  stage_bytes(ctx, reinterpret_cast<void**>(dst), v.data(), sizeof(T) * v.size());
 }
 
-sedacs_status stage_views(sedacs_ctx* ctx, int sl, int copy, SubView** dst) {
-  const Layout& L = ctx->lay;
-  std::vector<SubView> v(L.n_sub);
-  for (int i = 0; i < L.n_sub; ++i) {
-    SubView s;
-    s.master = mptr(ctx, sl, i, copy);
-    s.planes = pptr_(ctx, sl, i, copy);
-    s.plane_stride = ctx->slot[sl].plane_stride;
-    s.n_pad = L.n_pad[i];
-    s.rows_pad = ctx->slot[sl].rows ? L.m_pad[i] : L.n_pad[i];
-    s.n_real = L.n_real[i];
-    s.pad = 0;
-    v[i] = s;
-  }
-  return stage_vec(ctx, dst, v);
+SlotViews views(const sedacs_ctx* ctx, int sl) {
+  const Slot& S = ctx->slot[sl];
+  return SlotViews{ctx->d_subs, S.base, S.planes ? S.base + S.master_bytes : -1, S.plane_stride, S.rows ? 1 : 0,
+                   ctx->f64 ? 8 : 4};
 }
+const SlotViews kNoViews{};
 
-// The caller synchronises the stream before the next staging round reuses the pinned buffer.
+// The pinned buffer is free here: rebuild_layout waits for the stream after the last flush's copy.
 sedacs_status flush_staged(sedacs_ctx* ctx) {
   const size_t n = ctx->stage_host.size();
   if (n > ctx->stage_pinned_cap) {
@@ -415,72 +394,92 @@ sedacs_status flush_staged(sedacs_ctx* ctx) {
     CUCHK(cudaHostAlloc(reinterpret_cast<void**>(&ctx->stage_pinned), want, cudaHostAllocDefault));
     ctx->stage_pinned_cap = want;
   }
-  if (n) std::memcpy(ctx->stage_pinned, ctx->stage_host.data(), n);
-  for (const auto& r : ctx->stage_recs)
-    CUCHK(cudaMemcpyAsync(std::get<0>(r), ctx->stage_pinned + std::get<1>(r), std::get<2>(r), cudaMemcpyHostToDevice,
-                          ctx->stream));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_tables), std::max<size_t>(n, 16)));
+  if (n) {
+    std::memcpy(ctx->stage_pinned, ctx->stage_host.data(), n);
+    CUCHK(cudaMemcpyAsync(ctx->d_tables, ctx->stage_pinned, n, cudaMemcpyHostToDevice, ctx->stream));
+  }
+  for (const auto& r : ctx->stage_recs) *r.first = ctx->d_tables + r.second;
   ctx->stage_host.clear();
   ctx->stage_recs.clear();
   return SEDACS_OK;
 }
 
-sedacs_status build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode, double alpha, double beta,
-                       bool b_from_sp2, bool a_from_sp2 = false, int c1 = -1, double g1 = 0.0, int c2 = -1,
-                       double g2 = 0.0, bool c_from_sp2 = false, bool sym = false, int ca = 0, int cb = 0,
-                       int cout = 0, int cc1 = 0) {
+// Placement table and tile lists of the current layout.  FP64 tiles (64 x 64) with nothing but padding are left
+// out: the products read rows of listed tiles and columns below the valid inner dimension only.
+sedacs_status build_work(sedacs_ctx* ctx) {
   const Layout& L = ctx->lay;
-  std::vector<GemmMat> mats(L.n_sub);
-  std::vector<GemmWork> work;
-  const bool rows_out = ctx->slot[out].rows;
+  std::vector<GemmSub> subs(L.n_sub);
+  std::vector<GemmWork> work[kNumWork];
   for (int i = 0; i < L.n_sub; ++i) {
-    GemmMat m{};
-    m.a_off = ctx->f64 ? mptr(ctx, a, i, ca) : pptr_(ctx, a, i, ca);
-    m.b_off = ctx->f64 ? mptr(ctx, b, i, cb) : pptr_(ctx, b, i, cb);
-    m.a_plane = ctx->slot[a].plane_stride;
-    m.b_plane = ctx->slot[b].plane_stride;
-    m.out_off = mptr(ctx, out, i, cout);
-    m.outp_off = ctx->f64 ? -1 : pptr_(ctx, out, i, cout);
-    m.outp_plane = ctx->slot[out].plane_stride;
-    m.x_off = (mode == kModeRsp) ? mptr(ctx, kR2, i) : mptr(ctx, kX, i);
-    m.c_off = (mode == kModeRsp) ? mptr(ctx, kR1, i) : (c1 >= 0 ? mptr(ctx, c1, i, cc1) : -1);
-    m.c2_off = (c2 >= 0) ? mptr(ctx, c2, i) : -1;
-    m.c_from_sp2 = c_from_sp2 ? 1 : 0;
-    m.sym_out = sym && !rows_out ? 1 : 0;
-    m.buf_stride = ctx->slot[kX].copy_stride;
-    m.tr_off = L.tr_off[i];
-    m.n_pad = L.n_pad[i];
-    m.m_real = rows_out ? L.n_core_orb[i] : L.n_real[i];
-    m.n_real = L.n_real[i];
-    m.k_real = L.n_real[i];
-    m.b_from_sp2 = b_from_sp2 ? 1 : 0;
-    m.a_from_sp2 = a_from_sp2 ? 1 : 0;
-    // three-plane bf16 and two-plane fp16 SP2 iterates carry no fp32 master: the SP2 epilogue
-    // reads the planes (the value the MMAs see), and the consumers of X as an addend (C1) read
-    // the three bf16 planes, whose sum is the fp32 value exactly (fp16 iterates are rewritten
-    // in that format once the recursion has stopped)
-    const bool x3 = !ctx->f64 && (ctx->nsplit_sp2 == 3 || ctx->nsplit_sp2 == kPlanesF16x2);
-    if (x3 && mode == kModeSp2) {
-      m.x_planes = 1;
-      m.out_off = -1;
-    }
-    if (x3 && mode == kModeGeneric && c1 == kX) {
-      m.c_off = pptr_(ctx, kX, i);
-      m.c_plane = ctx->slot[kX].plane_stride;
-      m.c_planes = 1;
-    }
-    mats[i] = m;
+    subs[i] = GemmSub{L.sq_off[i], L.rw_off[i], L.tr_off[i], L.n_pad[i], L.n_real[i], L.n_core_orb[i], L.m_pad[i]};
     if (L.n_real[i] == 0) continue;
-    const int tiles_n = L.n_pad[i] / ctx->tile;
-    const int tiles_m = (rows_out ? L.m_pad[i] : L.n_pad[i]) / ctx->tile;
-    for (int tm = 0; tm < tiles_m; ++tm)
-      for (int tn = (m.sym_out ? tm : 0); tn < tiles_n; ++tn) work.push_back({i, tm, tn, 0});
+    const int tile = ctx->tile;
+    const int n = ctx->f64 ? (L.n_real[i] + tile - 1) / tile : L.n_pad[i] / tile;
+    const int m = ctx->f64 ? (L.n_core_orb[i] + tile - 1) / tile : L.m_pad[i] / tile;
+    for (int tm = 0; tm < n; ++tm)
+      for (int tn = 0; tn < n; ++tn) {
+        work[kWorkSquare].push_back({i, tm, tn, 0});
+        if (tn >= tm) work[kWorkSym].push_back({i, tm, tn, 0});
+      }
+    for (int tm = 0; tm < m; ++tm)
+      for (int tn = 0; tn < n; ++tn) work[kWorkRows].push_back({i, tm, tn, 0});
   }
+  stage_vec(ctx, &ctx->d_subs, subs);
+  for (int k = 0; k < kNumWork; ++k) {
+    stage_vec(ctx, &ctx->d_work[k], work[k]);
+    ctx->n_work[k] = (int)work[k].size();
+  }
+  return SEDACS_OK;
+}
+
+// C = alpha A B^T + beta I + g1 C1 + g2 C2 over every subgraph (slots a, b, out, c1, c2; -1: none).
+void build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode, double alpha, double beta, bool b_from_sp2,
+              bool a_from_sp2 = false, int c1 = -1, double g1 = 0.0, int c2 = -1, double g2 = 0.0,
+              bool c_from_sp2 = false, bool sym = false, int ca = 0, int cb = 0, int cout = 0, int cc1 = 0) {
   GemmOp& op = ctx->ops[id];
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&op.mats_d), sizeof(GemmMat) * std::max(1, L.n_sub)));
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&op.work_d), sizeof(GemmWork) * std::max<size_t>(1, work.size())));
-  stage_bytes(ctx, op.mats_d, mats.data(), sizeof(GemmMat) * L.n_sub);
-  stage_bytes(ctx, op.work_d, work.data(), sizeof(GemmWork) * work.size());
-  op.n_work = (int)work.size();
+  auto master = [&](int sl, int copy) { return ctx->slot[sl].base + copy * ctx->slot[sl].copy_stride; };
+  auto planes = [&](int sl, int copy) {
+    return ctx->slot[sl].planes ? master(sl, copy) + ctx->slot[sl].master_bytes : -1LL;
+  };
+  const bool rows_out = ctx->slot[out].rows;
+  GemmMat m{};
+  m.a_off = ctx->f64 ? master(a, ca) : planes(a, ca);
+  m.b_off = ctx->f64 ? master(b, cb) : planes(b, cb);
+  m.a_plane = ctx->slot[a].plane_stride;
+  m.b_plane = ctx->slot[b].plane_stride;
+  m.out_off = master(out, cout);
+  m.outp_off = ctx->f64 ? -1 : planes(out, cout);
+  m.outp_plane = ctx->slot[out].plane_stride;
+  m.x_off = master(mode == kModeRsp ? kR2 : kX, 0);
+  m.c_off = mode == kModeRsp ? master(kR1, 0) : (c1 >= 0 ? master(c1, cc1) : -1);
+  m.c2_off = c2 >= 0 ? master(c2, 0) : -1;
+  m.c_from_sp2 = c_from_sp2 ? 1 : 0;
+  m.sym_out = sym && !rows_out ? 1 : 0;
+  m.buf_stride = ctx->slot[kX].copy_stride;
+  m.b_from_sp2 = b_from_sp2 ? 1 : 0;
+  m.a_from_sp2 = a_from_sp2 ? 1 : 0;
+  // three-plane bf16 and two-plane fp16 SP2 iterates carry no fp32 master: the SP2 epilogue
+  // reads the planes (the value the MMAs see), and the consumers of X as an addend (C1) read
+  // the three bf16 planes, whose sum is the fp32 value exactly (fp16 iterates are rewritten
+  // in that format once the recursion has stopped)
+  const bool x3 = !ctx->f64 && (ctx->nsplit_sp2 == 3 || ctx->nsplit_sp2 == kPlanesF16x2);
+  if (x3 && mode == kModeSp2) {
+    m.x_planes = 1;
+    m.out_off = -1;
+  }
+  if (x3 && mode == kModeGeneric && c1 == kX) {
+    m.c_off = planes(kX, 0);
+    m.c_plane = ctx->slot[kX].plane_stride;
+    m.c_planes = 1;
+  }
+  op.slot = m;
+  op.a_rows = ctx->slot[a].rows;
+  op.b_rows = ctx->slot[b].rows;
+  op.out_rows = rows_out;
+  op.c_rows = mode != kModeRsp && c1 >= 0 && ctx->slot[c1].rows;
+  op.c2_rows = c2 >= 0 && ctx->slot[c2].rows;
+  op.work = rows_out ? kWorkRows : (sym ? kWorkSym : kWorkSquare);
   op.same_ab = (a == b && ca == cb && a_from_sp2 == b_from_sp2) ? 1 : 0;
   op.n_addends = (c1 >= 0 ? 1 : 0) + (c2 >= 0 ? 1 : 0);
   op.alpha = alpha;
@@ -490,14 +489,21 @@ sedacs_status build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode,
   op.mode = mode;
   op.sym = sym && !rows_out;
   op.ops_upper = 0;
-  return SEDACS_OK;
 }
 
 void run_op(sedacs_ctx* ctx, int id, int nsplit_in, int nsplit_out) {
   const GemmOp& op = ctx->ops[id];
+  const int n_work = ctx->n_work[op.work];
   GemmParams p;
-  p.work = op.work_d;
-  p.mats = op.mats_d;
+  p.work = ctx->d_work[op.work];
+  p.subs = ctx->d_subs;
+  p.slot = op.slot;
+  p.a_rows = op.a_rows;
+  p.b_rows = op.b_rows;
+  p.out_rows = op.out_rows;
+  p.c_rows = op.c_rows;
+  p.c2_rows = op.c2_rows;
+  p.f64 = ctx->f64 ? 1 : 0;
   p.arena = ctx->arena;
   p.tr_slots = ctx->d_slots;
   p.sp2 = ctx->d_sp2;
@@ -509,9 +515,9 @@ void run_op(sedacs_ctx* ctx, int id, int nsplit_in, int nsplit_out) {
   p.g1 = op.g1;
   p.g2 = op.g2;
   p.ops_upper = op.ops_upper;
-  if (ctx->f64) launch_gemm_f64(p, op.n_work, ctx->stream);
-  else launch_gemm_tc(p, op.n_work, nsplit_in, ctx->stream);
-  ctx->launches += op.n_work > 0 ? 1 : 0;
+  if (ctx->f64) launch_gemm_f64(p, n_work, ctx->stream);
+  else launch_gemm_tc(p, n_work, nsplit_in, ctx->stream);
+  ctx->launches += n_work > 0 ? 1 : 0;
 }
 
 template <typename T>
@@ -568,77 +574,77 @@ sedacs_status build_fermi_ops(sedacs_ctx* ctx) {
   const bool T = true, F = false;
   if (!ctx->chain) {                    // (chains describe their products when they run, see fermi_chain)
     // start: Z2 = z z, Z4 = Z2 Z2
-    STCHK(build_op(ctx, OP_F_Z2, kP, kP, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
-    STCHK(build_op(ctx, OP_F_Z4, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
+    build_op(ctx, OP_F_Z2, kP, kP, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T);
+    build_op(ctx, OP_F_Z4, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T);
     // q(Z2) = sum_k a_k Z2^k = B_0 + Z4 (B_1 + Z4 (... B_J)), B_j = a_2j + a_2j+1 Z2:
     // T_1 = B_{J-1} + Z4 B_J = a_2J+1 (Z2 Z4) + a_2J Z4 + a_2J-1 Z2 + a_2J-2 I
-    STCHK(build_op(ctx, OP_F_ST1, kY0, kY1, horner_slot(1), kModeGeneric, a[2 * J + 1], a[2 * J - 2], F, F, kY1,
-                   a[2 * J], kY0, a[2 * J - 1], F, T));
+    build_op(ctx, OP_F_ST1, kY0, kY1, horner_slot(1), kModeGeneric, a[2 * J + 1], a[2 * J - 2], F, F, kY1,
+                   a[2 * J], kY0, a[2 * J - 1], F, T);
     // T_j = B_{J-j} + Z4 T_{j-1}
     for (int j = 2; j <= J; ++j)
-      STCHK(build_op(ctx, OP_F_SH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
-                     a[2 * (J - j)], F, F, kY0, a[2 * (J - j) + 1], -1, 0.0, F, T));
+      build_op(ctx, OP_F_SH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
+                     a[2 * (J - j)], F, F, kY0, a[2 * (J - j) + 1], -1, 0.0, F, T);
     // U_0 = z q into either copy of kX
     for (int cu = 0; cu < 2; ++cu)
-      STCHK(build_op(ctx, OP_F_U0_0 + cu, kP, horner_slot(J), kX, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F,
-                     T, 0, 0, cu));
+      build_op(ctx, OP_F_U0_0 + cu, kP, horner_slot(J), kX, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F,
+                     T, 0, 0, cu);
     // doubling: V = U U (from either copy), V2 = V V
     for (int cu = 0; cu < 2; ++cu)
-      STCHK(build_op(ctx, OP_F_V_0 + cu, kX, kX, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T, cu, cu, 0));
-    STCHK(build_op(ctx, OP_F_V2, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
+      build_op(ctx, OP_F_V_0 + cu, kX, kX, kY0, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T, cu, cu, 0);
+    build_op(ctx, OP_F_V2, kY0, kY0, kY1, kModeGeneric, 1.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T);
     // r(V) = sum_k c_k V^k = B_0 + V2 (B_1 + ... V2 B_M), B_j = c_2j + c_2j+1 V:
     // T_1 = c_2M+1 (V V2) + c_2M V2 + c_2M-1 V + c_2M-2 I, T_j = B_{M-j} + V2 T_{j-1}
-    STCHK(build_op(ctx, OP_F_IT1, kY0, kY1, horner_slot(1), kModeGeneric, c[2 * M + 1], c[2 * M - 2], F, F, kY1,
-                   c[2 * M], kY0, c[2 * M - 1], F, T));
+    build_op(ctx, OP_F_IT1, kY0, kY1, horner_slot(1), kModeGeneric, c[2 * M + 1], c[2 * M - 2], F, F, kY1,
+                   c[2 * M], kY0, c[2 * M - 1], F, T);
     for (int j = 2; j <= M; ++j)
-      STCHK(build_op(ctx, OP_F_IH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
-                     c[2 * (M - j)], F, F, kY0, c[2 * (M - j) + 1], -1, 0.0, F, T));
+      build_op(ctx, OP_F_IH0 + (j - 2), kY1, horner_slot(j - 1), horner_slot(j), kModeGeneric, 1.0,
+                     c[2 * (M - j)], F, F, kY0, c[2 * (M - j) + 1], -1, 0.0, F, T);
     // U' = 2 U r(V) into the other copy; the last doubling (from copy 1): F = U r(V) + I / 2
     for (int cu = 0; cu < 2; ++cu)
-      STCHK(build_op(ctx, OP_F_UP_0 + cu, kX, horner_slot(M), kX, kModeGeneric, 2.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T,
-                     cu, 0, 1 - cu));
+      build_op(ctx, OP_F_UP_0 + cu, kX, horner_slot(M), kX, kModeGeneric, 2.0, 0.0, F, F, -1, 0.0, -1, 0.0, F, T,
+                     cu, 0, 1 - cu);
   }
-  STCHK(build_op(ctx, OP_F_FIN, kX, horner_slot(M), kX, kModeGeneric, 1.0, 0.5, F, F, -1, 0.0, -1, 0.0, F, T, 1, 0,
-                 0));
+  build_op(ctx, OP_F_FIN, kX, horner_slot(M), kX, kModeGeneric, 1.0, 0.5, F, F, -1, 0.0, -1, 0.0, F, T, 1, 0,
+                 0);
   // s = F - F^2 without the cancellation of F - F F on the saturated levels: with V = U^2 and
   // r = (I + V)^-1 of the last doubling, I - U'^2 = ((I - V) r)^2, so s = (I - U'^2) / 4 = G^2 / 4
   // with G = r - V r (small where F is 0 or 1)
   // (G goes to the Horner slot that does not hold r: kT for M even, kR1 copy 0 for M odd)
   const int gslot = horner_slot(M) == kT ? kR1 : kT;
   if (!ctx->chain)
-    STCHK(build_op(ctx, OP_F_G, kY0, horner_slot(M), gslot, kModeGeneric, -1.0, 0.0, F, F, horner_slot(M), 1.0,
-                   -1, 0.0, F, T));
-  STCHK(build_op(ctx, OP_F_S, gslot, gslot, kR2, kModeGeneric, 0.25, 0.0, F, F, -1, 0.0, -1, 0.0, F, T));
+    build_op(ctx, OP_F_G, kY0, horner_slot(M), gslot, kModeGeneric, -1.0, 0.0, F, F, horner_slot(M), 1.0,
+                   -1, 0.0, F, T);
+  build_op(ctx, OP_F_S, gslot, gslot, kR2, kModeGeneric, 0.25, 0.0, F, F, -1, 0.0, -1, 0.0, F, T);
   // core rows of F into the response slots: dT1 = Z_c F = F_c + E_z,c F
-  STCHK(build_op(ctx, OP_F_FT1_0, kZ0, kX, kdT1, kModeGeneric, 1.0, 0.0, T, F, kX, 1.0, -1, 0.0, T));
-  STCHK(build_op(ctx, OP_F_FT1_1, kZ1, kX, kdT1, kModeGeneric, 1.0, 0.0, T, F, kX, 1.0, -1, 0.0, T));
+  build_op(ctx, OP_F_FT1_0, kZ0, kX, kdT1, kModeGeneric, 1.0, 0.0, T, F, kX, 1.0, -1, 0.0, T);
+  build_op(ctx, OP_F_FT1_1, kZ1, kX, kdT1, kModeGeneric, 1.0, 0.0, T, F, kX, 1.0, -1, 0.0, T);
   // energy-weighted rows of s: T2 = dT1 h~, Ws = 2 (T2 + T2 E_z) into kT1
-  STCHK(build_op(ctx, OP_F_T2S, kdT1, kHt, kT2, kModeGeneric, 1.0, 0.0, F));
-  STCHK(build_op(ctx, OP_F_WS0, kT2, kZ0, kT1, kModeGeneric, 2.0, 0.0, F, F, kT2, 2.0));
-  STCHK(build_op(ctx, OP_F_WS1, kT2, kZ1, kT1, kModeGeneric, 2.0, 0.0, F, F, kT2, 2.0));
+  build_op(ctx, OP_F_T2S, kdT1, kHt, kT2, kModeGeneric, 1.0, 0.0, F);
+  build_op(ctx, OP_F_WS0, kT2, kZ0, kT1, kModeGeneric, 2.0, 0.0, F, F, kT2, 2.0);
+  build_op(ctx, OP_F_WS1, kT2, kZ1, kT1, kModeGeneric, 2.0, 0.0, F, F, kT2, 2.0);
   // second-order term: t = s (I - 2F) = s - 2 s F into kR1 copy 1; d^2 F / dmu^2 = beta^2 t
-  STCHK(build_op(ctx, OP_F_T, kR2, kX, kR1, kModeGeneric, -2.0, 0.0, T, T, kR2, 1.0, -1, 0.0, T, T, 0, 0, 1));
-  STCHK(build_op(ctx, OP_F_TT1_0, kZ0, kR1, kdT2, kModeGeneric, 1.0, 0.0, F, F, kR1, 1.0, -1, 0.0, F, F, 0, 1, 0, 1));
-  STCHK(build_op(ctx, OP_F_TT1_1, kZ1, kR1, kdT2, kModeGeneric, 1.0, 0.0, F, F, kR1, 1.0, -1, 0.0, F, F, 0, 1, 0, 1));
-  STCHK(build_op(ctx, OP_F_DT0, kdT2, kZ0, kdDt, kModeGeneric, 2.0, 0.0, F, F, kdT2, 2.0));
-  STCHK(build_op(ctx, OP_F_DT1, kdT2, kZ1, kdDt, kModeGeneric, 2.0, 0.0, F, F, kdT2, 2.0));
-  STCHK(build_op(ctx, OP_F_T2T, kdT2, kHt, kT2, kModeGeneric, 1.0, 0.0, F));
+  build_op(ctx, OP_F_T, kR2, kX, kR1, kModeGeneric, -2.0, 0.0, T, T, kR2, 1.0, -1, 0.0, T, T, 0, 0, 1);
+  build_op(ctx, OP_F_TT1_0, kZ0, kR1, kdT2, kModeGeneric, 1.0, 0.0, F, F, kR1, 1.0, -1, 0.0, F, F, 0, 1, 0, 1);
+  build_op(ctx, OP_F_TT1_1, kZ1, kR1, kdT2, kModeGeneric, 1.0, 0.0, F, F, kR1, 1.0, -1, 0.0, F, F, 0, 1, 0, 1);
+  build_op(ctx, OP_F_DT0, kdT2, kZ0, kdDt, kModeGeneric, 2.0, 0.0, F, F, kdT2, 2.0);
+  build_op(ctx, OP_F_DT1, kdT2, kZ1, kdDt, kModeGeneric, 2.0, 0.0, F, F, kdT2, 2.0);
+  build_op(ctx, OP_F_T2T, kdT2, kHt, kT2, kModeGeneric, 1.0, 0.0, F);
   // third order: P = t F into kT, u = -2 s s + t - 2 P into kY0 (both free after the pass); rows
-  STCHK(build_op(ctx, OP_F_TF, kR1, kX, kT, kModeGeneric, 1.0, 0.0, T, F, -1, 0.0, -1, 0.0, F, T, 1, 0, 0));
-  STCHK(build_op(ctx, OP_F_U, kR2, kR2, kY0, kModeGeneric, -2.0, 0.0, T, T, kR1, 1.0, kT, -2.0, F, T, 0, 0, 0, 1));
-  STCHK(build_op(ctx, OP_F_UT1_0, kZ0, kY0, kdT3, kModeGeneric, 1.0, 0.0, F, F, kY0, 1.0, -1, 0.0, F, F));
-  STCHK(build_op(ctx, OP_F_UT1_1, kZ1, kY0, kdT3, kModeGeneric, 1.0, 0.0, F, F, kY0, 1.0, -1, 0.0, F, F));
-  STCHK(build_op(ctx, OP_F_DU0, kdT3, kZ0, kdDu, kModeGeneric, 2.0, 0.0, F, F, kdT3, 2.0));
-  STCHK(build_op(ctx, OP_F_DU1, kdT3, kZ1, kdDu, kModeGeneric, 2.0, 0.0, F, F, kdT3, 2.0));
-  STCHK(build_op(ctx, OP_F_T2U, kdT3, kHt, kT2, kModeGeneric, 1.0, 0.0, F));
+  build_op(ctx, OP_F_TF, kR1, kX, kT, kModeGeneric, 1.0, 0.0, T, F, -1, 0.0, -1, 0.0, F, T, 1, 0, 0);
+  build_op(ctx, OP_F_U, kR2, kR2, kY0, kModeGeneric, -2.0, 0.0, T, T, kR1, 1.0, kT, -2.0, F, T, 0, 0, 0, 1);
+  build_op(ctx, OP_F_UT1_0, kZ0, kY0, kdT3, kModeGeneric, 1.0, 0.0, F, F, kY0, 1.0, -1, 0.0, F, F);
+  build_op(ctx, OP_F_UT1_1, kZ1, kY0, kdT3, kModeGeneric, 1.0, 0.0, F, F, kY0, 1.0, -1, 0.0, F, F);
+  build_op(ctx, OP_F_DU0, kdT3, kZ0, kdDu, kModeGeneric, 2.0, 0.0, F, F, kdT3, 2.0);
+  build_op(ctx, OP_F_DU1, kdT3, kZ1, kdDu, kModeGeneric, 2.0, 0.0, F, F, kdT3, 2.0);
+  build_op(ctx, OP_F_T2U, kdT3, kHt, kT2, kModeGeneric, 1.0, 0.0, F);
   // fourth order: Q = u F into kT, w = -6 s t + u - 2 Q into kY1; rows
-  STCHK(build_op(ctx, OP_F_UF, kY0, kX, kT, kModeGeneric, 1.0, 0.0, T, F, -1, 0.0, -1, 0.0, F, T));
-  STCHK(build_op(ctx, OP_F_W, kR2, kR1, kY1, kModeGeneric, -6.0, 0.0, F, T, kY0, 1.0, kT, -2.0, F, T, 0, 1, 0));
-  STCHK(build_op(ctx, OP_F_WT1_0, kZ0, kY1, kdT4, kModeGeneric, 1.0, 0.0, F, F, kY1, 1.0, -1, 0.0, F, F));
-  STCHK(build_op(ctx, OP_F_WT1_1, kZ1, kY1, kdT4, kModeGeneric, 1.0, 0.0, F, F, kY1, 1.0, -1, 0.0, F, F));
-  STCHK(build_op(ctx, OP_F_DW0, kdT4, kZ0, kdDw, kModeGeneric, 2.0, 0.0, F, F, kdT4, 2.0));
-  STCHK(build_op(ctx, OP_F_DW1, kdT4, kZ1, kdDw, kModeGeneric, 2.0, 0.0, F, F, kdT4, 2.0));
-  STCHK(build_op(ctx, OP_F_T2W, kdT4, kHt, kT2, kModeGeneric, 1.0, 0.0, F));
+  build_op(ctx, OP_F_UF, kY0, kX, kT, kModeGeneric, 1.0, 0.0, T, F, -1, 0.0, -1, 0.0, F, T);
+  build_op(ctx, OP_F_W, kR2, kR1, kY1, kModeGeneric, -6.0, 0.0, F, T, kY0, 1.0, kT, -2.0, F, T, 0, 1, 0);
+  build_op(ctx, OP_F_WT1_0, kZ0, kY1, kdT4, kModeGeneric, 1.0, 0.0, F, F, kY1, 1.0, -1, 0.0, F, F);
+  build_op(ctx, OP_F_WT1_1, kZ1, kY1, kdT4, kModeGeneric, 1.0, 0.0, F, F, kY1, 1.0, -1, 0.0, F, F);
+  build_op(ctx, OP_F_DW0, kdT4, kZ0, kdDw, kModeGeneric, 2.0, 0.0, F, F, kdT4, 2.0);
+  build_op(ctx, OP_F_DW1, kdT4, kZ1, kdDw, kModeGeneric, 2.0, 0.0, F, F, kdT4, 2.0);
+  build_op(ctx, OP_F_T2W, kdT4, kHt, kT2, kModeGeneric, 1.0, 0.0, F);
   if (ctx->chain) {
     // the recursion's last products read its results, kept as upper tiles; F and s are written in full
     ctx->ops[OP_F_FIN].ops_upper = ctx->ops[OP_F_S].ops_upper = 1;
@@ -647,8 +653,8 @@ sedacs_status build_fermi_ops(sedacs_ctx* ctx) {
   // mu shift at a saved stage: U' = U Q + tau Q (U in kY0, Q = (I + tau U)^-1 in the Horner slot)
   // into either copy of kX; tau is set in g1 at run time
   for (int cu = 0; cu < 2; ++cu)
-    STCHK(build_op(ctx, OP_F_MOB_0 + cu, kY0, horner_slot(M), kX, kModeGeneric, 1.0, 0.0, F, F, horner_slot(M), 0.0,
-                   -1, 0.0, F, T, 0, 0, cu));
+    build_op(ctx, OP_F_MOB_0 + cu, kY0, horner_slot(M), kX, kModeGeneric, 1.0, 0.0, F, F, horner_slot(M), 0.0,
+                   -1, 0.0, F, T, 0, 0, cu);
   set_horner(ctx, fermi_inv(ctx));
   return SEDACS_OK;
 }
@@ -676,8 +682,8 @@ sedacs_status build_chain_tables(sedacs_ctx* ctx) {
   if (win.back() < n) win.push_back(n);
   ctx->n_ctiles = n;
   ctx->n_cwin = (int)win.size() - 1;
-  STCHK(stage_vec(ctx, &ctx->d_ctiles, tiles));
-  STCHK(stage_vec(ctx, &ctx->d_cwin, win));
+  stage_vec(ctx, &ctx->d_ctiles, tiles);
+  stage_vec(ctx, &ctx->d_cwin, win);
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_cdone), sizeof(unsigned) * std::max(1, L.n_sub)));
   return SEDACS_OK;
 }
@@ -691,23 +697,21 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   L = Layout();
   L.n_sub = P;
   const long long tot_rows = ctx->sub_ptr_h[P];
+  ctx->stage_host.clear();              // (an earlier rebuild may have stopped half way)
+  ctx->stage_recs.clear();
   // per-subgraph core counts
   std::vector<int> ncore(P);
   for (int i = 0; i < P; ++i) ncore[i] = ctx->part.leaves[i].count;
-  STCHK(upload_vec(ctx, &ctx->d_n_core, ncore));
   CUCHK(grow(&ctx->d_orb_off, &ctx->loc_cap, tot_rows) == cudaSuccess ? cudaSuccess : cudaErrorMemoryAllocation);
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_n_orb_sub), sizeof(int) * std::max(1, P)));
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_n_core_orb), sizeof(int) * std::max(1, P)));
-  launch_orb_offsets(ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_species, ctx->model, ctx->d_orb_off, ctx->d_n_orb_sub,
-                     ctx->d_n_core, ctx->d_n_core_orb, P, s);
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_n_orb), sizeof(int) * 2 * std::max(1, P)));
+  launch_orb_offsets(ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_species, ctx->model, ctx->d_orb_off, ctx->d_n_orb,
+                     ctx->part.leaves_d, ctx->d_n_orb + P, P, s);
   CUCHK(cudaGetLastError());
-  L.n_real.resize(P);
-  L.n_core_orb.resize(P);
-  CUCHK(cudaMemcpyAsync(L.n_real.data(), ctx->d_n_orb_sub, sizeof(int) * P, cudaMemcpyDeviceToHost, s));
-  CUCHK(cudaMemcpyAsync(L.n_core_orb.data(), ctx->d_n_core_orb, sizeof(int) * P, cudaMemcpyDeviceToHost, s));
-  ctx->sub_atoms_h.resize(tot_rows);
-  CUCHK(cudaMemcpyAsync(ctx->sub_atoms_h.data(), ctx->d_sub_atoms, sizeof(int) * tot_rows, cudaMemcpyDeviceToHost, s));
+  std::vector<int> orb(2 * P);
+  CUCHK(cudaMemcpyAsync(orb.data(), ctx->d_n_orb, sizeof(int) * 2 * P, cudaMemcpyDeviceToHost, s));
   CUCHK(cudaStreamSynchronize(s));
+  L.n_real.assign(orb.begin(), orb.begin() + P);
+  L.n_core_orb.assign(orb.begin() + P, orb.end());
   L.n_pad.resize(P);
   L.m_pad.resize(P);
   L.n_core_atoms = ncore;
@@ -761,8 +765,7 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
     ctx->arena_cap = want;
   }
   // views and per-subgraph offset arrays
-  for (int k = 0; k < kNumSlots; ++k) STCHK(stage_views(ctx, k, 0, &ctx->d_views[k]));
-  STCHK(stage_views(ctx, kX, 1, &ctx->d_views_x1));
+  STCHK(build_work(ctx));
   std::vector<long long> hoff(P), soff(P), dco(P), wco(P), rbase(P), troff(P), ddco(P), dhoff(P), dtco(P), duco(P),
       dwco(P);
   std::vector<int> npad(P), nreal(P), ndiag(P);
@@ -784,88 +787,83 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
     nreal[i] = L.n_real[i];
     ndiag[i] = L.n_diag[i];
   }
-  STCHK(stage_vec(ctx, &ctx->d_hoff, hoff));
-  STCHK(stage_vec(ctx, &ctx->d_soff, soff));
-  STCHK(stage_vec(ctx, &ctx->d_dcoff, dco));
-  STCHK(stage_vec(ctx, &ctx->d_wcoff, wco));
-  STCHK(stage_vec(ctx, &ctx->d_dcoff_d, ddco));
-  STCHK(stage_vec(ctx, &ctx->d_dcoff_t, dtco));
-  STCHK(stage_vec(ctx, &ctx->d_dcoff_u, duco));
-  STCHK(stage_vec(ctx, &ctx->d_dcoff_w, dwco));
-  STCHK(stage_vec(ctx, &ctx->d_dhoff, dhoff));
-  STCHK(stage_vec(ctx, &ctx->d_rowbase, rbase));
-  STCHK(stage_vec(ctx, &ctx->d_tr_off, troff));
-  STCHK(stage_vec(ctx, &ctx->d_n_pad, npad));
-  STCHK(stage_vec(ctx, &ctx->d_n_real, nreal));
-  STCHK(stage_vec(ctx, &ctx->d_n_diag, ndiag));
+  stage_vec(ctx, &ctx->d_hoff, hoff);
+  stage_vec(ctx, &ctx->d_soff, soff);
+  stage_vec(ctx, &ctx->d_dcoff, dco);
+  stage_vec(ctx, &ctx->d_wcoff, wco);
+  stage_vec(ctx, &ctx->d_dcoff_d, ddco);
+  stage_vec(ctx, &ctx->d_dcoff_t, dtco);
+  stage_vec(ctx, &ctx->d_dcoff_u, duco);
+  stage_vec(ctx, &ctx->d_dcoff_w, dwco);
+  stage_vec(ctx, &ctx->d_dhoff, dhoff);
+  stage_vec(ctx, &ctx->d_rowbase, rbase);
+  stage_vec(ctx, &ctx->d_tr_off, troff);
+  stage_vec(ctx, &ctx->d_n_pad, npad);
+  stage_vec(ctx, &ctx->d_n_real, nreal);
+  stage_vec(ctx, &ctx->d_n_diag, ndiag);
   if (ctx->chain) STCHK(build_chain_tables(ctx));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_glo), sizeof(double) * std::max(1LL, rb)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_ghi), sizeof(double) * std::max(1LL, rb)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_bounds), sizeof(double) * 2 * std::max(1, P)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_slots), sizeof(double) * std::max(1LL, L.tr_total)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_sp2), sizeof(Sp2State) * std::max(1, P)));
-  // subgraph-of-row, core lists, local index table, density-graph row pointers
-  std::vector<int> sor(tot_rows), csub, cloc;
-  std::vector<long long> gdp(N + 1, 0);
-  std::vector<int> gdlen(N, 0);
+  // local index table, subgraph-of-row, core lists and density-graph row pointers, filled on the device
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_loc), sizeof(int) * (size_t)N * std::max(1, P)));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_sub_of_row), sizeof(int) * std::max(1LL, tot_rows)));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_sub), sizeof(int) * N));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_local), sizeof(int) * N));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_len), sizeof(int) * N));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_ptr), sizeof(long long) * (N + 1)));
+  launch_sub_tables(ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->part.leaves_d, ctx->d_loc, ctx->d_sub_of_row, ctx->d_core_sub,
+                    ctx->d_core_local, ctx->d_gd_len, N, P, s);
+  launch_scan(ctx->d_gd_len, N, ctx->d_gd_ptr, s);
+  CUCHK(cudaGetLastError());
+  ctx->n_core_total = 0;
+  ctx->gd_nnz = 0;
   for (int i = 0; i < P; ++i) {
-    for (long long q = ctx->sub_ptr_h[i]; q < ctx->sub_ptr_h[i + 1]; ++q) sor[q] = i;
-    for (int a = 0; a < ncore[i]; ++a) {
-      csub.push_back(i);
-      cloc.push_back(a);
-      gdlen[ctx->sub_atoms_h[ctx->sub_ptr_h[i] + a]] = L.n_atoms[i];
-    }
+    ctx->n_core_total += ncore[i];
+    ctx->gd_nnz += (long long)ncore[i] * L.n_atoms[i];
   }
-  for (int A = 0; A < N; ++A) gdp[A + 1] = gdp[A] + gdlen[A];
-  ctx->n_core_total = (int)csub.size();
-  STCHK(stage_vec(ctx, &ctx->d_sub_of_row, sor));
-  STCHK(stage_vec(ctx, &ctx->d_core_sub, csub));
-  STCHK(stage_vec(ctx, &ctx->d_core_local, cloc));
-  STCHK(stage_vec(ctx, &ctx->d_gd_ptr, gdp));
-  ctx->gd_nnz = gdp[N];
   CUCHK(grow(&ctx->d_gd_col, &ctx->gd_cap, ctx->gd_nnz + 1) == cudaSuccess ? cudaSuccess : cudaErrorMemoryAllocation);
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_val), sizeof(double) * ctx->gd_cap));
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_loc), sizeof(int) * (size_t)N * std::max(1, P)));
-  launch_loc_fill(ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_loc, N, P, s);
-  CUCHK(cudaGetLastError());
   // GEMM tables
   // S^-1/2 in deviation form: Y = I + E_y (kY*), Z = I + E_z (kZ*), T = I + E_t (kT);
   // only products of the small deviations go through the tensor cores.
-  STCHK(build_op(ctx, OP_NS_Y1, kY0, kZ1, kY1, kModeGeneric, 1.f, 0.f, false, false, kY0, 1.f, kZ1, 1.f, false, true));
-  STCHK(build_op(ctx, OP_NS_T0, kZ0, kY0, kT, kModeGeneric, -0.5f, 0.f, false, false, kZ0, -0.5f, kY0, -0.5f, false, true));
-  STCHK(build_op(ctx, OP_NS_T1, kZ1, kY1, kT, kModeGeneric, -0.5f, 0.f, false, false, kZ1, -0.5f, kY1, -0.5f, false, true));
-  STCHK(build_op(ctx, OP_NS_Y0, kY0, kT, kY1, kModeGeneric, 1.f, 0.f, false, false, kY0, 1.f, kT, 1.f, false, true));
-  STCHK(build_op(ctx, OP_NS_Y1b, kY1, kT, kY0, kModeGeneric, 1.f, 0.f, false, false, kY1, 1.f, kT, 1.f, false, true));
-  STCHK(build_op(ctx, OP_NS_Z0, kT, kZ0, kZ1, kModeGeneric, 1.f, 0.f, false, false, kT, 1.f, kZ0, 1.f, false, true));
-  STCHK(build_op(ctx, OP_NS_Z1, kT, kZ1, kZ0, kModeGeneric, 1.f, 0.f, false, false, kT, 1.f, kZ1, 1.f, false, true));
-  STCHK(build_op(ctx, OP_TE2, kY0, kY0, kY1, kModeGeneric, 1.f, 0.f, false, false, -1, 0.f, -1, 0.f, false, true));
-  STCHK(build_op(ctx, OP_TE3, kY1, kY0, kT, kModeGeneric, 1.f, 0.f, false, false, -1, 0.f, -1, 0.f, false, true));
-  STCHK(build_op(ctx, OP_TZ, kT, kZ1, kZ0, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true));
+  build_op(ctx, OP_NS_Y1, kY0, kZ1, kY1, kModeGeneric, 1.f, 0.f, false, false, kY0, 1.f, kZ1, 1.f, false, true);
+  build_op(ctx, OP_NS_T0, kZ0, kY0, kT, kModeGeneric, -0.5f, 0.f, false, false, kZ0, -0.5f, kY0, -0.5f, false, true);
+  build_op(ctx, OP_NS_T1, kZ1, kY1, kT, kModeGeneric, -0.5f, 0.f, false, false, kZ1, -0.5f, kY1, -0.5f, false, true);
+  build_op(ctx, OP_NS_Y0, kY0, kT, kY1, kModeGeneric, 1.f, 0.f, false, false, kY0, 1.f, kT, 1.f, false, true);
+  build_op(ctx, OP_NS_Y1b, kY1, kT, kY0, kModeGeneric, 1.f, 0.f, false, false, kY1, 1.f, kT, 1.f, false, true);
+  build_op(ctx, OP_NS_Z0, kT, kZ0, kZ1, kModeGeneric, 1.f, 0.f, false, false, kT, 1.f, kZ0, 1.f, false, true);
+  build_op(ctx, OP_NS_Z1, kT, kZ1, kZ0, kModeGeneric, 1.f, 0.f, false, false, kT, 1.f, kZ1, 1.f, false, true);
+  build_op(ctx, OP_TE2, kY0, kY0, kY1, kModeGeneric, 1.f, 0.f, false, false, -1, 0.f, -1, 0.f, false, true);
+  build_op(ctx, OP_TE3, kY1, kY0, kT, kModeGeneric, 1.f, 0.f, false, false, -1, 0.f, -1, 0.f, false, true);
+  build_op(ctx, OP_TZ, kT, kZ1, kZ0, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true);
   // h~ = Z h Z = P + P E_z with P = h + E_z h
-  STCHK(build_op(ctx, OP_P0, kZ0, kH, kP, kModeGeneric, 1.f, 0.f, false, false, kH, 1.f));
-  STCHK(build_op(ctx, OP_P1, kZ1, kH, kP, kModeGeneric, 1.f, 0.f, false, false, kH, 1.f));
-  STCHK(build_op(ctx, OP_HT0, kP, kZ0, kHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true));
-  STCHK(build_op(ctx, OP_HT1, kP, kZ1, kHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true));
-  STCHK(build_op(ctx, OP_SP2, kX, kX, kX, kModeSp2, 1.f, 0.f, false, false, -1, 0.f, -1, 0.f, false, true));
+  build_op(ctx, OP_P0, kZ0, kH, kP, kModeGeneric, 1.f, 0.f, false, false, kH, 1.f);
+  build_op(ctx, OP_P1, kZ1, kH, kP, kModeGeneric, 1.f, 0.f, false, false, kH, 1.f);
+  build_op(ctx, OP_HT0, kP, kZ0, kHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true);
+  build_op(ctx, OP_HT1, kP, kZ1, kHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true);
+  build_op(ctx, OP_SP2, kX, kX, kX, kModeSp2, 1.f, 0.f, false, false, -1, 0.f, -1, 0.f, false, true);
   // core rows: T1 = Z_c X = X_c + E_z,c X ; D_c = 2 T1 Z = 2 (T1 + T1 E_z); W_c = 2 (T1 h~) Z
-  STCHK(build_op(ctx, OP_T1_0, kZ0, kX, kT1, kModeGeneric, 1.f, 0.f, true, false, kX, 1.f, -1, 0.f, true));
-  STCHK(build_op(ctx, OP_T1_1, kZ1, kX, kT1, kModeGeneric, 1.f, 0.f, true, false, kX, 1.f, -1, 0.f, true));
-  STCHK(build_op(ctx, OP_DC0, kT1, kZ0, kDc, kModeGeneric, 2.f, 0.f, false, false, kT1, 2.f));
-  STCHK(build_op(ctx, OP_DC1, kT1, kZ1, kDc, kModeGeneric, 2.f, 0.f, false, false, kT1, 2.f));
-  STCHK(build_op(ctx, OP_T2, kT1, kHt, kT2, kModeGeneric, 1.f, 0.f, false));
-  STCHK(build_op(ctx, OP_WC0, kT2, kZ0, kWc, kModeGeneric, 2.f, 0.f, false, false, kT2, 2.f));
-  STCHK(build_op(ctx, OP_WC1, kT2, kZ1, kWc, kModeGeneric, 2.f, 0.f, false, false, kT2, 2.f));
+  build_op(ctx, OP_T1_0, kZ0, kX, kT1, kModeGeneric, 1.f, 0.f, true, false, kX, 1.f, -1, 0.f, true);
+  build_op(ctx, OP_T1_1, kZ1, kX, kT1, kModeGeneric, 1.f, 0.f, true, false, kX, 1.f, -1, 0.f, true);
+  build_op(ctx, OP_DC0, kT1, kZ0, kDc, kModeGeneric, 2.f, 0.f, false, false, kT1, 2.f);
+  build_op(ctx, OP_DC1, kT1, kZ1, kDc, kModeGeneric, 2.f, 0.f, false, false, kT1, 2.f);
+  build_op(ctx, OP_T2, kT1, kHt, kT2, kModeGeneric, 1.f, 0.f, false);
+  build_op(ctx, OP_WC0, kT2, kZ0, kWc, kModeGeneric, 2.f, 0.f, false, false, kT2, 2.f);
+  build_op(ctx, OP_WC1, kT2, kZ1, kWc, kModeGeneric, 2.f, 0.f, false, false, kT2, 2.f);
   // response tables
-  STCHK(build_op(ctx, OP_RSP_A, kX, kR2, kR1, kModeGeneric, 1.f, 0.f, true, true));
-  STCHK(build_op(ctx, OP_RSP_B, kR2, kX, kR2, kModeRsp, 1.f, 0.f, false));
-  STCHK(build_op(ctx, OP_DP0, kZ0, kdH, kP, kModeGeneric, 1.f, 0.f, false, false, kdH, 1.f));
-  STCHK(build_op(ctx, OP_DP1, kZ1, kdH, kP, kModeGeneric, 1.f, 0.f, false, false, kdH, 1.f));
-  STCHK(build_op(ctx, OP_DHT0, kP, kZ0, kdHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true));
-  STCHK(build_op(ctx, OP_DHT1, kP, kZ1, kdHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true));
-  STCHK(build_op(ctx, OP_DT1_0, kZ0, kR2, kdT1, kModeGeneric, 1.f, 0.f, true, false, kR2, 1.f, -1, 0.f, true));
-  STCHK(build_op(ctx, OP_DT1_1, kZ1, kR2, kdT1, kModeGeneric, 1.f, 0.f, true, false, kR2, 1.f, -1, 0.f, true));
-  STCHK(build_op(ctx, OP_DDC0, kdT1, kZ0, kdDc, kModeGeneric, 2.f, 0.f, false, false, kdT1, 2.f));
-  STCHK(build_op(ctx, OP_DDC1, kdT1, kZ1, kdDc, kModeGeneric, 2.f, 0.f, false, false, kdT1, 2.f));
+  build_op(ctx, OP_RSP_A, kX, kR2, kR1, kModeGeneric, 1.f, 0.f, true, true);
+  build_op(ctx, OP_RSP_B, kR2, kX, kR2, kModeRsp, 1.f, 0.f, false);
+  build_op(ctx, OP_DP0, kZ0, kdH, kP, kModeGeneric, 1.f, 0.f, false, false, kdH, 1.f);
+  build_op(ctx, OP_DP1, kZ1, kdH, kP, kModeGeneric, 1.f, 0.f, false, false, kdH, 1.f);
+  build_op(ctx, OP_DHT0, kP, kZ0, kdHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true);
+  build_op(ctx, OP_DHT1, kP, kZ1, kdHt, kModeGeneric, 1.f, 0.f, false, false, kP, 1.f, -1, 0.f, false, true);
+  build_op(ctx, OP_DT1_0, kZ0, kR2, kdT1, kModeGeneric, 1.f, 0.f, true, false, kR2, 1.f, -1, 0.f, true);
+  build_op(ctx, OP_DT1_1, kZ1, kR2, kdT1, kModeGeneric, 1.f, 0.f, true, false, kR2, 1.f, -1, 0.f, true);
+  build_op(ctx, OP_DDC0, kdT1, kZ0, kdDc, kModeGeneric, 2.f, 0.f, false, false, kdT1, 2.f);
+  build_op(ctx, OP_DDC1, kdT1, kZ1, kdDc, kModeGeneric, 2.f, 0.f, false, false, kdT1, 2.f);
   STCHK(build_fermi_ops(ctx));
   CUCHK(cudaGetLastError());
   STCHK(flush_staged(ctx));
@@ -873,7 +871,15 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   ctx->have_subs = true;
   ctx->z_valid = false;
   ctx->sp2_iters_h.assign(P, 0);
-  CUCHK(cudaStreamSynchronize(s));
+  return SEDACS_OK;
+}
+
+// Subgraph atom lists on the host.
+sedacs_status sub_atoms_host(sedacs_ctx* ctx, std::vector<int>* atoms) {
+  atoms->resize(ctx->sub_ptr_h.back());
+  CUCHK(cudaStreamSynchronize(ctx->stream));
+  if (!atoms->empty())
+    CUCHK(cudaMemcpy(atoms->data(), ctx->d_sub_atoms, sizeof(int) * atoms->size(), cudaMemcpyDeviceToHost));
   return SEDACS_OK;
 }
 
@@ -892,7 +898,7 @@ void gather_hs(sedacs_ctx* ctx, const double* V = nullptr) {
                 ctx->d_n_pad, ctx->arena, L.n_sub, ctx->d_sub_of_row, ctx->sub_ptr_h[L.n_sub], 0, ctx->f64, s);
   ctx->launches += 3;
   if (!ctx->f64) {
-    launch_split_planes(ctx->d_views[kH], L.n_sub, max_rows(ctx), ctx->arena, ctx->nsplit_ns, false, s);
+    launch_split_planes(views(ctx, kH), L.n_sub, max_rows(ctx), ctx->arena, ctx->nsplit_ns, false, s);
     ctx->launches += 1;
   }
 }
@@ -919,10 +925,10 @@ bool compute_z_taylor(sedacs_ctx* ctx) {
   const Layout& L = ctx->lay;
   const int mr = max_rows(ctx);
   const int ns = ctx->nsplit_ns;
-  launch_affine_planes(ctx->d_views[kS], ctx->d_views[kY0], 1.0, -1.0, 1, ns, nullptr, 0.0, 0.0, 0, 0, 0, nullptr,
+  launch_affine_planes(views(ctx, kS), views(ctx, kY0), 1.0, -1.0, 1, ns, kNoViews, 0.0, 0.0, 0, 0, 0, nullptr,
                        L.n_sub, mr, ctx->arena, ctx->f64, s);                              // E = s - I
   run_op(ctx, OP_TE2, ns, ns);                                                         // E^2
-  launch_gershgorin(ctx->d_views[kY1], L.n_sub, mr, ctx->arena, ctx->d_glo, ctx->d_ghi, ctx->d_rowbase,
+  launch_gershgorin(views(ctx, kY1), L.n_sub, mr, ctx->arena, ctx->d_glo, ctx->d_ghi, ctx->d_rowbase,
                     ctx->d_bounds, ctx->f64, s);
   ctx->launches += 4;
   std::vector<double> b(2 * L.n_sub);
@@ -935,8 +941,8 @@ bool compute_z_taylor(sedacs_ctx* ctx) {
     if (L.n_real[i] > 0) worst = std::max(worst, b[2 * i + 1]);
   if (!(worst <= kTaylorMaxNorm * kTaylorMaxNorm)) return false;
   run_op(ctx, OP_TE3, ns, ns);                                                         // E^3
-  launch_poly3(ctx->d_views[kY0], ctx->d_views[kY1], ctx->d_views[kT], ctx->d_views[kZ1], 35.0 / 128, -63.0 / 256,
-               231.0 / 1024, 0, ns, ctx->d_views[kP], -0.5, 3.0 / 8, -5.0 / 16, 1, 0, L.n_sub, mr, ctx->arena,
+  launch_poly3(views(ctx, kY0), views(ctx, kY1), views(ctx, kT), views(ctx, kZ1), 35.0 / 128, -63.0 / 256,
+               231.0 / 1024, 0, ns, views(ctx, kP), -0.5, 3.0 / 8, -5.0 / 16, 1, 0, L.n_sub, mr, ctx->arena,
                ctx->f64, s);                                                           // Q (planes), L (master)
   run_op(ctx, OP_TZ, ns, ns);                                                          // E_z = E^3 Q + L
   ctx->launches += 1;
@@ -953,7 +959,7 @@ void compute_z(sedacs_ctx* ctx) {
   if (ctx->prm.ns_iters == 0 && !ctx->f64 && compute_z_taylor(ctx)) return;   // mixed forms
   // first step from Z0 = I: E_t = -E_y0 / 2 is also E_z1, so one pass writes E_y0 = s - I and
   // E_z1 = -(s - I) / 2 (masters and planes), and E_y1 = E_y0 + E_z1 + E_y0 E_z1
-  launch_affine_planes(ctx->d_views[kS], ctx->d_views[kY0], 1.0, -1.0, 1, ns, ctx->d_views[kZ1], -0.5, 0.5, 1, ns, 0,
+  launch_affine_planes(views(ctx, kS), views(ctx, kY0), 1.0, -1.0, 1, ns, views(ctx, kZ1), -0.5, 0.5, 1, ns, 0,
                        nullptr, L.n_sub, mr, ctx->arena, ctx->f64, s);
   run_op(ctx, OP_NS_Y1, ns, ns);                       // E_y1
   ctx->launches += 1;
@@ -973,7 +979,7 @@ void compute_ht(sedacs_ctx* ctx) {
   const int ns = ctx->nsplit_ns;
   run_op(ctx, ctx->zc == 0 ? OP_P0 : OP_P1, ns, ns);     // P = Z h
   run_op(ctx, ctx->zc == 0 ? OP_HT0 : OP_HT1, ns, ns);   // h~ = P Z
-  launch_gershgorin(ctx->d_views[kHt], ctx->lay.n_sub, max_rows(ctx), ctx->arena, ctx->d_glo, ctx->d_ghi,
+  launch_gershgorin(views(ctx, kHt), ctx->lay.n_sub, max_rows(ctx), ctx->arena, ctx->d_glo, ctx->d_ghi,
                     ctx->d_rowbase, ctx->d_bounds, ctx->f64, ctx->stream);
   ctx->launches += 2;
   ctx->bounds_h.resize(2 * ctx->lay.n_sub);
@@ -988,10 +994,10 @@ void launch_sp2_start(sedacs_ctx* ctx, bool with_dx) {
   const Layout& L = ctx->lay;
   const int n2 = with_dx ? ctx->nsplit_rsp : ctx->nsplit_sp2;
   const int x_master = (!ctx->f64 && (n2 == 3 || n2 == kPlanesF16x2)) ? 0 : 1;
-  launch_affine_planes(ctx->d_views[kHt], ctx->d_views[kX], 0.0, 0.0, x_master, n2, nullptr, 0.0, 0.0, 0, 0, 1,
+  launch_affine_planes(views(ctx, kHt), views(ctx, kX), 0.0, 0.0, x_master, n2, kNoViews, 0.0, 0.0, 0, 0, 1,
                        ctx->d_bounds, L.n_sub, max_rows(ctx), ctx->arena, ctx->f64, ctx->stream);
   if (with_dx)
-    launch_affine_planes(ctx->d_views[kdHt], ctx->d_views[kR2], 0.0, 0.0, 1, n2, nullptr, 0.0, 0.0, 0, 0, 2,
+    launch_affine_planes(views(ctx, kdHt), views(ctx, kR2), 0.0, 0.0, 1, n2, kNoViews, 0.0, 0.0, 0, 0, 2,
                          ctx->d_bounds, L.n_sub, max_rows(ctx), ctx->arena, ctx->f64, ctx->stream);
 }
 
@@ -1042,7 +1048,7 @@ sedacs_status run_sp2(sedacs_ctx* ctx, double mu, int kmax) {
     ctx->launches += 1;
   }
   if (ctx->nsplit_sp2 == kPlanesF16x2) {
-    launch_f16x2_to_bf16x3(ctx->d_views[kX], ctx->d_sp2, ctx->slot[kX].copy_stride, L.n_sub, mr, ctx->arena, s);
+    launch_f16x2_to_bf16x3(views(ctx, kX), ctx->d_sp2, ctx->slot[kX].copy_stride, L.n_sub, mr, ctx->arena, s);
     ctx->launches += 2;
   }
   if (ctx->kstats) {
@@ -1381,7 +1387,7 @@ sedacs_status run_fermi(sedacs_ctx* ctx, double mu, int nd) {
   const Layout& L = ctx->lay;
   const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
   const double b0 = std::ldexp(beta_of(ctx), -nd);
-  launch_affine_planes(ctx->d_views[kHt], ctx->d_views[kP], -0.5 * b0, 0.5 * b0 * mu, ctx->f64 ? 1 : 0, nf, nullptr,
+  launch_affine_planes(views(ctx, kHt), views(ctx, kP), -0.5 * b0, 0.5 * b0 * mu, ctx->f64 ? 1 : 0, nf, kNoViews,
                        0.0, 0.0, 0, 0, 0, nullptr, L.n_sub, max_rows(ctx), ctx->arena, ctx->f64, s);   // z
   ctx->launches += 1;
   const int js = std::max(0, nd - kReentryStages);
@@ -1796,13 +1802,16 @@ sedacs_status graph_core(sedacs_ctx* ctx, const long long* gptr, const int* gcol
   return check_dev_err(ctx);
 }
 
-sedacs_status halos_core(sedacs_ctx* ctx) {
+// wait: the tables are in place on return (a cycle waits at the end of its graph phase anyway).
+sedacs_status halos_core(sedacs_ctx* ctx, bool wait = true) {
   if (!ctx->have_graph || !ctx->have_cores) { ctx->err = "graph and cores are required"; return SEDACS_EINVAL; }
   std::vector<long long> old = ctx->sub_ptr_h;
   CUCHK(ctx->part.halos(ctx->d_row_ptr, ctx->d_col, ctx->N, &ctx->d_sub_ptr, &ctx->d_sub_atoms, &ctx->sub_cap,
                         ctx->sub_ptr_h, ctx->stream));
   ctx->launches += 3;
-  return rebuild_layout(ctx);
+  STCHK(rebuild_layout(ctx));
+  if (wait) CUCHK(cudaStreamSynchronize(ctx->stream));
+  return SEDACS_OK;
 }
 
 // one graph -> halos -> density cycle with the previous density graph
@@ -1817,7 +1826,7 @@ sedacs_status cycle(sedacs_ctx* ctx, double* mu, bool keep_prev = false) {
     STCHK(graph_core(ctx, ctx->d_xgd_ptr, ctx->d_xgd_col, ctx->d_xgd_val, keep_prev));
   else
     STCHK(graph_core(ctx, nullptr, nullptr, nullptr, keep_prev));
-  STCHK(halos_core(ctx));
+  STCHK(halos_core(ctx, false));
   phase_end(ctx, 0, 0);
   return density_core(ctx, mu);
 }
@@ -1845,7 +1854,7 @@ sedacs_status response_sp2(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
   launch_gather(ctx->model, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_species, ctx->d_pptr,
                 ctx->d_pcol, ctx->d_h0b, ctx->d_sb, ctx->d_loc, ctx->N, ctx->d_tmp, ctx->d_dhoff, ctx->d_soff,
                 ctx->d_n_pad, ctx->arena, L.n_sub, ctx->d_sub_of_row, ctx->sub_ptr_h[L.n_sub], 1, ctx->f64, s);
-  if (!ctx->f64) launch_split_planes(ctx->d_views[kdH], L.n_sub, mr, ctx->arena, ns, false, s);
+  if (!ctx->f64) launch_split_planes(views(ctx, kdH), L.n_sub, mr, ctx->arena, ns, false, s);
   ctx->launches += 8;
   run_op(ctx, ctx->zc == 0 ? OP_DP0 : OP_DP1, ns, ns);
   run_op(ctx, ctx->zc == 0 ? OP_DHT0 : OP_DHT1, ns, ns);
@@ -2186,21 +2195,12 @@ void sedacs_destroy(sedacs_ctx* ctx) {
                   ctx->d_dU, ctx->d_F, ctx->d_erep, ctx->d_tmp, ctx->d_tmp2, ctx->d_scal, ctx->d_vel, ctx->d_hist,
                   ctx->d_mass, ctx->d_zval, ctx->d_vec, ctx->d_row_ptr, ctx->d_col, ctx->d_pptr, ctx->d_pcol,
                   ctx->d_h0b, ctx->d_sb, ctx->d_gd_ptr, ctx->d_gd_col, ctx->d_gd_val, ctx->d_xgd_ptr, ctx->d_xgd_col,
-                  ctx->d_xgd_val, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_n_orb_sub, ctx->d_n_core,
-                  ctx->d_n_core_orb, ctx->d_sub_of_row, ctx->d_core_sub, ctx->d_core_local, ctx->d_loc, ctx->arena,
-                  ctx->d_views_x1, ctx->d_hoff, ctx->d_soff, ctx->d_dcoff, ctx->d_wcoff, ctx->d_rowbase,
-                  ctx->d_tr_off, ctx->d_n_pad, ctx->d_n_real, ctx->d_n_diag, ctx->d_glo, ctx->d_ghi, ctx->d_bounds,
-                  ctx->d_slots, ctx->d_sp2, ctx->d_nactive, ctx->d_dcoff_d, ctx->d_dqpop, ctx->d_dhoff,
-                  ctx->d_steps, ctx->d_rsp, ctx->d_dcoff_t, ctx->d_dcoff_u, ctx->d_dcoff_w, ctx->d_ctiles,
-                  ctx->d_cwin, ctx->d_cdone};
+                  ctx->d_xgd_val, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_n_orb, ctx->d_sub_of_row,
+                  ctx->d_core_sub, ctx->d_core_local, ctx->d_loc, ctx->d_gd_len, ctx->d_tables, ctx->arena,
+                  ctx->d_glo, ctx->d_ghi, ctx->d_bounds, ctx->d_slots, ctx->d_sp2, ctx->d_nactive, ctx->d_dqpop,
+                  ctx->d_steps, ctx->d_rsp, ctx->d_cdone};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  for (auto* v : ctx->d_views)
-    if (v) cudaFree(v);
-  for (auto& op : ctx->ops) {
-    if (op.mats_d) cudaFree(op.mats_d);
-    if (op.work_d) cudaFree(op.work_d);
-  }
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
   for (auto& e : ctx->kev)
@@ -2349,12 +2349,13 @@ sedacs_status sedacs_refine_cores(sedacs_ctx* ctx, int32_t rounds, int32_t min_c
   CUCHK(cudaMemcpy(rp.data(), ctx->d_row_ptr, sizeof(long long) * (N + 1), cudaMemcpyDeviceToHost));
   std::vector<int> col(rp[N]);
   if (rp[N] > 0) CUCHK(cudaMemcpy(col.data(), ctx->d_col, sizeof(int) * rp[N], cudaMemcpyDeviceToHost));
-  std::vector<int> norb(N), core_of(N, -1);
+  std::vector<int> norb(N), core_of(N, -1), sub_atoms;
+  STCHK(sub_atoms_host(ctx, &sub_atoms));
   for (int a = 0; a < N; ++a) norb[a] = ctx->model.n_orb[ctx->species_h[a]];
   std::vector<std::vector<int>> mem(P);
   for (int c = 0; c < P; ++c) {
     const int nc = ctx->lay.n_core_atoms[c];
-    for (int k = 0; k < nc; ++k) mem[c].push_back(ctx->sub_atoms_h[ctx->sub_ptr_h[c] + k]);
+    for (int k = 0; k < nc; ++k) mem[c].push_back(sub_atoms[ctx->sub_ptr_h[c] + k]);
     std::sort(mem[c].begin(), mem[c].end());
     for (int a : mem[c]) core_of[a] = c;
   }
@@ -2447,7 +2448,10 @@ sedacs_status sedacs_parts_get(sedacs_ctx* ctx, int64_t* sub_ptr, int32_t* sub_a
   if (!ctx || !ctx->have_subs) return SEDACS_EINVAL;
   const int P = ctx->lay.n_sub;
   if (sub_ptr) CUCHK(cudaMemcpy(sub_ptr, ctx->sub_ptr_h.data(), sizeof(int64_t) * (P + 1), cudaMemcpyDefault));
-  if (sub_atoms) CUCHK(cudaMemcpy(sub_atoms, ctx->sub_atoms_h.data(), sizeof(int) * ctx->sub_ptr_h[P], cudaMemcpyDefault));
+  if (sub_atoms) {
+    CUCHK(cudaMemcpyAsync(sub_atoms, ctx->d_sub_atoms, sizeof(int) * ctx->sub_ptr_h[P], cudaMemcpyDefault, ctx->stream));
+    CUCHK(cudaStreamSynchronize(ctx->stream));
+  }
   if (n_core) CUCHK(cudaMemcpy(n_core, ctx->lay.n_core_atoms.data(), sizeof(int) * P, cudaMemcpyDefault));
   return SEDACS_OK;
 }
@@ -2745,10 +2749,11 @@ sedacs_status sedacs_checkpoint_save(sedacs_ctx* ctx, const char* path) {
   CUCHK(cudaMemcpy(gcol.data(), ctx->d_gd_col, sizeof(int) * nnz, cudaMemcpyDeviceToHost));
   CUCHK(cudaMemcpy(gval.data(), ctx->d_gd_val, sizeof(double) * nnz, cudaMemcpyDeviceToHost));
   std::vector<long long> cptr(P + 1, 0);
-  std::vector<int> core;
+  std::vector<int> core, sub_atoms;
+  STCHK(sub_atoms_host(ctx, &sub_atoms));
   for (int i = 0; i < P; ++i) {
     const int nc = ctx->lay.n_core_atoms[i];
-    for (int a = 0; a < nc; ++a) core.push_back(ctx->sub_atoms_h[ctx->sub_ptr_h[i] + a]);
+    for (int a = 0; a < nc; ++a) core.push_back(sub_atoms[ctx->sub_ptr_h[i] + a]);
     cptr[i + 1] = cptr[i] + nc;
   }
   CkHeader h{};

@@ -38,10 +38,12 @@ enum SlotId : int {
   kNumSlots
 };
 
+enum WorkKind : int { kWorkSym = 0, kWorkSquare, kWorkRows, kNumWork };   // tile lists of a layout
+
 struct GemmOp {
-  GemmMat* mats_d = nullptr;
-  GemmWork* work_d = nullptr;
-  int n_work = 0;
+  GemmMat slot{};            // slot offsets, strides and flags
+  int a_rows = 0, b_rows = 0, out_rows = 0, c_rows = 0, c2_rows = 0;
+  WorkKind work = kWorkSym;
   double alpha = 1.0, beta = 0.0, g1 = 0.0, g2 = 0.0;
   int mode = kModeGeneric;
   bool sym = false;          // symmetric output: upper tiles only (counted as n^3 flops)
@@ -194,8 +196,8 @@ struct sedacs_ctx {
   int* d_sub_atoms = nullptr;
   long long sub_cap = 0;
   std::vector<long long> sub_ptr_h;
-  std::vector<int> sub_atoms_h;
-  int *d_orb_off = nullptr, *d_n_orb_sub = nullptr, *d_n_core = nullptr, *d_n_core_orb = nullptr;
+  int *d_orb_off = nullptr, *d_n_orb = nullptr;   // orbital offsets; orbitals per subgraph, then per core
+  int* d_gd_len = nullptr;                          // density-graph row lengths
   int *d_sub_of_row = nullptr, *d_core_sub = nullptr, *d_core_local = nullptr, *d_loc = nullptr;
   long long loc_cap = 0, rows_cap = 0;
   int n_core_total = 0;
@@ -205,8 +207,9 @@ struct sedacs_ctx {
   uint8_t* arena = nullptr;
   size_t arena_cap = 0;
   sedacs::GemmOp ops[sedacs::OP_NUM];
-  sedacs::SubView* d_views[sedacs::kNumSlots] = {};
-  sedacs::SubView* d_views_x1 = nullptr;   // X copy 1
+  sedacs::GemmSub* d_subs = nullptr;           // placement of every subgraph (one table per layout)
+  sedacs::GemmWork* d_work[sedacs::kNumWork] = {};
+  int n_work[sedacs::kNumWork] = {};
   long long *d_hoff = nullptr, *d_soff = nullptr, *d_dcoff = nullptr, *d_wcoff = nullptr, *d_rowbase = nullptr;
   long long* d_tr_off = nullptr;
   int *d_n_pad = nullptr, *d_n_real = nullptr, *d_n_diag = nullptr;
@@ -245,10 +248,11 @@ struct sedacs_ctx {
   // SP2 step control: per-step active counts copied into pinned host memory, one event per
   // step, so that the host waits on a step a few launches back instead of draining the stream
   bool have_xgd = false;  // a density graph was given to sedacs_graph_build (d_xgd_*)
-  // Layout uploads staged in one host buffer and sent from pinned memory in one go
-  // (rebuild_layout): (device destination, offset in stage_host, bytes)
+  // a layout's tables: staged in one host buffer, sent to one device block (rebuild_layout); the table
+  // pointers of this context point into the block: (pointer, offset in the block)
   std::vector<uint8_t> stage_host;
-  std::vector<std::tuple<void*, size_t, size_t>> stage_recs;
+  std::vector<std::pair<void**, size_t>> stage_recs;
+  uint8_t* d_tables = nullptr;
   uint8_t* stage_pinned = nullptr;
   size_t stage_pinned_cap = 0;
   bool fuse_forces = false;  // the next density's observables pass also contracts the forces

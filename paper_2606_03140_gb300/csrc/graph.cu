@@ -782,12 +782,27 @@ cudaError_t GraphBuilder::build(const double* dR, int N, const double box[3], do
 Partitioner::~Partitioner() { release(); }
 
 void Partitioner::release() {
-  for (void* p : {(void*)perm, (void*)skey, (void*)wrapped, (void*)sidx, (void*)segs_d, (void*)bits, (void*)hcnt})
+  for (void* p : {(void*)perm, (void*)skey, (void*)wrapped, (void*)sidx, (void*)segs_d, (void*)leaves_d, (void*)bits, (void*)hcnt})
     if (p) cudaFree(p);
-  perm = nullptr; skey = wrapped = nullptr; sidx = nullptr; segs_d = nullptr; bits = nullptr; hcnt = nullptr;
-  cap_n = cap_scr = cap_seg = 0;
+  perm = nullptr; skey = wrapped = nullptr; sidx = nullptr; segs_d = leaves_d = nullptr; bits = nullptr; hcnt = nullptr;
+  cap_n = cap_scr = cap_seg = cap_leaves = 0;
   cap_hcnt = cap_subptr = 0;
   cap_bits = 0;
+}
+
+void launch_scan(const int* cnt, int N, long long* out, cudaStream_t s) { scan_kernel<<<1, 1024, 0, s>>>(cnt, N, out); }
+
+cudaError_t Partitioner::upload_leaves(cudaStream_t s) {
+  const int n = (int)leaves.size();
+  if (n > cap_leaves) {
+    if (leaves_d) cudaFree(leaves_d);
+    leaves_d = nullptr;
+    cap_leaves = 0;
+    const cudaError_t e = cudaMalloc(&leaves_d, sizeof(RcbSeg) * n);
+    if (e) return e;
+    cap_leaves = n;
+  }
+  return cudaMemcpyAsync(leaves_d, leaves.data(), sizeof(RcbSeg) * n, cudaMemcpyHostToDevice, s);
 }
 
 static int next_pow2(int n) { int p = 1; while (p < n) p <<= 1; return p; }
@@ -848,8 +863,7 @@ cudaError_t Partitioner::rcb(const double* dR, int N, const double box[3], int c
     if ((e = cudaMalloc(&wrapped, sizeof(double) * 3 * need_scr))) return e;   // (need_scr >= N)
     cap_scr = need_scr;
   }
-  const int n_seg = (int)hs.size();
-  hs.insert(hs.end(), leaves.begin(), leaves.end());
+  if ((e = upload_leaves(s))) return e;
   if ((int)hs.size() > cap_seg) {
     if (segs_d) cudaFree(segs_d);
     segs_d = nullptr;
@@ -858,11 +872,11 @@ cudaError_t Partitioner::rcb(const double* dR, int N, const double box[3], int c
     cap_seg = (int)hs.size();
   }
   CellGrid g = make_grid(box, 1.0);
-  cudaMemcpyAsync(segs_d, hs.data(), sizeof(RcbSeg) * hs.size(), cudaMemcpyHostToDevice, s);
+  if (!hs.empty()) cudaMemcpyAsync(segs_d, hs.data(), sizeof(RcbSeg) * hs.size(), cudaMemcpyHostToDevice, s);
   rcb_wrap_kernel<<<(N + 127) / 128, 128, 0, s>>>(dR, N, g, wrapped, perm);
   for (size_t l = 0; l + 1 < first.size(); ++l)
     rcb_split_kernel<<<first[l + 1] - first[l], 1024, 0, s>>>(segs_d + first[l], perm, wrapped, N, skey, sidx);
-  rcb_leaf_kernel<<<(int)leaves.size(), 256, 0, s>>>(segs_d + n_seg, perm, skey, sidx);
+  rcb_leaf_kernel<<<(int)leaves.size(), 256, 0, s>>>(leaves_d, perm, skey, sidx);
   if ((e = cudaGetLastError())) return e;
   return cudaStreamSynchronize(s);
 }
@@ -875,11 +889,6 @@ cudaError_t Partitioner::set_cores(const std::vector<std::vector<int>>& cores, i
     cap_n = N;
   }
   n_parts = (int)cores.size();
-  if (n_parts + 1 > cap_seg) {
-    if (segs_d) cudaFree(segs_d);
-    if ((e = cudaMalloc(&segs_d, sizeof(RcbSeg) * (n_parts + 1)))) return e;
-    cap_seg = n_parts + 1;
-  }
   std::vector<int> hp;
   leaves.clear();
   for (auto& c : cores) {
@@ -888,6 +897,7 @@ cudaError_t Partitioner::set_cores(const std::vector<std::vector<int>>& cores, i
   }
   if ((int)hp.size() > cap_n) return cudaErrorInvalidValue;
   cudaMemcpyAsync(perm, hp.data(), sizeof(int) * hp.size(), cudaMemcpyHostToDevice, s);
+  if ((e = upload_leaves(s))) return e;
   return cudaStreamSynchronize(s);
 }
 
@@ -907,8 +917,7 @@ cudaError_t Partitioner::halos(const long long* row_ptr, const int* col, int N, 
     if ((e = cudaMalloc(&hcnt, sizeof(int) * n_parts))) return e;
     cap_hcnt = n_parts;
   }
-  cudaMemcpyAsync(segs_d, leaves.data(), sizeof(RcbSeg) * leaves.size(), cudaMemcpyHostToDevice, s);
-  halo_mark_kernel<<<n_parts, 256, 0, s>>>(row_ptr, col, perm, segs_d, bits, words);
+  halo_mark_kernel<<<n_parts, 256, 0, s>>>(row_ptr, col, perm, leaves_d, bits, words);
   halo_count_kernel<<<n_parts, 256, 0, s>>>(bits, words, hcnt);
   std::vector<int> hh(n_parts);
   cudaMemcpyAsync(hh.data(), hcnt, sizeof(int) * n_parts, cudaMemcpyDeviceToHost, s);
@@ -929,8 +938,8 @@ cudaError_t Partitioner::halos(const long long* row_ptr, const int* col, int N, 
     cap_subptr = n_parts + 1;
   }
   cudaMemcpyAsync(*sub_ptr_d, sub_ptr_h.data(), sizeof(long long) * (n_parts + 1), cudaMemcpyHostToDevice, s);
-  sub_fill_kernel<<<n_parts, 128, 0, s>>>(bits, words, perm, segs_d, *sub_ptr_d, *sub_atoms_d);
-  return cudaStreamSynchronize(s);
+  sub_fill_kernel<<<n_parts, 128, 0, s>>>(bits, words, perm, leaves_d, *sub_ptr_d, *sub_atoms_d);
+  return cudaGetLastError();
 }
 
 }  // namespace sedacs

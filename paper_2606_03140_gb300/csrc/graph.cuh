@@ -55,20 +55,25 @@ struct Partitioner {
   double* wrapped = nullptr;  // wrapped coordinates, [axis][atom]
   int* sidx = nullptr;
   RcbSeg* segs_d = nullptr;
+  RcbSeg* leaves_d = nullptr; // core segments in perm
   unsigned* bits = nullptr;
   int* hcnt = nullptr;
-  int cap_n = 0, cap_seg = 0, cap_hcnt = 0, cap_subptr = 0;
+  int cap_n = 0, cap_seg = 0, cap_leaves = 0, cap_hcnt = 0, cap_subptr = 0;
   long long cap_scr = 0, cap_bits = 0;
   int n_parts = 0;
   std::vector<RcbSeg> leaves;       // core segments in perm (host copy)
   std::vector<int> halo_count_h;
   ~Partitioner();
   void release();
+  cudaError_t upload_leaves(cudaStream_t s);
   cudaError_t rcb(const double* dR, int N, const double box[3], int core_size, cudaStream_t s);
   cudaError_t set_cores(const std::vector<std::vector<int>>& cores, int N, cudaStream_t s);
   // Halos of the current cores on graph (row_ptr, col); writes the subgraph atom lists.
   cudaError_t halos(const long long* row_ptr, const int* col, int N, long long** sub_ptr_d, int** sub_atoms_d,
                     long long* sub_cap, std::vector<long long>& sub_ptr_h, cudaStream_t s);
 };
+
+// Exclusive scan of N counts into offsets out[0 .. N].
+void launch_scan(const int* cnt, int N, long long* out, cudaStream_t s);
 
 }  // namespace sedacs

@@ -144,22 +144,36 @@ __global__ void pair_blocks_kernel(const ModelDev m, const double* R, const int*
   }
 }
 
-__global__ void loc_fill_kernel(const long long* sub_ptr, const int* sub_atoms, int* loc, int N) {
+// Per-atom tables of the subgraphs, block per subgraph: local index of every atom (loc), subgraph of every row of
+// the atom lists, subgraph and local index of every core atom (in the order of the cores) and the length of its
+// density-graph row.
+__global__ void sub_tables_kernel(const long long* sub_ptr, const int* sub_atoms, const RcbSeg* leaves, int* loc,
+                                  int* sub_of_row, int* core_sub, int* core_local, int* gd_len, int N) {
   const int i = blockIdx.x;
+  const RcbSeg lf = leaves[i];
   int* L = loc + (long long)i * N;
-  for (long long q = sub_ptr[i] + threadIdx.x; q < sub_ptr[i + 1]; q += blockDim.x)
-    L[sub_atoms[q]] = (int)(q - sub_ptr[i]);
+  const long long q0 = sub_ptr[i], q1 = sub_ptr[i + 1];
+  for (long long q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
+    const int a = sub_atoms[q], k = (int)(q - q0);
+    L[a] = k;
+    sub_of_row[q] = i;
+    if (k < lf.count) {
+      core_sub[lf.start + k] = i;
+      core_local[lf.start + k] = k;
+      gd_len[a] = (int)(q1 - q0);
+    }
+  }
 }
 
 // Orbital offsets of every subgraph atom: warp per subgraph, shuffle prefix sums over chunks
 // of 32 atoms.
 __global__ void orb_offsets_kernel(const long long* sub_ptr, const int* sub_atoms, const int* species, ModelDev m,
-                                   int* orb_off, int* n_orb_sub, const int* n_core, int* n_core_orb, int n_sub) {
+                                   int* orb_off, int* n_orb_sub, const RcbSeg* leaves, int* n_core_orb, int n_sub) {
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n_sub) return;
   const long long q0 = sub_ptr[i], q1 = sub_ptr[i + 1];
-  const int nc = n_core[i];
+  const int nc = leaves[i].count;
   int o = 0;                                   // orbitals before this chunk
   for (long long qb = q0; qb < q1; qb += 32) {
     const long long q = qb + lane;
@@ -412,14 +426,15 @@ void launch_pair_blocks(const ModelDev& m, const double* R, const int* species, 
   else pair_blocks_kernel<float><<<N, 64, 0, s>>>(m, R, species, pptr, pcol, N, g, (float*)h0b, (float*)sb);
 }
 
-void launch_loc_fill(const long long* sub_ptr, const int* sub_atoms, int* loc, int N, int n_sub, cudaStream_t s) {
+void launch_sub_tables(const long long* sub_ptr, const int* sub_atoms, const RcbSeg* leaves, int* loc, int* sub_of_row,
+                       int* core_sub, int* core_local, int* gd_len, int N, int n_sub, cudaStream_t s) {
   cudaMemsetAsync(loc, 0xFF, sizeof(int) * (size_t)N * n_sub, s);
-  loc_fill_kernel<<<n_sub, 128, 0, s>>>(sub_ptr, sub_atoms, loc, N);
+  sub_tables_kernel<<<n_sub, 128, 0, s>>>(sub_ptr, sub_atoms, leaves, loc, sub_of_row, core_sub, core_local, gd_len, N);
 }
 
 void launch_orb_offsets(const long long* sub_ptr, const int* sub_atoms, const int* species, const ModelDev& m,
-                        int* orb_off, int* n_orb_sub, const int* n_core, int* n_core_orb, int n_sub, cudaStream_t s) {
-  orb_offsets_kernel<<<(n_sub + 3) / 4, 128, 0, s>>>(sub_ptr, sub_atoms, species, m, orb_off, n_orb_sub, n_core,
+                        int* orb_off, int* n_orb_sub, const RcbSeg* leaves, int* n_core_orb, int n_sub, cudaStream_t s) {
+  orb_offsets_kernel<<<(n_sub + 3) / 4, 128, 0, s>>>(sub_ptr, sub_atoms, species, m, orb_off, n_orb_sub, leaves,
                                                      n_core_orb, n_sub);
 }
 

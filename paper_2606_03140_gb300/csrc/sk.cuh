@@ -1,6 +1,7 @@
 // Slater-Koster model kernels: pair blocks, padded H/S gather, collected observables.
 #pragma once
 #include "common.cuh"
+#include "graph.cuh"
 
 namespace sedacs {
 
@@ -11,9 +12,11 @@ struct SkGeom {
 
 void launch_pair_blocks(const ModelDev& m, const double* R, const int* species, const long long* pptr, const int* pcol,
                         int N, const SkGeom& g, void* h0b, void* sb, bool f64, cudaStream_t s);
-void launch_loc_fill(const long long* sub_ptr, const int* sub_atoms, int* loc, int N, int n_sub, cudaStream_t s);
+// Local index table loc [n_sub][N] (-1: not in the subgraph) and the per-atom tables of the subgraphs.
+void launch_sub_tables(const long long* sub_ptr, const int* sub_atoms, const RcbSeg* leaves, int* loc, int* sub_of_row,
+                       int* core_sub, int* core_local, int* gd_len, int N, int n_sub, cudaStream_t s);
 void launch_orb_offsets(const long long* sub_ptr, const int* sub_atoms, const int* species, const ModelDev& m,
-                        int* orb_off, int* n_orb_sub, const int* n_core, int* n_core_orb, int n_sub, cudaStream_t s);
+                        int* orb_off, int* n_orb_sub, const RcbSeg* leaves, int* n_core_orb, int n_sub, cudaStream_t s);
 void launch_gather(const ModelDev& m, const long long* sub_ptr, const int* sub_atoms, const int* orb_off,
                    const int* species, const long long* pptr, const int* pcol, const void* h0b, const void* sb,
                    const int* loc, int N, const double* V, const long long* hoff, const long long* soff,
