@@ -39,6 +39,8 @@ struct GemmMat {
   long long c_plane;             // bytes between the planes of C1
 };
 
+constexpr int kF64Tile = 32, kF64Threads = 128;   // FP64 products
+
 struct GemmWork {
   int mat, tm, tn, pad;
 };

@@ -405,26 +405,29 @@ sedacs_status flush_staged(sedacs_ctx* ctx) {
   return SEDACS_OK;
 }
 
-// Placement table and tile lists of the current layout.  FP64 tiles (64 x 64) with nothing but padding are left
-// out: the products read rows of listed tiles and columns below the valid inner dimension only.
+// Placement table and tile lists of the current layout, tiles of padding (which are only set to zero) last.
 sedacs_status build_work(sedacs_ctx* ctx) {
   const Layout& L = ctx->lay;
   std::vector<GemmSub> subs(L.n_sub);
   std::vector<GemmWork> work[kNumWork];
-  for (int i = 0; i < L.n_sub; ++i) {
+  const int tile = ctx->tile;
+  for (int i = 0; i < L.n_sub; ++i)
     subs[i] = GemmSub{L.sq_off[i], L.rw_off[i], L.tr_off[i], L.n_pad[i], L.n_real[i], L.n_core_orb[i], L.m_pad[i]};
-    if (L.n_real[i] == 0) continue;
-    const int tile = ctx->tile;
-    const int n = ctx->f64 ? (L.n_real[i] + tile - 1) / tile : L.n_pad[i] / tile;
-    const int m = ctx->f64 ? (L.n_core_orb[i] + tile - 1) / tile : L.m_pad[i] / tile;
-    for (int tm = 0; tm < n; ++tm)
-      for (int tn = 0; tn < n; ++tn) {
-        work[kWorkSquare].push_back({i, tm, tn, 0});
-        if (tn >= tm) work[kWorkSym].push_back({i, tm, tn, 0});
-      }
-    for (int tm = 0; tm < m; ++tm)
-      for (int tn = 0; tn < n; ++tn) work[kWorkRows].push_back({i, tm, tn, 0});
-  }
+  for (const bool padding : {false, true})
+    for (int i = 0; i < L.n_sub; ++i) {
+      if (L.n_real[i] == 0) continue;
+      auto add = [&](int kind, int tm, int tn, int rows) {
+        if (padding == (tm * tile >= rows || tn * tile >= L.n_real[i])) work[kind].push_back({i, tm, tn, 0});
+      };
+      const int n = L.n_pad[i] / tile, m = L.m_pad[i] / tile;
+      for (int tm = 0; tm < n; ++tm)
+        for (int tn = 0; tn < n; ++tn) {
+          add(kWorkSquare, tm, tn, L.n_real[i]);
+          if (tn >= tm) add(kWorkSym, tm, tn, L.n_real[i]);
+        }
+      for (int tm = 0; tm < m; ++tm)
+        for (int tn = 0; tn < n; ++tn) add(kWorkRows, tm, tn, L.n_core_orb[i]);
+    }
   stage_vec(ctx, &ctx->d_subs, subs);
   for (int k = 0; k < kNumWork; ++k) {
     stage_vec(ctx, &ctx->d_work[k], work[k]);
@@ -2143,7 +2146,7 @@ sedacs_status sedacs_create(int32_t n_atoms, const int32_t* species, const doubl
   ctx->n_electrons = 0.0;
   for (int i = 0; i < n_atoms; ++i) ctx->n_electrons += model->z_val[species[i]];
   ctx->f64 = params->precision == 0;
-  ctx->tile = ctx->f64 ? 64 : 128;
+  ctx->tile = ctx->f64 ? kF64Tile : 128;
   ctx->nsplit_ns = 3;
   // SP2 operand format: 1 = two fp16 planes; 4 = three bf16 planes; 2 = two bf16 planes; 3 = one
   const int sp2_fmt[5] = {3, kPlanesF16x2, 2, 1, 3};
