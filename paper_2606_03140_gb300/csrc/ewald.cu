@@ -7,11 +7,11 @@
 //   a_IJ = 1 / sqrt(2 (sigma_I^2 + sigma_J^2)),  sigma_I = 1 / (sqrt(pi) U_I).
 //
 // Reciprocal space uses separable phase tables: e^{ik.R} = X[m1] Y[m2] Z[m3] with
-// X[m] = exp(2 pi i m x / L).  k-vectors are grouped in rows of fixed (m1, m2); one CTA
-// accumulates a row's structure factor over a chunk of atoms (products X*Y once per atom
-// in shared memory, the Z table row read coalesced), partial sums are reduced in FP64 in a
-// fixed order.  The potential kernel keeps each atom's Z row in shared memory and streams
-// the k-rows.  T = float for the mixed path (FP64 final sums), double for the plain path.
+// X[m] = exp(2 pi i m x / L).  k-vectors are grouped in rows of fixed (m1, m2).  The structure factor runs a
+// block over a few rows and a chunk of atoms, a thread per pair +-m3, with the products X Y of the rows and the
+// Z phases of the atoms staged in shared memory; partial sums are reduced in FP64 in a fixed order.  The
+// potential kernel keeps each atom's Z phases in shared memory and takes four k-rows at a time.  T = float for
+// the mixed path (FP64 final sums), double for the plain path.
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -33,12 +33,16 @@ __device__ __forceinline__ typename C2<T>::t cmul(typename C2<T>::t a, typename 
   return r;
 }
 
+// a b + c d with one rounding of c d: which product is rounded first is the same for a phase and its conjugate.
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+
 // Phase tables in FP64, stored as T: tab[(axis * N + J) * (nmax + 1) + m] = exp(2 pi i m u), u = x / L.
 template <typename T>
 __global__ void phase_table_kernel(const double* R, int N, EwaldGeom g, typename C2<T>::t* tab) {
-  const int J = blockIdx.x * blockDim.x + threadIdx.x;
+  const int J = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
   if (J >= N) return;
-  for (int a = 0; a < 3; ++a) {
+  {
     const double u = R[3 * J + a] / g.box_b[a] / kBohrA * 1.0;   // x (A) -> bohr -> fraction
     double s, c;
     sincospi(2.0 * (u - floor(u)), &s, &c);
@@ -55,102 +59,118 @@ __global__ void phase_table_kernel(const double* R, int N, EwaldGeom g, typename
   }
 }
 
-// S_row[m3] partial over an atom chunk, for nvec charge vectors.
-template <typename T, int NV>
-__global__ void structure_factor_kernel(const KRow* rows, const typename C2<T>::t* tab, const double* b0,
-                                        const double* b1, int N, int nmax_all, int chunk, double* part,
-                                        long long nk_total) {
+// S(k) partial over an atom chunk.  A block takes the k-row entries (row, m3 >= 0) of its table line, one thread
+// each, which also covers -m3 (the conjugate phase); four sums per k-vector, over every fourth atom of the chunk,
+// are added in a fixed order in FP64.  Per 64 atoms the block forms b X Y for its rows and stages the atoms' Z
+// phases.  Five FP32 operations a k-vector and atom (the products that +-m3 share are formed once) against three
+// shared-memory reads for both, which bound it.  Measured (GB300, 30,000 atoms): 0.59 ms against 2.95 ms with a
+// block per row, whose lanes were half empty and which fetched Z for every row again.
+constexpr int kSfThreads = 256, kSfRows = 32, kSfAtoms = 64;
+
+template <typename T>
+__global__ void __launch_bounds__(kSfThreads) structure_factor_kernel(const SfBlock* blocks, const int2* entries,
+                                                                      const KRow* rows, const typename C2<T>::t* tab,
+                                                                      const double* b, int N, int nmax_all, int m3max,
+                                                                      int chunk, double* part, long long nk_total) {
   using CT = typename C2<T>::t;
-  const KRow kr = rows[blockIdx.x];
-  const int a0 = blockIdx.y * chunk;
-  const int a1 = min(N, a0 + chunk);
+  const SfBlock blk = blocks[blockIdx.x];
+  const int a0 = blockIdx.y * chunk, a1 = min(N, a0 + chunk);
   extern __shared__ unsigned char sm[];
-  CT* c12 = reinterpret_cast<CT*>(sm);   // [chunk][NV]
-  for (int J = a0 + threadIdx.x; J < a1; J += blockDim.x) {
-    CT x = tab[(0LL * N + J) * (nmax_all + 1) + kr.m1];
-    const int am2 = abs(kr.m2);
-    CT y = tab[(1LL * N + J) * (nmax_all + 1) + am2];
-    if (kr.m2 < 0) y.y = -y.y;
-    const CT xy = cmul<T>(x, y);
-    CT v0;
-    v0.x = (T)b0[J] * xy.x;
-    v0.y = (T)b0[J] * xy.y;
-    c12[(J - a0) * NV] = v0;
-    if (NV > 1) {
-      CT v1;
-      v1.x = (T)b1[J] * xy.x;
-      v1.y = (T)b1[J] * xy.y;
-      c12[(J - a0) * NV + 1] = v1;
+  CT* c12 = reinterpret_cast<CT*>(sm);                       // [row][kSfAtoms + 1]
+  CT* zs = c12 + kSfRows * (kSfAtoms + 1);                   // [atom][m3max + 1]
+  const int zw = m3max + 1;
+  const bool mine = (int)threadIdx.x < blk.n_entries;
+  const int2 en = mine ? entries[blk.entry0 + threadIdx.x] : make_int2(blk.row0, 0);
+  const CT* c = c12 + (en.x - blk.row0) * (kSfAtoms + 1);
+  T pr[4], pi[4], nr[4], ni[4];                              // +m3 and -m3
+#pragma unroll
+  for (int g = 0; g < 4; ++g) pr[g] = pi[g] = nr[g] = ni[g] = 0;
+  for (int j0 = a0; j0 < a1; j0 += kSfAtoms) {
+    const int n = min(kSfAtoms, a1 - j0);
+    __syncthreads();
+    for (int q = threadIdx.x; q < blk.n_rows * kSfAtoms; q += kSfThreads) {
+      const int r = q / kSfAtoms, j = q % kSfAtoms;
+      CT v;
+      v.x = v.y = 0;
+      if (j < n) {
+        const KRow kr = rows[blk.row0 + r];
+        const int J = j0 + j;
+        const CT x = tab[(0LL * N + J) * (nmax_all + 1) + kr.m1];
+        CT y = tab[(1LL * N + J) * (nmax_all + 1) + abs(kr.m2)];
+        if (kr.m2 < 0) y.y = -y.y;
+        v.x = (T)b[J] * dot2(x.x, y.x, -x.y, y.y);
+        v.y = (T)b[J] * dot2(x.y, y.x, x.x, y.y);
+      }
+      c12[r * (kSfAtoms + 1) + j] = v;
     }
-  }
-  __syncthreads();
-  // 4 groups of 64 threads: lane = m3 slot, group = every 4th atom of the chunk; the group
-  // partials are added in a fixed order through shared memory.
-  const int nm3 = kr.m3hi - kr.m3lo + 1;
-  const int grp = threadIdx.x >> 6, ln = threadIdx.x & 63;
-  T* red = reinterpret_cast<T*>(c12 + (size_t)chunk * NV);   // [4][64][NV][2] after the products
-  for (int base = 0; base < nm3; base += 64) {      // block-uniform loop over 64 m3 slots at a time
-    T sr[NV], si[NV];
+    for (int q = threadIdx.x; q < n * zw; q += kSfThreads) {
+      const int j = q / zw, m = q % zw;
+      zs[j * zw + m] = tab[(2LL * N + j0 + j) * (nmax_all + 1) + m];
+    }
+    __syncthreads();
+    if (!mine) continue;
+    const CT* z = zs + en.y;
+    int j = 0;
+    for (; j + 4 <= n; j += 4) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) { sr[v] = 0; si[v] = 0; }
-    const int t = base + ln;
-    const int m3 = kr.m3lo + t;
-    const int am3 = abs(m3);
-    if (t < nm3) {
-      for (int J = a0 + grp; J < a1; J += 4) {
-        CT z = tab[(2LL * N + J) * (nmax_all + 1) + am3];
-        if (m3 < 0) z.y = -z.y;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const CT c = c12[(J - a0) * NV + v];
-          sr[v] += c.x * z.x - c.y * z.y;
-          si[v] += c.x * z.y + c.y * z.x;
-        }
+      for (int g = 0; g < 4; ++g) {
+        const CT cv = c[j + g], zp = z[(j + g) * zw];
+        pr[g] += dot2(cv.x, zp.x, -cv.y, zp.y);
+        pi[g] += dot2(cv.x, zp.y, cv.y, zp.x);
+        nr[g] += dot2(cv.x, zp.x, cv.y, zp.y);
+        ni[g] += dot2(cv.x, -zp.y, cv.y, zp.x);
       }
     }
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      red[((grp * 64 + ln) * NV + v) * 2] = sr[v];
-      red[((grp * 64 + ln) * NV + v) * 2 + 1] = si[v];
-    }
-    __syncthreads();
-    if (grp == 0 && t < nm3) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        double re = 0.0, im = 0.0;
-        for (int g2 = 0; g2 < 4; ++g2) {
-          re += (double)red[((g2 * 64 + ln) * NV + v) * 2];
-          im += (double)red[((g2 * 64 + ln) * NV + v) * 2 + 1];
-        }
-        const long long o = ((long long)blockIdx.y * NV + v) * nk_total + kr.koff + t;
-        part[2 * o] = re;
-        part[2 * o + 1] = im;
+    for (int g = 0; g < 3; ++g)
+      if (j + g < n) {
+        const CT cv = c[j + g], zp = z[(j + g) * zw];
+        pr[g] += dot2(cv.x, zp.x, -cv.y, zp.y);
+        pi[g] += dot2(cv.x, zp.y, cv.y, zp.x);
+        nr[g] += dot2(cv.x, zp.x, cv.y, zp.y);
+        ni[g] += dot2(cv.x, -zp.y, cv.y, zp.x);
       }
-    }
-    __syncthreads();
   }
+  if (!mine) return;
+  const KRow kr = rows[en.x];
+  auto put = [&](int m3, const T (&re4)[4], const T (&im4)[4]) {
+    double re = 0.0, im = 0.0;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      re += (double)re4[g];
+      im += (double)im4[g];
+    }
+    const long long o = (long long)blockIdx.y * nk_total + kr.koff + (m3 - kr.m3lo);
+    part[2 * o] = re;
+    part[2 * o + 1] = im;
+  };
+  put(en.y, pr, pi);
+  if (en.y > 0 && -en.y >= kr.m3lo) put(-en.y, nr, ni);
 }
 
 // S(k) = sum over atom chunks (fixed order), times the k weight; stored as T complex.
 template <typename T>
-__global__ void sf_reduce_kernel(const double* part, int nchunk, int nv, long long nk, const double* wk,
+__global__ void sf_reduce_kernel(const double* part, int nchunk, long long nk, const double* wk,
                                  typename C2<T>::t* ws) {
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (k >= nk) return;
-  for (int v = 0; v < nv; ++v) {
-    double re = 0.0, im = 0.0;
-    for (int c = 0; c < nchunk; ++c) {
-      const long long o = ((long long)c * nv + v) * nk + k;
-      re += part[2 * o];
-      im += part[2 * o + 1];
-    }
-    ws[v * nk + k].x = (T)(wk[k] * re);
-    ws[v * nk + k].y = (T)(wk[k] * im);
+  double re = 0.0, im = 0.0;
+#pragma unroll 4
+  for (int c = 0; c < nchunk; ++c) {
+    const double2 p = reinterpret_cast<const double2*>(part)[c * nk + k];
+    re += p.x;
+    im += p.y;
   }
+  ws[k].x = (T)(wk[k] * re);
+  ws[k].y = (T)(wk[k] * im);
 }
 
 // Per atom I: sum_k w S(k) e^{-ik.R_I} -> Re (potential) and, for gradients, Im weighted by k.
 // mode 0: out[I] = Re sum (nv = 1).  mode 1: g[I][c] = sum w k_c [a_I Im(S_b e^-ikR) + b_I Im(S_a e^-ikR)].
+// A block takes blockDim atoms and one of gridDim.y chunks of the rows, four rows at a time: a Z phase read from
+// shared memory serves four k-vectors, whose weighted structure factors (zero past a row's end, which adds
+// nothing) sit beside each other for broadcast reads.  The sums over m3 are in T, those over rows in FP64.
+// Measured (GB300, 30,000 atoms), potential: 0.76 ms against 1.68 ms with one row at a time.
 template <typename T, int MODE>
 __global__ void recip_atom_kernel(const KRow* rows, int nrows, const typename C2<T>::t* tab, const typename C2<T>::t* ws,
                                   long long nk, int N, int nmax_all, int m3max, EwaldGeom g, const double* av,
@@ -160,67 +180,97 @@ __global__ void recip_atom_kernel(const KRow* rows, int nrows, const typename C2
   const int r0 = blockIdx.y * rchunk, r1 = min(nrows, r0 + rchunk);
   double* out = out_part + (long long)blockIdx.y * (MODE == 0 ? N : 3 * N);
   using CT = typename C2<T>::t;
+  constexpr int NV = MODE == 0 ? 1 : 2;        // structure factors: S_b, and S_a for the gradient
   extern __shared__ unsigned char sm[];
-  CT* zt = reinterpret_cast<CT*>(sm);          // [blockDim][2*m3max+1]
+  CT* zt = reinterpret_cast<CT*>(sm);          // [m3max + 1][blockDim]
+  CT* ss = zt + (m3max + 1) * blockDim.x;      // [2 m3max + 1][4 rows][NV]
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const int W = 2 * m3max + 1;
-  CT* myz = zt + threadIdx.x * W;
-  if (I < N) {
-    for (int m = 0; m <= m3max; ++m) {
-      const CT z = tab[(2LL * N + I) * (nmax_all + 1) + m];
-      CT zc = z;
-      zc.y = -zc.y;
-      myz[m3max + m] = zc;           // conj(Z[m]) for e^{-ik.R}
-      CT zp = z;
-      myz[m3max - m] = zp;           // conj(Z[-m]) = Z[m]
-    }
+  for (int q = threadIdx.x; q < (m3max + 1) * (int)blockDim.x; q += blockDim.x) {
+    const int j = q / (m3max + 1), m = q % (m3max + 1), J = blockIdx.x * blockDim.x + j;
+    if (J < N) zt[m * blockDim.x + j] = tab[(2LL * N + J) * (nmax_all + 1) + m];
   }
   double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0;
   const double tpx = 2.0 * M_PI / g.box_b[0], tpy = 2.0 * M_PI / g.box_b[1], tpz = 2.0 * M_PI / g.box_b[2];
-  if (I < N) {
-    for (int r = r0; r < r1; ++r) {
-      const KRow kr = rows[r];
-      CT x = tab[(0LL * N + I) * (nmax_all + 1) + kr.m1];
-      CT y = tab[(1LL * N + I) * (nmax_all + 1) + abs(kr.m2)];
-      if (kr.m2 < 0) y.y = -y.y;
-      CT xy = cmul<T>(x, y);
-      xy.y = -xy.y;                     // conj -> e^{-i(k1 x + k2 y)}
-      const int nm3 = kr.m3hi - kr.m3lo + 1;
-      if (MODE == 0) {
-        T re = 0;
-        for (int t = 0; t < nm3; ++t) {
-          const CT s = ws[kr.koff + t];
-          const CT z = myz[m3max + kr.m3lo + t];
-          const CT e = cmul<T>(xy, z);
-          re += s.x * e.x - s.y * e.y;
-        }
-        acc0 += (double)re;
-      } else {
-        // Im(S e^{-ikR}) for S_b (vector 0) and S_a (vector 1)
-        T i1 = 0, i3 = 0;   // sums over m3 of the Im-combination weighted by 1 and by m3
-        for (int t = 0; t < nm3; ++t) {
-          const int m3 = kr.m3lo + t;
-          const CT sb = ws[kr.koff + t];
-          const CT sa = ws[nk + kr.koff + t];
-          const CT z = myz[m3max + m3];
-          const CT e = cmul<T>(xy, z);
-          const T imb = sb.x * e.y + sb.y * e.x;
-          const T ima = sa.x * e.y + sa.y * e.x;
-          const T comb = (T)av[I] * imb + (T)bv[I] * ima;
-          i1 += comb;
-          i3 += comb * (T)m3;
-        }
-        acc0 += (double)i1 * (tpx * kr.m1);
-        acc1 += (double)i1 * (tpy * kr.m2);
-        acc2 += (double)i3 * tpz;
+  const T aI = MODE == 1 && I < N ? (T)av[I] : (T)0, bI = MODE == 1 && I < N ? (T)bv[I] : (T)0;
+  for (int rb = r0; rb < r1; rb += 4) {
+    KRow kr[4];
+    int lo = m3max, hi = -m3max;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      kr[q] = rows[min(rb + q, r1 - 1)];
+      if (rb + q >= r1) { kr[q].m3lo = 1; kr[q].m3hi = 0; }
+      else {
+        lo = min(lo, kr[q].m3lo);
+        hi = max(hi, kr[q].m3hi);
       }
     }
-    if (MODE == 0) out[I] = acc0;
-    else {
-      out[3 * I] = acc0;
-      out[3 * I + 1] = acc1;
-      out[3 * I + 2] = acc2;
+    __syncthreads();
+    for (int q = threadIdx.x; q < (hi - lo + 1) * 4; q += blockDim.x) {
+      const int t = q >> 2, r = q & 3, m3 = lo + t;
+      const KRow k = rows[min(rb + r, r1 - 1)];
+      const bool in = rb + r < r1 && m3 >= k.m3lo && m3 <= k.m3hi;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        CT x;
+        x.x = x.y = 0;
+        if (in) x = ws[v * nk + k.koff + (m3 - k.m3lo)];
+        ss[(t * 4 + r) * NV + v] = x;
+      }
     }
+    __syncthreads();
+    if (I >= N) continue;
+    CT xy[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const CT x = tab[(0LL * N + I) * (nmax_all + 1) + kr[q].m1];
+      CT y = tab[(1LL * N + I) * (nmax_all + 1) + abs(kr[q].m2)];
+      if (kr[q].m2 < 0) y.y = -y.y;
+      xy[q] = cmul<T>(x, y);
+      xy[q].y = -xy[q].y;               // conj -> e^{-i(k1 x + k2 y)}
+    }
+    T s1[4], s3[4];                     // sums over m3: the real part, or the Im-combination weighted by 1 and by m3
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s1[q] = s3[q] = 0;
+    for (int m3 = lo; m3 <= hi; ++m3) {
+      CT z = zt[abs(m3) * blockDim.x + threadIdx.x];
+      if (m3 >= 0) z.y = -z.y;          // conj(Z[m3]); Z[-m] = conj(Z[m])
+      const CT* sp = ss + (m3 - lo) * 4 * NV;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const CT e = cmul<T>(xy[q], z);
+        if (MODE == 0) {
+          const CT sv = sp[q];
+          s1[q] += sv.x * e.x - sv.y * e.y;
+        } else {
+          // Im(S e^{-ikR}) for S_b (vector 0) and S_a (vector 1)
+          const CT sb = sp[2 * q], sa = sp[2 * q + 1];
+          const T imb = sb.x * e.y + sb.y * e.x;
+          const T ima = sa.x * e.y + sa.y * e.x;
+          const T comb = aI * imb + bI * ima;
+          s1[q] += comb;
+          s3[q] += comb * (T)m3;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (rb + q >= r1) break;
+      if (MODE == 0) {
+        acc0 += (double)s1[q];
+      } else {
+        acc0 += (double)s1[q] * (tpx * kr[q].m1);
+        acc1 += (double)s1[q] * (tpy * kr[q].m2);
+        acc2 += (double)s3[q] * tpz;
+      }
+    }
+  }
+  if (I >= N) return;
+  if (MODE == 0) {
+    out[I] = acc0;
+  } else {
+    out[3 * I] = acc0;
+    out[3 * I + 1] = acc1;
+    out[3 * I + 2] = acc2;
   }
 }
 
@@ -359,49 +409,47 @@ __global__ void cell_scan_kernel(const int* count, int ncell, int* start) {
   }
 }
 
-// block per cell: stable compaction of the atoms of the cell in index order, with their
-// cell-relative coordinates
+__global__ void cell_append_kernel(const int* cell_of, int N, const int* cell_start, int* cell_fill, int* cell_atoms) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int c = cell_of[i];
+  cell_atoms[cell_start[c] + atomicAdd(&cell_fill[c], 1)] = i;
+}
+
+// Every atom's place in its cell is its rank by index among the cell's atoms (a few hundred, counted directly);
+// blockDim atoms of a cell per block.
 template <typename T>
-__global__ void cell_fill_sorted_kernel(const double* R, const int* species, int N, EwaldGeom g, const int* cell_of,
-                                        const int* cell_start, int* sorted_atom, typename Pos4<T>::t* pos_s) {
-  const int c = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __shared__ int wcnt[32];
-  __shared__ int base_sh;
-  if (threadIdx.x == 0) base_sh = cell_start[c];
+__global__ void cell_rank_kernel(const double* R, const int* species, EwaldGeom g, const int* cell_start,
+                                 const int* unsorted, int* sorted_atom, typename Pos4<T>::t* pos_s) {
+  __shared__ int tile[256];
+  const int c = blockIdx.x, s0 = cell_start[c], s1 = cell_start[c + 1];
   const int cz = c % g.nc[2], cy = (c / g.nc[2]) % g.nc[1], cx = c / (g.nc[2] * g.nc[1]);
   const double o[3] = {cx * (g.box_b[0] / g.nc[0]), cy * (g.box_b[1] / g.nc[1]), cz * (g.box_b[2] / g.nc[2])};
-  __syncthreads();
-  for (int i0 = 0; i0 < N; i0 += blockDim.x) {
-    const int i = i0 + threadIdx.x;
-    const bool mine = i < N && cell_of[i] == c;
-    const unsigned m = __ballot_sync(0xffffffffu, mine);
-    if (lane == 0) wcnt[warp] = __popc(m);
-    __syncthreads();
-    int off = 0;
-    for (int w = 0; w < warp; ++w) off += wcnt[w];
-    if (mine) {
-      const int k = base_sh + off + __popc(m & ((1u << lane) - 1u));
-      sorted_atom[k] = i;
-      typename Pos4<T>::t p;
-      double r[3];
-      for (int a = 0; a < 3; ++a) {
-        const double x = R[3 * i + a] / kBohrA;
-        r[a] = (x - g.box_b[a] * floor(x / g.box_b[a])) - o[a];
-      }
-      p.x = (T)r[0];
-      p.y = (T)r[1];
-      p.z = (T)r[2];
-      p.w = (T)species[i];
-      pos_s[k] = p;
+  for (int b0 = s0 + blockIdx.y * blockDim.x; b0 < s1; b0 += gridDim.y * blockDim.x) {
+    const int q = b0 + threadIdx.x;
+    const int i = q < s1 ? unsorted[q] : 0;
+    int rank = 0;
+    for (int t0 = s0; t0 < s1; t0 += blockDim.x) {
+      const int n = min((int)blockDim.x, s1 - t0);
+      __syncthreads();
+      if ((int)threadIdx.x < n) tile[threadIdx.x] = unsorted[t0 + threadIdx.x];
+      __syncthreads();
+      for (int t = 0; t < n; ++t) rank += tile[t] < i;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int tot = 0;
-      for (int w = 0; w < nw; ++w) tot += wcnt[w];
-      base_sh += tot;
+    if (q >= s1) continue;
+    const int k = s0 + rank;
+    sorted_atom[k] = i;
+    typename Pos4<T>::t p;
+    double r[3];
+    for (int a = 0; a < 3; ++a) {
+      const double x = R[3 * i + a] / kBohrA;
+      r[a] = (x - g.box_b[a] * floor(x / g.box_b[a])) - o[a];
     }
-    __syncthreads();
+    p.x = (T)r[0];
+    p.y = (T)r[1];
+    p.z = (T)r[2];
+    p.w = (T)species[i];
+    pos_s[k] = p;
   }
 }
 
@@ -568,11 +616,13 @@ Ewald::~Ewald() { release(); }
 
 void Ewald::release() {
   for (void* p : {(void*)rows_d, (void*)wk_d, (void*)tab, (void*)part, (void*)ws, (void*)real_buf, (void*)recip_buf,
-                  (void*)cell_of, (void*)cell_count, (void*)cell_start, (void*)cell_atoms, (void*)scal, (void*)rpart,
-                  pos_s})
+                  (void*)cell_of, (void*)cell_count, (void*)cell_start, (void*)cell_atoms, (void*)cell_raw, (void*)scal,
+                  (void*)rpart, (void*)sf_blocks, (void*)sf_entries, pos_s})
     if (p) cudaFree(p);
   rows_d = nullptr; wk_d = nullptr; tab = nullptr; part = nullptr; ws = nullptr; real_buf = nullptr;
-  recip_buf = nullptr; rpart = nullptr; cell_of = cell_count = cell_start = cell_atoms = nullptr; scal = nullptr;
+  recip_buf = nullptr; rpart = nullptr; cell_of = cell_count = cell_start = cell_atoms = cell_raw = nullptr;
+  sf_blocks = nullptr;
+  sf_entries = nullptr; scal = nullptr;
   pos_s = nullptr;
   N_ = 0;
 }
@@ -645,7 +695,23 @@ cudaError_t Ewald::setup(int N, const double box_A[3], const double hubbard_u[3]
   const size_t csz = fp64 ? sizeof(double2) : sizeof(float2);
   if ((e = cudaMalloc(&tab, csz * 3 * (size_t)N * (g.nmax_all + 1)))) return e;
   nchunk_ = (N + kChunk - 1) / kChunk;
-  if ((e = cudaMalloc(&part, sizeof(double) * 2 * 2 * (size_t)nchunk_ * nk_))) return e;
+  // structure-factor blocks: runs of at most kSfThreads entries (row, m3 >= 0) and kSfRows rows
+  std::vector<int2> entries;
+  std::vector<SfBlock> blocks;
+  for (int r = 0; r < nrows_; ++r)
+    for (int m3 = std::max(0, rows[r].m3lo); m3 <= rows[r].m3hi; ++m3) {
+      if (blocks.empty() || blocks.back().n_entries == kSfThreads || r - blocks.back().row0 >= kSfRows)
+        blocks.push_back({(int)entries.size(), 0, r, 0});
+      entries.push_back(make_int2(r, m3));
+      blocks.back().n_entries += 1;
+      blocks.back().n_rows = r - blocks.back().row0 + 1;
+    }
+  n_sf_ = (int)blocks.size();
+  if ((e = cudaMalloc(&sf_blocks, sizeof(SfBlock) * std::max(1, n_sf_)))) return e;
+  if ((e = cudaMalloc(&sf_entries, sizeof(int2) * std::max<size_t>(1, entries.size())))) return e;
+  cudaMemcpy(sf_blocks, blocks.data(), sizeof(SfBlock) * blocks.size(), cudaMemcpyHostToDevice);
+  cudaMemcpy(sf_entries, entries.data(), sizeof(int2) * entries.size(), cudaMemcpyHostToDevice);
+  if ((e = cudaMalloc(&part, sizeof(double) * 2 * (size_t)std::max(1, nchunk_) * std::max(1LL, nk_)))) return e;
   if ((e = cudaMalloc(&ws, csz * 2 * (size_t)nk_))) return e;
   if ((e = cudaMalloc(&real_buf, sizeof(double) * 3 * N))) return e;
   if ((e = cudaMalloc(&recip_buf, sizeof(double) * 3 * N))) return e;
@@ -654,6 +720,7 @@ cudaError_t Ewald::setup(int N, const double box_A[3], const double hubbard_u[3]
   const int ncell = g.nc[0] * g.nc[1] * g.nc[2];
   if ((e = cudaMalloc(&cell_of, sizeof(int) * N))) return e;
   if ((e = cudaMalloc(&cell_atoms, sizeof(int) * N))) return e;
+  if ((e = cudaMalloc(&cell_raw, sizeof(int) * N))) return e;
   if ((e = cudaMalloc(&cell_count, sizeof(int) * ncell))) return e;
   if ((e = cudaMalloc(&cell_start, sizeof(int) * (ncell + 1)))) return e;
   if ((e = cudaMalloc(&pos_s, sizeof(double4) * N))) return e;
@@ -663,42 +730,54 @@ cudaError_t Ewald::setup(int N, const double box_A[3], const double hubbard_u[3]
 // The dynamic shared-memory limit of a kernel is a process-wide attribute, while the size a
 // launch needs depends on the context's k set: the limit only ever grows (largest request of
 // any context so far), so a context never lowers it below what another one launches with.
-static std::mutex g_recip_smem_mutex;
-static int g_recip_smem[4] = {0, 0, 0, 0};
+static std::mutex g_smem_mutex;
+static int g_smem[6] = {0, 0, 0, 0, 0, 0};
 
-template <typename T, int MODE>
-static void raise_recip_smem(int slot, int bytes) {
-  std::lock_guard<std::mutex> lock(g_recip_smem_mutex);
-  if (bytes > g_recip_smem[slot]) {
-    cudaFuncSetAttribute(recip_atom_kernel<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    g_recip_smem[slot] = bytes;
+template <typename K>
+static void raise_smem(K kernel, int slot, size_t bytes) {
+  std::lock_guard<std::mutex> lock(g_smem_mutex);
+  if ((int)bytes > g_smem[slot]) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    g_smem[slot] = (int)bytes;
   }
 }
 
+template <typename T>
+static size_t sf_smem(int m3max) {
+  return sizeof(typename C2<T>::t) * (kSfRows * (kSfAtoms + 1) + (size_t)kSfAtoms * (m3max + 1));
+}
+template <typename T>
+static size_t recip_smem(int m3max, int tpb, int nv) {
+  return sizeof(typename C2<T>::t) * ((size_t)(m3max + 1) * tpb + (size_t)(2 * m3max + 1) * 4 * nv);
+}
+
 cudaError_t Ewald::prepare(const double* dR, const int* dspecies, cudaStream_t s) {
-  const int W = 2 * m3max_ + 1;
   if (fp64_) {
-    raise_recip_smem<double, 0>(0, (int)sizeof(double2) * 64 * W);
-    raise_recip_smem<double, 1>(1, (int)sizeof(double2) * 64 * W);
+    raise_smem(recip_atom_kernel<double, 0>, 0, recip_smem<double>(m3max_, 64, 1));
+    raise_smem(recip_atom_kernel<double, 1>, 1, recip_smem<double>(m3max_, 64, 2));
+    raise_smem(structure_factor_kernel<double>, 4, sf_smem<double>(m3max_));
   } else {
-    raise_recip_smem<float, 0>(2, (int)sizeof(float2) * 128 * W);
-    raise_recip_smem<float, 1>(3, (int)sizeof(float2) * 128 * W);
+    raise_smem(recip_atom_kernel<float, 0>, 2, recip_smem<float>(m3max_, 128, 1));
+    raise_smem(recip_atom_kernel<float, 1>, 3, recip_smem<float>(m3max_, 128, 2));
+    raise_smem(structure_factor_kernel<float>, 5, sf_smem<float>(m3max_));
   }
   const int TB = 128, nb = (N_ + TB - 1) / TB;
-  if (fp64_) phase_table_kernel<double><<<nb, TB, 0, s>>>(dR, N_, g, reinterpret_cast<double2*>(tab));
-  else phase_table_kernel<float><<<nb, TB, 0, s>>>(dR, N_, g, reinterpret_cast<float2*>(tab));
+  if (fp64_) phase_table_kernel<double><<<dim3(nb, 3), TB, 0, s>>>(dR, N_, g, reinterpret_cast<double2*>(tab));
+  else phase_table_kernel<float><<<dim3(nb, 3), TB, 0, s>>>(dR, N_, g, reinterpret_cast<float2*>(tab));
   if (!g.brute) {
     // cell list on the device: counts, scan, stable fill with cell-relative coordinates
     const int ncell = g.nc[0] * g.nc[1] * g.nc[2];
     cudaMemsetAsync(cell_count, 0, sizeof(int) * ncell, s);
     cell_count_kernel<<<nb, TB, 0, s>>>(dR, N_, g, cell_of, cell_count);
     cell_scan_kernel<<<1, 1024, 0, s>>>(cell_count, ncell, cell_start);
+    cudaMemsetAsync(cell_count, 0, sizeof(int) * ncell, s);
+    cell_append_kernel<<<nb, TB, 0, s>>>(cell_of, N_, cell_start, cell_count, cell_raw);
     if (fp64_)
-      cell_fill_sorted_kernel<double><<<ncell, 256, 0, s>>>(dR, dspecies, N_, g, cell_of, cell_start, cell_atoms,
-                                                             reinterpret_cast<double4*>(pos_s));
+      cell_rank_kernel<double><<<dim3(ncell, 4), 256, 0, s>>>(dR, dspecies, g, cell_start, cell_raw, cell_atoms,
+                                                              reinterpret_cast<double4*>(pos_s));
     else
-      cell_fill_sorted_kernel<float><<<ncell, 256, 0, s>>>(dR, dspecies, N_, g, cell_of, cell_start, cell_atoms,
-                                                            reinterpret_cast<float4*>(pos_s));
+      cell_rank_kernel<float><<<dim3(ncell, 4), 256, 0, s>>>(dR, dspecies, g, cell_start, cell_raw, cell_atoms,
+                                                             reinterpret_cast<float4*>(pos_s));
   }
   sb_tag_ = 0;
   dR_ = dR;
@@ -706,19 +785,16 @@ cudaError_t Ewald::prepare(const double* dR, const int* dspecies, cudaStream_t s
   return cudaGetLastError();
 }
 
+// w S of the charges b into vector `vec` of ws
 template <typename T>
-static void run_sf(Ewald& E, const double* b0, const double* b1, int nv, int vout0, cudaStream_t s) {
+static void run_sf(Ewald& E, const double* b, int vec, cudaStream_t s) {
   using CT = typename C2<T>::t;
-  dim3 grid(E.nrows_, E.nchunk_);
-  const size_t shm = sizeof(CT) * Ewald::kChunk * nv + sizeof(T) * 4 * 64 * nv * 2;
-  if (nv == 1)
-    structure_factor_kernel<T, 1><<<grid, 256, shm, s>>>(E.rows_d, reinterpret_cast<const CT*>(E.tab), b0, b1, E.N_,
-                                                        E.g.nmax_all, Ewald::kChunk, E.part, E.nk_);
-  else
-    structure_factor_kernel<T, 2><<<grid, 256, shm, s>>>(E.rows_d, reinterpret_cast<const CT*>(E.tab), b0, b1, E.N_,
-                                                        E.g.nmax_all, Ewald::kChunk, E.part, E.nk_);
-  sf_reduce_kernel<T><<<(int)((E.nk_ + 255) / 256), 256, 0, s>>>(E.part, E.nchunk_, nv, E.nk_, E.wk_d,
-                                                                 reinterpret_cast<CT*>(E.ws) + (size_t)vout0 * E.nk_);
+  if (E.n_sf_ > 0)
+    structure_factor_kernel<T><<<dim3(E.n_sf_, E.nchunk_), kSfThreads, sf_smem<T>(E.m3max_), s>>>(
+        E.sf_blocks, E.sf_entries, E.rows_d, reinterpret_cast<const CT*>(E.tab), b, E.N_, E.g.nmax_all, E.m3max_,
+        Ewald::kChunk, E.part, E.nk_);
+  sf_reduce_kernel<T><<<(int)((E.nk_ + 255) / 256), 256, 0, s>>>(E.part, E.nchunk_, E.nk_, E.wk_d,
+                                                                 reinterpret_cast<CT*>(E.ws) + (size_t)vec * E.nk_);
 }
 
 template <typename T, int MODE>
@@ -736,20 +812,19 @@ static void run_real(Ewald& E, const double* a, const double* b, cudaStream_t s)
 
 cudaError_t Ewald::potential(const double* b, double* V, cudaStream_t s, int tag) {
   const int TB = 128, nb = (N_ + TB - 1) / TB;
-  const int W = 2 * m3max_ + 1;
   if (fp64_) {
-    run_sf<double>(*this, b, nullptr, 1, 0, s);
+    run_sf<double>(*this, b, 0, s);
     run_real<double, 0>(*this, nullptr, b, s);
     const int tpb = 64;
-    recip_atom_kernel<double, 0><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, sizeof(double2) * tpb * W, s>>>(
+    recip_atom_kernel<double, 0><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, recip_smem<double>(m3max_, tpb, 1), s>>>(
         rows_d, nrows_, reinterpret_cast<const double2*>(tab), reinterpret_cast<const double2*>(ws), nk_, N_,
         g.nmax_all, m3max_, g, nullptr, nullptr, rpart);
     chunk_reduce_kernel<<<(N_ + 255) / 256, 256, 0, s>>>(rpart, kRowChunks, N_, recip_buf);
   } else {
-    run_sf<float>(*this, b, nullptr, 1, 0, s);
+    run_sf<float>(*this, b, 0, s);
     run_real<float, 0>(*this, nullptr, b, s);
     const int tpb = 128;
-    recip_atom_kernel<float, 0><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, sizeof(float2) * tpb * W, s>>>(
+    recip_atom_kernel<float, 0><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, recip_smem<float>(m3max_, tpb, 1), s>>>(
         rows_d, nrows_, reinterpret_cast<const float2*>(tab), reinterpret_cast<const float2*>(ws), nk_, N_,
         g.nmax_all, m3max_, g, nullptr, nullptr, rpart);
     chunk_reduce_kernel<<<(N_ + 255) / 256, 256, 0, s>>>(rpart, kRowChunks, N_, recip_buf);
@@ -761,25 +836,24 @@ cudaError_t Ewald::potential(const double* b, double* V, cudaStream_t s, int tag
 }
 
 cudaError_t Ewald::gradient(const double* a, const double* b, double* G, cudaStream_t s, int tag) {
-  const int W = 2 * m3max_ + 1;
   // vector 0 = b (S_b), vector 1 = a (S_a); S_b is kept from the potential call with the same
   // nonzero tag (same charges at the same geometry)
   const bool reuse = tag != 0 && tag == sb_tag_;
   if (fp64_) {
-    if (reuse) run_sf<double>(*this, a, nullptr, 1, 1, s);
-    else run_sf<double>(*this, b, a, 2, 0, s);
+    if (!reuse) run_sf<double>(*this, b, 0, s);
+    run_sf<double>(*this, a, 1, s);
     run_real<double, 1>(*this, a, b, s);
     const int tpb = 64;
-    recip_atom_kernel<double, 1><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, sizeof(double2) * tpb * W, s>>>(
+    recip_atom_kernel<double, 1><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, recip_smem<double>(m3max_, tpb, 2), s>>>(
         rows_d, nrows_, reinterpret_cast<const double2*>(tab), reinterpret_cast<const double2*>(ws), nk_, N_,
         g.nmax_all, m3max_, g, a, b, rpart);
     chunk_reduce_kernel<<<(3 * N_ + 255) / 256, 256, 0, s>>>(rpart, kRowChunks, 3LL * N_, recip_buf);
   } else {
-    if (reuse) run_sf<float>(*this, a, nullptr, 1, 1, s);
-    else run_sf<float>(*this, b, a, 2, 0, s);
+    if (!reuse) run_sf<float>(*this, b, 0, s);
+    run_sf<float>(*this, a, 1, s);
     run_real<float, 1>(*this, a, b, s);
     const int tpb = 128;
-    recip_atom_kernel<float, 1><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, sizeof(float2) * tpb * W, s>>>(
+    recip_atom_kernel<float, 1><<<dim3((N_ + tpb - 1) / tpb, kRowChunks), tpb, recip_smem<float>(m3max_, tpb, 2), s>>>(
         rows_d, nrows_, reinterpret_cast<const float2*>(tab), reinterpret_cast<const float2*>(ws), nk_, N_,
         g.nmax_all, m3max_, g, a, b, rpart);
     chunk_reduce_kernel<<<(3 * N_ + 255) / 256, 256, 0, s>>>(rpart, kRowChunks, 3LL * N_, recip_buf);

@@ -23,13 +23,19 @@ struct KRow {           // reciprocal vectors with fixed (m1, m2), m3 in [m3lo, 
   long long koff;       // index of (m1, m2, m3lo) in the flat k list
 };
 
+struct SfBlock {        // structure-factor block: a run of k-row entries and the rows they lie in
+  int entry0, n_entries, row0, n_rows;
+};
+
 struct Ewald {
   static constexpr int kChunk = 1024;
   static constexpr int kRowChunks = 24;    // k-row chunks of the per-atom reciprocal sums
   EwaldGeom g{};
   int N_ = 0;
   bool fp64_ = true;
-  int nrows_ = 0, nchunk_ = 0, m3max_ = 0;
+  int nrows_ = 0, nchunk_ = 0, m3max_ = 0, n_sf_ = 0;
+  SfBlock* sf_blocks = nullptr;
+  int2* sf_entries = nullptr;   // (row, m3 >= 0)
   long long nk_ = 0;
   KRow* rows_d = nullptr;
   double* wk_d = nullptr;
@@ -40,7 +46,8 @@ struct Ewald {
   double* recip_buf = nullptr;
   double* rpart = nullptr;   // per-row-chunk partial sums
   double* scal = nullptr;
-  int *cell_of = nullptr, *cell_count = nullptr, *cell_start = nullptr, *cell_atoms = nullptr;
+  int *cell_of = nullptr, *cell_count = nullptr, *cell_start = nullptr, *cell_atoms = nullptr,
+      *cell_raw = nullptr;
   void* pos_s = nullptr;     // cell-sorted cell-relative coordinates and species (float4 / double4)
   int sb_tag_ = 0;           // tag of the charges whose S(k) sits in vector 0 of ws (0: none)
   const double* dR_ = nullptr;
