@@ -23,7 +23,7 @@ struct KRow {           // reciprocal vectors with fixed (m1, m2), m3 in [m3lo, 
   long long koff;       // index of (m1, m2, m3lo) in the flat k list
 };
 
-struct SfBlock {        // structure-factor block: a run of k-row entries and the rows they lie in
+struct SfBlock {        // structure-factor block: a run of entries and the rows they lie in
   int entry0, n_entries, row0, n_rows;
 };
 
@@ -33,9 +33,9 @@ struct Ewald {
   EwaldGeom g{};
   int N_ = 0;
   bool fp64_ = true;
-  int nrows_ = 0, nchunk_ = 0, m3max_ = 0, n_sf_ = 0;
+  int nrows_ = 0, nchunk_ = 0, m3max_ = 0, n_sf_ = 0, sf_rows_ = 0;
   SfBlock* sf_blocks = nullptr;
-  int2* sf_entries = nullptr;   // (row, m3 >= 0)
+  int2* sf_entries = nullptr;   // (first of two rows, m3 >= 0)
   long long nk_ = 0;
   KRow* rows_d = nullptr;
   double* wk_d = nullptr;
