@@ -1092,15 +1092,21 @@ void back_transform(sedacs_ctx* ctx, bool with_w) {
   }
 }
 
+// Populations of the core rows at dc_off.
+void launch_populations(sedacs_ctx* ctx, const long long* dc_off, double* pop) {
+  launch_observables(ctx->model, ctx->d_R, ctx->d_species, sk_geom(ctx), ctx->d_core_tab, ctx->n_core_total, ctx->d_pptr,
+                     ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, ctx->arena, dc_off,
+                     dc_off, pop, nullptr, ctx->d_dU, false, ctx->f64, ctx->stream);
+}
+
 // Populations / band energy (and forces) from the core rows; q = pop - Z; returns N_e count.
 sedacs_status observe(sedacs_ctx* ctx, bool with_forces, double* n_count) {
   cudaStream_t s = ctx->stream;
   const SkGeom g = sk_geom(ctx);
   if (with_forces) cudaMemsetAsync(ctx->d_dU, 0, sizeof(double) * 3 * ctx->N, s);
-  launch_observables(ctx->model, ctx->d_R, ctx->d_species, g, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off,
-                     ctx->part.perm, ctx->d_core_sub, ctx->d_core_local, ctx->n_core_total, ctx->d_pptr, ctx->d_pcol,
-                     ctx->d_h0b, ctx->d_sb, ctx->d_loc, ctx->N, ctx->d_V, ctx->arena, ctx->arena, ctx->d_dcoff,
-                     ctx->d_wcoff, ctx->d_n_pad, ctx->d_pop, ctx->d_eband, ctx->d_dU, with_forces ? 1 : 0, ctx->f64, s);
+  launch_observables(ctx->model, ctx->d_R, ctx->d_species, g, ctx->d_core_tab, ctx->n_core_total, ctx->d_pptr,
+                     ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, ctx->arena,
+                     ctx->d_dcoff, ctx->d_wcoff, ctx->d_pop, ctx->d_eband, ctx->d_dU, with_forces, ctx->f64, s);
   charges_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_pop, ctx->d_species, ctx->d_zval, ctx->d_q, ctx->N);
   dot_kernel<<<1, 1024, 0, s>>>(ctx->d_pop, nullptr, ctx->N, ctx->d_scal);
   ctx->launches += 3;
@@ -1473,13 +1479,10 @@ sedacs_status fermi_reentry(sedacs_ctx* ctx, double mu) {
 }
 
 // Populations of the core rows at dc_off (per atom, the FP64 sum over each core atom's orbitals
-// and its subgraph) into pop, band-energy partials into eb, and their sum into d_scal[k].
-void core_pops(sedacs_ctx* ctx, const long long* dc_off, double* pop, double* eb, int k) {
+// and its subgraph) into pop, their sum into d_scal[k].
+void core_pops(sedacs_ctx* ctx, const long long* dc_off, double* pop, int k) {
   cudaStream_t s = ctx->stream;
-  launch_observables(ctx->model, ctx->d_R, ctx->d_species, sk_geom(ctx), ctx->d_sub_ptr, ctx->d_sub_atoms,
-                     ctx->d_orb_off, ctx->part.perm, ctx->d_core_sub, ctx->d_core_local, ctx->n_core_total,
-                     ctx->d_pptr, ctx->d_pcol, ctx->d_h0b, ctx->d_sb, ctx->d_loc, ctx->N, ctx->d_V, ctx->arena,
-                     ctx->arena, dc_off, dc_off, ctx->d_n_pad, pop, eb, ctx->d_dU, 0, ctx->f64, s);
+  launch_populations(ctx, dc_off, pop);
   dot_kernel<<<1, 1024, 0, s>>>(pop, nullptr, ctx->N, ctx->d_scal + k);
   ctx->launches += 2;
 }
@@ -1574,7 +1577,6 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
   double dmu = 0.0, np = 0.0;
   int order = 2;                               // terms of the accepted mu expansion
   double* pop_s = ctx->d_rsp + 6LL * N;      // kept for the response calls (their dN/dmu weights)
-  double* scr = ctx->d_rsp + 7LL * N;
   double* pop_t = ctx->d_rsp + 5LL * N;
   double* pop_uw = ctx->d_rsp + 8LL * N;
   int pass = 0;
@@ -1594,11 +1596,11 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
     }
     back_transform(ctx, false);                                   // T1 = Z_c F, D_c
     if (given) { done = true; break; }
-    core_pops(ctx, ctx->d_dcoff, ctx->d_pop, ctx->d_eband, 9);     // N(mu)
+    core_pops(ctx, ctx->d_dcoff, ctx->d_pop, 9);                   // N(mu)
     STCHK(fermi_s_rows(ctx));
-    core_pops(ctx, ctx->d_dcoff_d, pop_s, scr, 10);                // sum of D_s populations
+    core_pops(ctx, ctx->d_dcoff_d, pop_s, 10);                     // sum of D_s populations
     fermi_t_rows(ctx);
-    core_pops(ctx, ctx->d_dcoff_t, pop_t, scr, 14);                // sum of D_t populations
+    core_pops(ctx, ctx->d_dcoff_t, pop_t, 14);                     // sum of D_t populations
     double sc[6];
     CUCHK(cudaMemcpyAsync(sc, ctx->d_scal + 9, sizeof(sc), cudaMemcpyDeviceToHost, s));
     CUCHK(cudaStreamSynchronize(s));
@@ -1636,8 +1638,8 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
       if (std::fabs(beta * d2) <= lin2) { dmu = d2; order = 2; done = true; break; }
       if (std::fabs(beta * d2) <= 1.5 * lin) {
         fermi_uw_rows(ctx);
-        core_pops(ctx, ctx->d_dcoff_u, pop_uw, scr, 11);           // sums of D_u and D_w populations
-        core_pops(ctx, ctx->d_dcoff_w, pop_uw, scr, 12);
+        core_pops(ctx, ctx->d_dcoff_u, pop_uw, 11);                // sums of D_u and D_w populations
+        core_pops(ctx, ctx->d_dcoff_w, pop_uw, 12);
         double s34[2];
         CUCHK(cudaMemcpyAsync(s34, ctx->d_scal + 11, sizeof(s34), cudaMemcpyDeviceToHost, s));
         CUCHK(cudaStreamSynchronize(s));
@@ -1715,7 +1717,15 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
   gather_hs(ctx);
   phase_end(ctx, 0, 2);
   phase_begin(ctx, 0);
-  if (!ctx->z_valid) compute_z(ctx);
+  if (!ctx->z_valid) {                  // new pairs or subgraphs
+    CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_tab), sizeof(int4) * std::max(1, ctx->n_core_total)));
+    CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_pair_orb), sizeof(int) * std::max(1LL, ctx->pnnz)));
+    launch_pair_orbs(ctx->model, ctx->d_species, ctx->d_sub_ptr, ctx->d_orb_off, ctx->part.perm, ctx->d_core_sub,
+                     ctx->d_core_local, ctx->n_core_total, ctx->d_pptr, ctx->d_pcol, ctx->d_loc, ctx->N, ctx->d_n_pad,
+                     ctx->d_core_tab, ctx->d_pair_orb, s);
+    ctx->launches += 1;
+    compute_z(ctx);
+  }
   compute_ht(ctx);                      // h's planes were written by gather_hs
   CUCHK(cudaStreamSynchronize(s));
   ctx->ht_stale = false;
@@ -1877,11 +1887,7 @@ sedacs_status response_sp2(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
   }
   run_op(ctx, ctx->zc == 0 ? OP_DT1_0 : OP_DT1_1, n2 > ns ? n2 : ns, ns);   // dT1 = Z_c dX
   run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);                     // dD_c = 2 dT1 Z
-  launch_observables(ctx->model, ctx->d_R, ctx->d_species, sk_geom(ctx), ctx->d_sub_ptr, ctx->d_sub_atoms,
-                     ctx->d_orb_off, ctx->part.perm, ctx->d_core_sub, ctx->d_core_local, ctx->n_core_total,
-                     ctx->d_pptr, ctx->d_pcol, ctx->d_h0b, ctx->d_sb, ctx->d_loc, ctx->N, ctx->d_tmp, ctx->arena,
-                     ctx->arena, ctx->d_dcoff_d, ctx->d_dcoff_d, ctx->d_n_pad, d_dq, ctx->d_tmp2, ctx->d_dU, 0,
-                     ctx->f64, s);
+  launch_populations(ctx, ctx->d_dcoff_d, d_dq);
   ctx->launches += 1;
   return check_dev_err(ctx);
 }
@@ -1903,7 +1909,6 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
   double* qp = ctx->d_rsp + 2LL * N;
   double* qm = ctx->d_rsp + 3LL * N;
   double* ps = ctx->d_rsp + 4LL * N;
-  double* eb = ctx->d_rsp + 5LL * N;
   absmax_kernel<<<1, 1024, 0, s>>>(d_v, N, ctx->d_scal + 11);
   ctx->launches += 1;
   const double vmax = host_scalar(ctx, ctx->d_scal + 11);
@@ -1942,9 +1947,9 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
     STCHK(run_fermi(ctx, ctx->mu, nd));
     run_op(ctx, ctx->zc == 0 ? OP_F_FT1_0 : OP_F_FT1_1, 3, ns);   // dT1 = Z_c F
     run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);         // 2 dT1 Z
-    core_pops(ctx, ctx->d_dcoff_d, q, eb, 9);
+    core_pops(ctx, ctx->d_dcoff_d, q, 9);
     STCHK(fermi_s_rows(ctx));
-    core_pops(ctx, ctx->d_dcoff_d, ps, eb, 10);
+    core_pops(ctx, ctx->d_dcoff_d, ps, 10);
     double sc[2];
     CUCHK(cudaMemcpyAsync(sc, ctx->d_scal + 9, sizeof(sc), cudaMemcpyDeviceToHost, s));
     CUCHK(cudaStreamSynchronize(s));
@@ -2199,9 +2204,9 @@ void sedacs_destroy(sedacs_ctx* ctx) {
                   ctx->d_mass, ctx->d_zval, ctx->d_vec, ctx->d_row_ptr, ctx->d_col, ctx->d_pptr, ctx->d_pcol,
                   ctx->d_h0b, ctx->d_sb, ctx->d_gd_ptr, ctx->d_gd_col, ctx->d_gd_val, ctx->d_xgd_ptr, ctx->d_xgd_col,
                   ctx->d_xgd_val, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_n_orb, ctx->d_sub_of_row,
-                  ctx->d_core_sub, ctx->d_core_local, ctx->d_loc, ctx->d_gd_len, ctx->d_tables, ctx->arena,
-                  ctx->d_glo, ctx->d_ghi, ctx->d_bounds, ctx->d_slots, ctx->d_sp2, ctx->d_nactive, ctx->d_dqpop,
-                  ctx->d_steps, ctx->d_rsp, ctx->d_cdone};
+                  ctx->d_core_sub, ctx->d_core_local, ctx->d_core_tab, ctx->d_pair_orb, ctx->d_loc, ctx->d_gd_len,
+                  ctx->d_tables, ctx->arena, ctx->d_glo, ctx->d_ghi, ctx->d_bounds, ctx->d_slots, ctx->d_sp2,
+                  ctx->d_nactive, ctx->d_dqpop, ctx->d_steps, ctx->d_rsp, ctx->d_cdone};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto& e : ctx->ev)

@@ -242,60 +242,91 @@ __global__ void gather_kernel(const ModelDev m, const long long* sub_ptr, const 
   }
 }
 
-// Collected observables, one warp per core atom (lanes split its neighbour list; sums are
-// combined by a fixed shuffle tree, the reaction on B by FP64 atomics).
-template <typename T>
-__global__ void observables_kernel(const ModelDev m, const double* R, const int* species, SkGeom g,
-                                   const long long* sub_ptr, const int* sub_atoms, const int* orb_off,
-                                   const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
-                                   const long long* pptr, const int* pcol, const T* h0b, const T* sb, const int* loc,
-                                   int N, const double* V, const float* Dc32, const double* Dc64, const float* Wc32,
-                                   const double* Wc64, const long long* dc_off, const long long* wc_off, const int* n_pad,
-                                   double* pop, double* eband, double* dU, int with_forces) {
+// Tables of the passes over core rows: per core atom {atom, subgraph, 8 x first orbital + orbitals, row length},
+// per pair of its list 8 x first orbital + orbitals of the neighbour in the atom's subgraph (-1: not in it).
+// Warp per core atom.
+__global__ void pair_orbs_kernel(const ModelDev m, const int* species, const long long* sub_ptr, const int* orb_off,
+                                 const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
+                                 const long long* pptr, const int* pcol, const int* loc, int N, const int* n_pad,
+                                 int4* core_tab, int* pair_orb) {
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= n_core_total) return;
-  const int A = core_list[t], i = core_sub[t], a = core_local[t];
-  const long long qa = sub_ptr[i] + a;
-  const int sa = species[A], na = m.n_orb[sa], oa = orb_off[qa];
-  const int ld = n_pad[i];
-  const long long base = dc_off[i] / (Dc64 ? 8 : 4);   // element offset of the core rows
-  const long long wbase = wc_off[i] / (Wc64 ? 8 : 4);
-  auto Dv = [&](int r, int c) -> double {
-    const long long k = base + (long long)r * ld + c;
-    return Dc64 ? Dc64[k] : (double)Dc32[k];
-  };
-  auto Wv = [&](int r, int c) -> double {
-    const long long k = wbase + (long long)r * ld + c;
-    return Wc64 ? Wc64[k] : (double)Wc32[k];
-  };
+  const int A = core_list[t], i = core_sub[t];
+  const long long q0 = sub_ptr[i];
+  if (lane == 0)
+    core_tab[t] = make_int4(A, i, orb_off[q0 + core_local[t]] * 8 + m.n_orb[species[A]], n_pad[i]);
   const int* L = loc + (long long)i * N;
+  for (long long p = pptr[A] + lane; p < pptr[A + 1]; p += 32) {
+    const int B = pcol[p], b = L[B];
+    pair_orb[p] = b < 0 ? -1 : orb_off[q0 + b] * 8 + m.n_orb[species[B]];
+  }
+}
+
+template <typename T> struct __align__(16) Row4 { T v[4]; };
+
+// Collected observables, one warp per core atom (lanes split its neighbour list; sums are
+// combined by a fixed shuffle tree, the reaction on B by FP64 atomics).  Populations alone (FORCES false, the form
+// the chemical potential's passes use four to eight times a density; eband may be null) are bound by the FP64
+// additions and by the latency of the gathers, which the tables of pair_orbs_kernel cut from six to three levels;
+// without the force blocks' registers twice the warps fit.  Measured (GB300, 9,000 atoms): 82 us, 160 us with
+// one kernel for both that looked up every pair; with forces 267 us, 306 us.
+template <typename T, bool FORCES>
+__global__ void __launch_bounds__(128) observables_kernel(const ModelDev m, const double* R, const int* species,
+                                                          SkGeom g, const int4* core_tab, int n_core_total,
+                                                          const long long* pptr, const int* pcol, const int* pair_orb,
+                                                          const T* h0b, const T* sb, const double* V,
+                                                          const uint8_t* dc, const uint8_t* wc, const long long* dc_off,
+                                                          const long long* wc_off, double* pop, double* eband,
+                                                          double* dU) {
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (t >= n_core_total) return;
+  const int4 ct = core_tab[t];
+  const int A = ct.x, na = ct.z & 7, oa = ct.z >> 3, ld = ct.w;
+  const T* D = reinterpret_cast<const T*>(dc + dc_off[ct.y]) + (long long)oa * ld;   // the core atom's rows
+  const T* W = FORCES ? reinterpret_cast<const T*>(wc + wc_off[ct.y]) + (long long)oa * ld : nullptr;
+  const bool band = FORCES || eband != nullptr;
+  const int sa = species[A];
   double p_acc = 0.0, e_acc = 0.0;
   double fa[3] = {0.0, 0.0, 0.0};
   if (lane == 0)
     for (int u = 0; u < na; ++u) {      // on-site block
-      const double d = Dv(oa + u, oa + u);
+      const double d = D[(long long)u * ld + oa + u];
       p_acc += d;
       e_acc += d * (u == 0 ? m.eps_s[sa] : m.eps_p[sa]);
     }
-  const double va = V[A];
+  const double va = FORCES ? V[A] : 0.0;
   const double roff2 = m.r_off * m.r_off;
   for (long long p = pptr[A] + lane; p < pptr[A + 1]; p += 32) {
-    const int B = pcol[p];
-    const int b = L[B];
-    if (b < 0) continue;
-    const int ob = orb_off[sub_ptr[i] + b];
-    const int sbp = species[B], nb = m.n_orb[sbp];
-    T Dm[4][4] = {}, Wm[4][4] = {};
-    for (int u = 0; u < na; ++u)
-      for (int v = 0; v < nb; ++v) {
-        const double d = Dv(oa + u, ob + v);
-        Dm[u][v] = (T)d;
-        if (with_forces) Wm[u][v] = (T)Wv(oa + u, ob + v);
-        p_acc += d * (double)sb[p * 16 + u * 4 + v];
-        e_acc += d * (double)h0b[p * 16 + u * 4 + v];
+    const int po = pair_orb[p];
+    if (po < 0) continue;
+    const int nb = po & 7, ob = po >> 3;
+    T Dm[4][4], Wm[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const bool in = u < na && v < nb;
+        Dm[u][v] = in ? D[(long long)u * ld + ob + v] : (T)0;
+        if (FORCES) Wm[u][v] = in ? W[(long long)u * ld + ob + v] : (T)0;
       }
-    if (!with_forces) continue;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (u >= na) break;
+      const Row4<T> sr = reinterpret_cast<const Row4<T>*>(sb + p * 16)[u];
+      Row4<T> hr{};
+      if (band) hr = reinterpret_cast<const Row4<T>*>(h0b + p * 16)[u];
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        if (v < nb) {
+          const double d = Dm[u][v];
+          p_acc += d * (double)sr.v[v];
+          if (band) e_acc += d * (double)hr.v[v];
+        }
+    }
+    if (!FORCES) continue;
+    const int B = pcol[p], sbp = species[B];
     const T vab = (T)(0.5 * (va + V[B]));
     T Ms[4][4];
 #pragma unroll
@@ -325,13 +356,13 @@ __global__ void observables_kernel(const ModelDev m, const double* R, const int*
     }
   }
   p_acc = warp_sum(p_acc);
-  e_acc = warp_sum(e_acc);
-  if (with_forces)
+  if (band) e_acc = warp_sum(e_acc);
+  if (FORCES)
     for (int c = 0; c < 3; ++c) fa[c] = warp_sum(fa[c]);
   if (lane == 0) {
     pop[A] = p_acc;
-    eband[A] = e_acc;
-    if (with_forces)
+    if (band) eband[A] = e_acc;
+    if (FORCES)
       for (int c = 0; c < 3; ++c) atomicAdd(&dU[3 * A + c], fa[c]);
   }
 }
@@ -455,24 +486,30 @@ void launch_gather(const ModelDev& m, const long long* sub_ptr, const int* sub_a
                                            total_rows, shift_only);
 }
 
-void launch_observables(const ModelDev& m, const double* R, const int* species, const SkGeom& g,
-                        const long long* sub_ptr, const int* sub_atoms, const int* orb_off, const int* core_list,
-                        const int* core_sub, const int* core_local, int n_core_total, const long long* pptr,
-                        const int* pcol, const void* h0b, const void* sb, const int* loc, int N, const double* V,
-                        const void* Dc, const void* Wc, const long long* dc_off, const long long* wc_off,
-                        const int* n_pad, double* pop, double* eband, double* dU, int with_forces, bool f64,
+void launch_pair_orbs(const ModelDev& m, const int* species, const long long* sub_ptr, const int* orb_off,
+                      const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
+                      const long long* pptr, const int* pcol, const int* loc, int N, const int* n_pad, int4* core_tab,
+                      int* pair_orb, cudaStream_t s) {
+  pair_orbs_kernel<<<(int)((32LL * n_core_total + 127) / 128), 128, 0, s>>>(
+      m, species, sub_ptr, orb_off, core_list, core_sub, core_local, n_core_total, pptr, pcol, loc, N, n_pad, core_tab,
+      pair_orb);
+}
+
+void launch_observables(const ModelDev& m, const double* R, const int* species, const SkGeom& g, const int4* core_tab,
+                        int n_core_total, const long long* pptr, const int* pcol, const int* pair_orb, const void* h0b,
+                        const void* sb, const double* V, const uint8_t* dc, const uint8_t* wc, const long long* dc_off,
+                        const long long* wc_off, double* pop, double* eband, double* dU, bool with_forces, bool f64,
                         cudaStream_t s) {
   const int TB = 128, nb = (int)((32LL * n_core_total + TB - 1) / TB);
-  if (f64)
-    observables_kernel<double><<<nb, TB, 0, s>>>(m, R, species, g, sub_ptr, sub_atoms, orb_off, core_list, core_sub,
-                                                 core_local, n_core_total, pptr, pcol, (const double*)h0b,
-                                                 (const double*)sb, loc, N, V, nullptr, (const double*)Dc, nullptr,
-                                                 (const double*)Wc, dc_off, wc_off, n_pad, pop, eband, dU, with_forces);
-  else
-    observables_kernel<float><<<nb, TB, 0, s>>>(m, R, species, g, sub_ptr, sub_atoms, orb_off, core_list, core_sub,
-                                                core_local, n_core_total, pptr, pcol, (const float*)h0b,
-                                                (const float*)sb, loc, N, V, (const float*)Dc, nullptr,
-                                                (const float*)Wc, nullptr, dc_off, wc_off, n_pad, pop, eband, dU, with_forces);
+  auto go = [&](auto kernel, auto type) {
+    using T = decltype(type);
+    kernel<<<nb, TB, 0, s>>>(m, R, species, g, core_tab, n_core_total, pptr, pcol, pair_orb, (const T*)h0b,
+                             (const T*)sb, V, dc, wc, dc_off, wc_off, pop, eband, dU);
+  };
+  if (f64 && with_forces) go(observables_kernel<double, true>, double());
+  else if (f64) go(observables_kernel<double, false>, double());
+  else if (with_forces) go(observables_kernel<float, true>, float());
+  else go(observables_kernel<float, false>, float());
 }
 
 void launch_gd(const ModelDev& m, const long long* sub_ptr, const int* sub_atoms, const int* orb_off,

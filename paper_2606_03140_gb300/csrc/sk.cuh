@@ -22,12 +22,14 @@ void launch_gather(const ModelDev& m, const long long* sub_ptr, const int* sub_a
                    const int* loc, int N, const double* V, const long long* hoff, const long long* soff,
                    const int* n_pad, uint8_t* arena, int n_sub, const int* sub_of_row, long long total_rows,
                    int shift_only, bool f64, cudaStream_t s);
-void launch_observables(const ModelDev& m, const double* R, const int* species, const SkGeom& g,
-                        const long long* sub_ptr, const int* sub_atoms, const int* orb_off, const int* core_list,
-                        const int* core_sub, const int* core_local, int n_core_total, const long long* pptr,
-                        const int* pcol, const void* h0b, const void* sb, const int* loc, int N, const double* V,
-                        const void* Dc, const void* Wc, const long long* dc_off, const long long* wc_off,
-                        const int* n_pad, double* pop, double* eband, double* dU, int with_forces, bool f64,
+void launch_pair_orbs(const ModelDev& m, const int* species, const long long* sub_ptr, const int* orb_off,
+                      const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
+                      const long long* pptr, const int* pcol, const int* loc, int N, const int* n_pad, int4* core_tab,
+                      int* pair_orb, cudaStream_t s);
+void launch_observables(const ModelDev& m, const double* R, const int* species, const SkGeom& g, const int4* core_tab,
+                        int n_core_total, const long long* pptr, const int* pcol, const int* pair_orb, const void* h0b,
+                        const void* sb, const double* V, const uint8_t* dc, const uint8_t* wc, const long long* dc_off,
+                        const long long* wc_off, double* pop, double* eband, double* dU, bool with_forces, bool f64,
                         cudaStream_t s);
 void launch_gd(const ModelDev& m, const long long* sub_ptr, const int* sub_atoms, const int* orb_off,
                const int* species, const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
