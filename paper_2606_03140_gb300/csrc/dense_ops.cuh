@@ -48,6 +48,14 @@ void launch_f16x2_to_bf16x3(SlotViews views, const Sp2State* st, long long copy_
 // out1 = a1 in + b1 I (kind 0), the SP2 start (kind 1) or its first-order change (kind 2) from
 // the subgraph bounds; optional out2 = a2 in + b2 I.  Each output: master and / or planes
 // (format nsplit).
+// Terms of a sum over core rows: byte distance of a term's master from the result's, and its factor.
+struct RowTerms {
+  long long delta[4];
+  double a[4];
+  int n;
+};
+void launch_rows_sum(SlotViews y, const RowTerms& w, int master, int nsplit, int n_sub, int max_rows, uint8_t* arena,
+                     bool f64, cudaStream_t s);
 void launch_affine_planes(SlotViews in, SlotViews out1, double a1, double b1, int master1, int nsplit1,
                           SlotViews out2, double a2, double b2, int master2, int nsplit2, int kind,
                           const double* bounds, int n_sub, int max_rows, uint8_t* arena, bool f64, cudaStream_t s);

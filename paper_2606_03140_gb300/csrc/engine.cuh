@@ -68,16 +68,16 @@ enum OpId : int {
   OP_F_Z2, OP_F_Z4, OP_F_ST1, OP_F_SH0, OP_F_SH1, OP_F_SH2, OP_F_SH3, OP_F_U0_0, OP_F_U0_1,
   OP_F_V_0, OP_F_V_1, OP_F_V2, OP_F_IT1, OP_F_IH0, OP_F_IH1, OP_F_IH2, OP_F_IH3, OP_F_IH4, OP_F_IH5,
   OP_F_UP_0, OP_F_UP_1, OP_F_FIN, OP_F_S,
-  // core rows of F into the response slots (dT1 = Z_c F), and W of s: T2 = dT1 h~, Ws = 2 T2 Z
-  OP_F_FT1_0, OP_F_FT1_1, OP_F_T2S, OP_F_WS0, OP_F_WS1,
-  // second-order mu term: t = s - 2 s F (kR1 copy 1), its core rows (kdT2, kdDt), T2 = kdT2 h~
-  OP_F_T, OP_F_TT1_0, OP_F_TT1_1, OP_F_DT0, OP_F_DT1, OP_F_T2T,
+  // core rows of F into the response slots (dT1 = Z_c F)
+  OP_F_FT1_0, OP_F_FT1_1,
+  // second-order mu term: t = s - 2 s F (kR1 copy 1), its core rows (kdT2, kdDt)
+  OP_F_T, OP_F_TT1_0, OP_F_TT1_1, OP_F_DT0, OP_F_DT1,
   // mu shift at a saved doubling stage: U' = U Q + tau Q, Q ~ (I + tau U)^-1 (U in kY0), into kX
   OP_F_MOB_0, OP_F_MOB_1,
   // third- and fourth-order mu terms: P = t F (kT), u = t - 2 P - 2 s s (kY0), its core rows
-  // (kdT3, kdDu), T2 = kdT3 h~; Q = u F (kT), w = u - 2 Q - 6 s t (kY1), rows (kdT4, kdDw), T2
-  OP_F_TF, OP_F_U, OP_F_UT1_0, OP_F_UT1_1, OP_F_DU0, OP_F_DU1, OP_F_T2U,
-  OP_F_UF, OP_F_W, OP_F_WT1_0, OP_F_WT1_1, OP_F_DW0, OP_F_DW1, OP_F_T2W,
+  // (kdT3, kdDu); Q = u F (kT), w = u - 2 Q - 6 s t (kY1), rows (kdT4, kdDw)
+  OP_F_TF, OP_F_U, OP_F_UT1_0, OP_F_UT1_1, OP_F_DU0, OP_F_DU1,
+  OP_F_UF, OP_F_W, OP_F_WT1_0, OP_F_WT1_1, OP_F_DW0, OP_F_DW1,
   // G = (I - V) r(V) from the last doubling (kT); s = F - F^2 = G^2 / 4 (OP_F_S)
   OP_F_G,
   OP_NUM
