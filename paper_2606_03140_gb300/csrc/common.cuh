@@ -243,6 +243,28 @@ __device__ __forceinline__ void write_planes8(uint8_t* arena, long long off, lon
   if (fmt > 2) *reinterpret_cast<uint4*>(arena + off + 2 * plane) = *reinterpret_cast<const uint4*>(l);
 }
 
+// Sums of the threads before this one in a block of 1024; *total: of all.
+template <typename T>
+__device__ __forceinline__ T scan1024(T v, T* total) {
+  __shared__ T sums[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto warp_scan = [&](T x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const T y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    return x;
+  };
+  const T incl = warp_scan(v);
+  if (lane == 31) sums[warp] = incl;
+  __syncthreads();
+  if (warp == 0) sums[lane] = warp_scan(sums[lane]);
+  __syncthreads();
+  *total = sums[31];
+  return incl - v + (warp > 0 ? sums[warp - 1] : (T)0);
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

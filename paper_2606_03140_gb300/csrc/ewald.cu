@@ -428,24 +428,13 @@ __global__ void cell_count_kernel(const double* R, int N, EwaldGeom g, int* cell
 
 // exclusive scan of the cell counts (one block)
 __global__ void cell_scan_kernel(const int* count, int ncell, int* start) {
-  __shared__ int part[1024];
   const int per = (ncell + blockDim.x - 1) / blockDim.x;
   const int b0 = threadIdx.x * per, b1 = min(ncell, b0 + per);
   int s = 0;
   for (int c = b0; c < b1; ++c) s += count[c];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const int v = part[t];
-      part[t] = acc;
-      acc += v;
-    }
-    start[ncell] = acc;
-  }
-  __syncthreads();
-  int acc = part[threadIdx.x];
+  int total;
+  int acc = scan1024(s, &total);
+  if (threadIdx.x == 0) start[ncell] = total;
   for (int c = b0; c < b1; ++c) {
     start[c] = acc;
     acc += count[c];

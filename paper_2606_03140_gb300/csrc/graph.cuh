@@ -17,7 +17,7 @@ struct GraphBuilder {
   int* cell_count = nullptr;
   int* cell_start = nullptr;
   int* cell_fill = nullptr;
-  int* cell_atoms = nullptr;
+  float4* cell_atoms = nullptr;   // rounded coordinates and index
   int* cnt = nullptr;
   int* fillc = nullptr;
   int* ucnt = nullptr;
