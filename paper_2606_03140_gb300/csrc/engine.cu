@@ -22,18 +22,39 @@ __global__ void charges_kernel(const double* pop, const int* species, const doub
   if (i < N) q[i] = pop[i] - zval[species[i]];
 }
 
-// out[0] = sum a*b (b may be null -> sum a); fixed-order tree in one CTA.
-__global__ void dot_kernel(const double* a, const double* b, int N, double* out) {
+// *out = sum a*b (b may be null -> sum a) for each of a few pairs of vectors, a CTA each; fixed-order tree.
+struct Dots {
+  const double* a[3];
+  const double* b[3];
+  double* out[3];
+};
+__global__ void __launch_bounds__(1024) dot_kernel(const Dots d, int N) {
   __shared__ double red[1024];
+  const double *a = d.a[blockIdx.x], *b = d.b[blockIdx.x];
+  const int t = threadIdx.x;
   double s = 0.0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) s += b ? a[i] * b[i] : a[i];
-  red[threadIdx.x] = s;
+  if (b) {
+#pragma unroll 8
+    for (int i = t; i < N; i += 1024) s += a[i] * b[i];
+  } else {
+#pragma unroll 8
+    for (int i = t; i < N; i += 1024) s += a[i];
+  }
+  red[t] = s;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+  for (int o = 512; o >= 32; o >>= 1) {
+    if (t < o) red[t] += red[t + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[0] = red[0];
+  if (t >= 32) return;
+  double v = red[t];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (t == 0) *d.out[blockIdx.x] = v;
+}
+void launch_dots(const Dots& d, int count, int N, cudaStream_t s) { dot_kernel<<<count, 1024, 0, s>>>(d, N); }
+void launch_dot(const double* a, const double* b, int N, double* out, cudaStream_t s) {
+  launch_dots(Dots{{a}, {b}, {out}}, 1, N, s);
 }
 
 // max |a - b|
@@ -195,7 +216,7 @@ void gnn_get_params_f64(sedacs_ctx* ctx, double* d_p, bool grad);
 double gnn_train_step(sedacs_ctx* ctx, const double* X, const double* V, int n, float lr, bool want_loss);
 
 void dev_dot_into(sedacs_ctx* ctx, const double* a, const double* b, double* out) {
-  dot_kernel<<<1, 1024, 0, ctx->stream>>>(a, b, ctx->N, out);
+  launch_dot(a, b, ctx->N, out, ctx->stream);
   ctx->launches += 1;
 }
 
@@ -1066,10 +1087,11 @@ void launch_populations(sedacs_ctx* ctx, const long long* dc_off, double* pop) {
   launch_observables(ctx->model, ctx->d_R, ctx->d_species, sk_geom(ctx), ctx->d_core_tab, ctx->n_core_total, ctx->d_pptr,
                      ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, ctx->arena, dc_off,
                      dc_off, pop, nullptr, ctx->d_dU, false, ctx->f64, ctx->stream);
+  ctx->launches += 1;
 }
 
-// Populations / band energy (and forces) from the core rows; q = pop - Z; returns N_e count.
-sedacs_status observe(sedacs_ctx* ctx, bool with_forces, double* n_count) {
+// Populations / band energy (and forces) from the core rows; q = pop - Z.
+void observe(sedacs_ctx* ctx, bool with_forces) {
   cudaStream_t s = ctx->stream;
   const SkGeom g = sk_geom(ctx);
   if (with_forces) cudaMemsetAsync(ctx->d_dU, 0, sizeof(double) * 3 * ctx->N, s);
@@ -1077,10 +1099,7 @@ sedacs_status observe(sedacs_ctx* ctx, bool with_forces, double* n_count) {
                      ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, ctx->arena,
                      ctx->d_dcoff, ctx->d_wcoff, ctx->d_pop, ctx->d_eband, ctx->d_dU, with_forces, ctx->f64, s);
   charges_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_pop, ctx->d_species, ctx->d_zval, ctx->d_q, ctx->N);
-  dot_kernel<<<1, 1024, 0, s>>>(ctx->d_pop, nullptr, ctx->N, ctx->d_scal);
-  ctx->launches += 3;
-  if (n_count) *n_count = host_scalar(ctx, ctx->d_scal);
-  return SEDACS_OK;
+  ctx->launches += 2;
 }
 
 // ---- finite-temperature Fermi operator (Eq. 2) and the chemical potential ------------------------
@@ -1447,13 +1466,15 @@ sedacs_status fermi_reentry(sedacs_ctx* ctx, double mu) {
   return SEDACS_OK;
 }
 
-// Populations of the core rows at dc_off (per atom, the FP64 sum over each core atom's orbitals
-// and its subgraph) into pop, their sum into d_scal[k].
-void core_pops(sedacs_ctx* ctx, const long long* dc_off, double* pop, int k) {
-  cudaStream_t s = ctx->stream;
-  launch_populations(ctx, dc_off, pop);
-  dot_kernel<<<1, 1024, 0, s>>>(pop, nullptr, ctx->N, ctx->d_scal + k);
-  ctx->launches += 2;
+// Sums of the populations pop[k] into d_scal[at[k]].
+void sum_pops(sedacs_ctx* ctx, std::initializer_list<const double*> pop, std::initializer_list<int> at) {
+  Dots d{};
+  int k = 0;
+  for (const double* p : pop) d.a[k++] = p;
+  k = 0;
+  for (const int q : at) d.out[k++] = ctx->d_scal + q;
+  launch_dots(d, k, ctx->N, ctx->stream);
+  ctx->launches += 1;
 }
 
 // s = F - F^2 (as G^2 / 4 from the last doubling's V and r, still in kY0 and the Horner slot) and
@@ -1542,7 +1563,8 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
   int order = 2;                               // terms of the accepted mu expansion
   double* pop_s = ctx->d_rsp + 6LL * N;      // kept for the response calls (their dN/dmu weights)
   double* pop_t = ctx->d_rsp + 5LL * N;
-  double* pop_uw = ctx->d_rsp + 8LL * N;
+  double* pop_u = ctx->d_rsp + 8LL * N;
+  double* pop_w = ctx->d_rsp + 7LL * N;
   int pass = 0;
   bool done = false, have_stage = false;
   double step_old = b - a, step_prev = b - a;
@@ -1560,11 +1582,12 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
     }
     back_transform(ctx, false);                                   // T1 = Z_c F, D_c
     if (given) { done = true; break; }
-    core_pops(ctx, ctx->d_dcoff, ctx->d_pop, 9);                   // N(mu)
+    launch_populations(ctx, ctx->d_dcoff, ctx->d_pop);             // N(mu)
     STCHK(fermi_s_rows(ctx));
-    core_pops(ctx, ctx->d_dcoff_d, pop_s, 10);                     // sum of D_s populations
+    launch_populations(ctx, ctx->d_dcoff_d, pop_s);
     fermi_t_rows(ctx);
-    core_pops(ctx, ctx->d_dcoff_t, pop_t, 14);                     // sum of D_t populations
+    launch_populations(ctx, ctx->d_dcoff_t, pop_t);
+    sum_pops(ctx, {ctx->d_pop, pop_s, pop_t}, {9, 10, 14});        // N(mu), sums of the D_s and D_t populations
     double sc[6];
     CUCHK(cudaMemcpyAsync(sc, ctx->d_scal + 9, sizeof(sc), cudaMemcpyDeviceToHost, s));
     CUCHK(cudaStreamSynchronize(s));
@@ -1602,8 +1625,9 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
       if (std::fabs(beta * d2) <= lin2) { dmu = d2; order = 2; done = true; break; }
       if (std::fabs(beta * d2) <= 1.5 * lin) {
         fermi_uw_rows(ctx);
-        core_pops(ctx, ctx->d_dcoff_u, pop_uw, 11);                // sums of D_u and D_w populations
-        core_pops(ctx, ctx->d_dcoff_w, pop_uw, 12);
+        launch_populations(ctx, ctx->d_dcoff_u, pop_u);
+        launch_populations(ctx, ctx->d_dcoff_w, pop_w);
+        sum_pops(ctx, {pop_u, pop_w}, {11, 12});
         double s34[2];
         CUCHK(cudaMemcpyAsync(s34, ctx->d_scal + 11, sizeof(s34), cudaMemcpyDeviceToHost, s));
         CUCHK(cudaStreamSynchronize(s));
@@ -1692,7 +1716,6 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
   ctx->ht_stale = false;
   phase_end(ctx, 0, 3);
   double mu = *mu_io;
-  double nel = 0.0;
   phase_begin(ctx, 0);
   if (finite_t) {
     STCHK(fermi_density(ctx, &mu));
@@ -1704,8 +1727,7 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
   if (!finite_t) back_transform(ctx, true);
   // when forces follow (XL-BOMD), the same pass also contracts the force blocks
   const bool fused = ctx->fuse_forces;
-  STCHK(observe(ctx, fused, &nel));
-  ctx->fermi_count_err = nel - ctx->n_electrons;
+  observe(ctx, fused);
   ctx->du_ready = fused;
   launch_gd(ctx->model, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_species, ctx->part.perm,
             ctx->d_core_sub, ctx->d_core_local, ctx->n_core_total, ctx->arena, ctx->f64, ctx->d_dcoff, ctx->d_n_pad,
@@ -1713,15 +1735,16 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
   ctx->launches += 1;
   nan_scan_kernel<<<nblk(ctx->N, 256), 256, 0, s>>>(ctx->d_q, ctx->N, ctx->d_err);
   ctx->launches += 1;
-  // band and Coulomb energies
-  dot_kernel<<<1, 1024, 0, s>>>(ctx->d_eband, nullptr, ctx->N, ctx->d_scal + 1);
+  // electron count, band and Coulomb energies
   coul_a_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_q, ctx->d_n, ctx->d_tmp, ctx->N);
-  dot_kernel<<<1, 1024, 0, s>>>(ctx->d_tmp, ctx->d_V, ctx->N, ctx->d_scal + 2);
-  ctx->launches += 3;
+  launch_dots(Dots{{ctx->d_pop, ctx->d_eband, ctx->d_tmp}, {nullptr, nullptr, ctx->d_V},
+                   {ctx->d_scal, ctx->d_scal + 1, ctx->d_scal + 2}}, 3, ctx->N, s);
+  ctx->launches += 2;
   double sc[3];
   CUCHK(cudaMemcpyAsync(sc, ctx->d_scal, sizeof(double) * 3, cudaMemcpyDeviceToHost, s));
   CUCHK(cudaStreamSynchronize(s));
   phase_end(ctx, 0, 5);
+  ctx->fermi_count_err = sc[0] - ctx->n_electrons;
   ctx->e_band = sc[1];
   ctx->e_coul = sc[2];
   ctx->mu = mu;
@@ -1743,7 +1766,7 @@ sedacs_status forces_core(sedacs_ctx* ctx) {
   if (!ctx->have_density) { ctx->err = "no density: call sedacs_subgraph_density first"; return SEDACS_EINVAL; }
   cudaStream_t s = ctx->stream;
   phase_begin(ctx, 0);
-  if (!ctx->du_ready) STCHK(observe(ctx, true, nullptr));   // else done with the density
+  if (!ctx->du_ready) observe(ctx, true);   // else done with the density
   ctx->du_ready = false;
   coul_a_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_q, ctx->d_n, ctx->d_tmp, ctx->N);
   CUCHK(ctx->ew.gradient(ctx->d_tmp, ctx->d_n, ctx->d_F, s, ctx->ew_tag));
@@ -1752,7 +1775,7 @@ sedacs_status forces_core(sedacs_ctx* ctx) {
                    ctx->d_dU, ctx->f64, s);
   neg_kernel<<<nblk(3 * ctx->N, 256), 256, 0, s>>>(ctx->d_dU, ctx->d_F, 3 * ctx->N);
   nan_scan_kernel<<<nblk(3 * ctx->N, 256), 256, 0, s>>>(ctx->d_F, 3 * ctx->N, ctx->d_err);
-  dot_kernel<<<1, 1024, 0, s>>>(ctx->d_erep, nullptr, ctx->N, ctx->d_scal + 3);
+  launch_dot(ctx->d_erep, nullptr, ctx->N, ctx->d_scal + 3, s);
   ctx->launches += 11;
   ctx->e_rep = host_scalar(ctx, ctx->d_scal + 3);
   phase_end(ctx, 0, 6);
@@ -1808,7 +1831,7 @@ sedacs_status cycle(sedacs_ctx* ctx, double* mu, bool keep_prev = false) {
 // ---- charge response and low-rank kernel (SI Sec. B) ------------------------------------------
 
 double dev_dot(sedacs_ctx* ctx, const double* a, const double* b) {
-  dot_kernel<<<1, 1024, 0, ctx->stream>>>(a, b, ctx->N, ctx->d_scal + 8);
+  launch_dot(a, b, ctx->N, ctx->d_scal + 8, ctx->stream);
   ctx->launches += 1;
   return host_scalar(ctx, ctx->d_scal + 8);
 }
@@ -1849,7 +1872,6 @@ sedacs_status response_sp2(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
   run_op(ctx, ctx->zc == 0 ? OP_DT1_0 : OP_DT1_1, n2 > ns ? n2 : ns, ns);   // dT1 = Z_c dX
   run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);                     // dD_c = 2 dT1 Z
   launch_populations(ctx, ctx->d_dcoff_d, d_dq);
-  ctx->launches += 1;
   return check_dev_err(ctx);
 }
 
@@ -1885,8 +1907,7 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
   // per side stays small.
   if (ctx->fermi_dndmu > 0.0) {
     const double* w = ctx->d_rsp + 6LL * N;
-    dot_kernel<<<1, 1024, 0, s>>>(w, dV, N, ctx->d_scal + 12);
-    dot_kernel<<<1, 1024, 0, s>>>(w, nullptr, N, ctx->d_scal + 13);
+    launch_dots(Dots{{w, w}, {dV, nullptr}, {ctx->d_scal + 12, ctx->d_scal + 13}}, 2, N, s);
     ctx->launches += 2;
     double sw[2];
     CUCHK(cudaMemcpyAsync(sw, ctx->d_scal + 12, sizeof(sw), cudaMemcpyDeviceToHost, s));
@@ -1908,9 +1929,10 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
     STCHK(run_fermi(ctx, ctx->mu, nd));
     run_op(ctx, ctx->zc == 0 ? OP_F_FT1_0 : OP_F_FT1_1, 3, ns);   // dT1 = Z_c F
     run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);         // 2 dT1 Z
-    core_pops(ctx, ctx->d_dcoff_d, q, 9);
+    launch_populations(ctx, ctx->d_dcoff_d, q);
     STCHK(fermi_s_rows(ctx));
-    core_pops(ctx, ctx->d_dcoff_d, ps, 10);
+    launch_populations(ctx, ctx->d_dcoff_d, ps);
+    sum_pops(ctx, {q, ps}, {9, 10});
     double sc[2];
     CUCHK(cudaMemcpyAsync(sc, ctx->d_scal + 9, sizeof(sc), cudaMemcpyDeviceToHost, s));
     CUCHK(cudaStreamSynchronize(s));
