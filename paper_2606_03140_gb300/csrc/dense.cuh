@@ -86,13 +86,17 @@ struct GemmParams {
                       // the fp16-operand kernel writes two fp16 planes unless 3 is asked for)
   double alpha, beta; // epilogue coefficients (FP64 in the FP64 path, rounded to FP32 on the tensor path)
   double g1, g2;
+  // products of one launch with the same B and coefficients: task t is product t % n_batch of work item t / n_batch
+  // (so that the tiles of B are read together); bytes from the first product's A, C1 and output
+  int n_batch;
+  long long batch_a[3], batch_c[3], batch_out[3];
   int ops_upper;      // generic mode: A and B are symmetric and may be stored as their upper 128x128 tiles
                       // only (blocks left of the diagonal read as transposes)
 };
 
 #if defined(__CUDACC__)
-// The problem of subgraph i: its offsets in the slots of the product.
-__device__ __forceinline__ GemmMat gemm_mat(const GemmParams& p, int i) {
+// The problem of subgraph i and product b of the launch: its offsets in the slots of the product.
+__device__ __forceinline__ GemmMat gemm_mat(const GemmParams& p, int i, int b) {
   const GemmSub s = p.subs[i];
   GemmMat m = p.slot;
   const int ob = p.f64 ? 8 : 2, mb = p.f64 ? 8 : 4;          // bytes an operand / a master element
@@ -104,6 +108,11 @@ __device__ __forceinline__ GemmMat gemm_mat(const GemmParams& p, int i) {
   m.x_off += s.sq * mb;
   if (m.c_off >= 0) m.c_off += (p.c_rows ? s.rw : s.sq) * (m.c_planes ? 2 : mb);
   if (m.c2_off >= 0) m.c2_off += (p.c2_rows ? s.rw : s.sq) * mb;
+  if (b > 0) {
+    m.a_off += p.batch_a[b];
+    m.c_off += p.batch_c[b];
+    m.out_off += p.batch_out[b];
+  }
   m.tr_off = s.tr_off;
   m.n_pad = s.n_pad;
   m.n_real = m.k_real = s.n_real;

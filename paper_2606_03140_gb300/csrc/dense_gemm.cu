@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_persistent(const GemmPa
     if (lane == 0) {
       long long g = 0;
       for (int t = blockIdx.x; t < n_work && ok; t += gridDim.x) {
-        const GemmWork w = p.work[t];
+        const GemmWork w = p.work[t / p.n_batch];
         if (!tile_live(w)) continue;
-        const GemmMat m = gemm_mat(p, w.mat);
+        const GemmMat m = gemm_mat(p, w.mat, t % p.n_batch);
         const int cur = tile_cur(w, m);
         const long long in_shift = stepping ? cur * m.buf_stride : 0;
         const uint8_t* A = p.arena + m.a_off + (stepping ? in_shift : (m.a_from_sp2 ? cur * m.buf_stride : 0));
@@ -178,9 +178,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_persistent(const GemmPa
       long long g = 0;
       int ti = 0;
       for (int t = blockIdx.x; t < n_work && ok; t += gridDim.x) {
-        const GemmWork w = p.work[t];
+        const GemmWork w = p.work[t / p.n_batch];
         if (!tile_live(w)) continue;
-        const GemmMat m = gemm_mat(p, w.mat);
+        const GemmMat m = gemm_mat(p, w.mat, t % p.n_batch);
         const int kb_end = (m.k_real + 63) >> 6;
         const uint32_t prev = (uint32_t)((ti - 1) & 1);
         // accumulator parts of the previous tile that the next k-block overwrites (all three at
@@ -241,9 +241,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_persistent(const GemmPa
     float* tb = tbuf + warp * (32 * 32);
     int ti = 0;
     for (int t = blockIdx.x; t < n_work && ok; t += gridDim.x) {
-      const GemmWork w = p.work[t];
+      const GemmWork w = p.work[t / p.n_batch];
       if (!tile_live(w)) continue;
-      const GemmMat m = gemm_mat(p, w.mat);
+      const GemmMat m = gemm_mat(p, w.mat, t % p.n_batch);
       const int cur = tile_cur(w, m);
       const int branch_sq = stepping ? (p.sp2[w.mat].y >= 0.5) : 0;
       const long long in_shift = stepping ? cur * m.buf_stride : 0;
@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(kF64Threads) f64_gemm_kernel(const GemmParams 
   __shared__ double As[16][kT + 2];
   __shared__ double Bs[16][kT + 2];
   __shared__ double red[2][4];
-  const GemmWork w = p.work[blockIdx.x];
-  const GemmMat m = gemm_mat(p, w.mat);
+  const GemmWork w = p.work[blockIdx.x / p.n_batch];
+  const GemmMat m = gemm_mat(p, w.mat, blockIdx.x % p.n_batch);
   int cur = 0, branch_sq = 0;
   const bool stepping = (p.mode == kModeSp2 || p.mode == kModeRsp);
   if (stepping) {

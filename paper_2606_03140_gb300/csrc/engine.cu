@@ -491,10 +491,18 @@ void build_op(sedacs_ctx* ctx, int id, int a, int b, int out, int mode, double a
   op.ops_upper = 0;
 }
 
-void run_op(sedacs_ctx* ctx, int id, int nsplit_in, int nsplit_out) {
-  const GemmOp& op = ctx->ops[id];
-  const int n_work = ctx->n_work[op.work];
-  GemmParams p;
+// The products ids (up to three) in one launch: they differ in A, C1 and the master output only.
+void run_ops(sedacs_ctx* ctx, std::initializer_list<int> ids, int nsplit_in, int nsplit_out) {
+  const GemmOp& op = ctx->ops[*ids.begin()];
+  const int n_work = ctx->n_work[op.work] * (int)ids.size();
+  GemmParams p{};
+  for (const int id : ids) {
+    const GemmMat& m = ctx->ops[id].slot;
+    p.batch_a[p.n_batch] = m.a_off - op.slot.a_off;
+    p.batch_c[p.n_batch] = m.c_off - op.slot.c_off;
+    p.batch_out[p.n_batch] = m.out_off - op.slot.out_off;
+    ++p.n_batch;
+  }
   p.work = ctx->d_work[op.work];
   p.subs = ctx->d_subs;
   p.slot = op.slot;
@@ -519,6 +527,8 @@ void run_op(sedacs_ctx* ctx, int id, int nsplit_in, int nsplit_out) {
   else launch_gemm_tc(p, n_work, nsplit_in, ctx->stream);
   ctx->launches += n_work > 0 ? 1 : 0;
 }
+
+void run_op(sedacs_ctx* ctx, int id, int nsplit_in, int nsplit_out) { run_ops(ctx, {id}, nsplit_in, nsplit_out); }
 
 template <typename T>
 sedacs_status upload_vec(sedacs_ctx* ctx, T** dst, const std::vector<T>& v) {
@@ -1478,7 +1488,7 @@ void sum_pops(sedacs_ctx* ctx, std::initializer_list<const double*> pop, std::in
 }
 
 // s = F - F^2 (as G^2 / 4 from the last doubling's V and r, still in kY0 and the Horner slot) and
-// the core rows D_s = 2 Z_c s Z (kdT1 -> kdDc); d/dmu of F is beta s.
+// the core rows Z_c s (kdT1); d/dmu of F is beta s.
 sedacs_status fermi_s_rows(sedacs_ctx* ctx) {
   const int ns = ctx->nsplit_ns;
   const int nf = ctx->f64 ? 0 : ctx->nsplit_fermi;
@@ -1493,16 +1503,14 @@ sedacs_status fermi_s_rows(sedacs_ctx* ctx) {
   }
   run_fop(ctx, OP_F_S, nf, ctx->f64 ? 0 : 3);
   run_op(ctx, ctx->zc == 0 ? OP_DT1_0 : OP_DT1_1, 3, ns);
-  run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);
   return SEDACS_OK;
 }
 
-// t = s (I - 2F) and its core rows D_t = 2 Z_c t Z (kdT2 -> kdDt); d^2 F / dmu^2 is beta^2 t.
+// t = s (I - 2F) and its core rows Z_c t (kdT2); d^2 F / dmu^2 is beta^2 t.
 void fermi_t_rows(sedacs_ctx* ctx) {
   const int ns = ctx->nsplit_ns;
   run_fop(ctx, OP_F_T, ctx->f64 ? 0 : 3, ctx->f64 ? 0 : 3);
   run_op(ctx, ctx->zc == 0 ? OP_F_TT1_0 : OP_F_TT1_1, 3, ns);
-  run_op(ctx, ctx->zc == 0 ? OP_F_DT0 : OP_F_DT1, ns, 0);
 }
 
 
@@ -1515,11 +1523,11 @@ void fermi_uw_rows(sedacs_ctx* ctx) {
   run_fop(ctx, OP_F_TF, nl, no);
   run_fop(ctx, OP_F_U, nl, no);
   run_op(ctx, ctx->zc == 0 ? OP_F_UT1_0 : OP_F_UT1_1, nl, ns);
-  run_op(ctx, ctx->zc == 0 ? OP_F_DU0 : OP_F_DU1, ns, 0);
   run_fop(ctx, OP_F_UF, nl, no);
   run_fop(ctx, OP_F_W, nl, no);
   run_op(ctx, ctx->zc == 0 ? OP_F_WT1_0 : OP_F_WT1_1, nl, ns);
-  run_op(ctx, ctx->zc == 0 ? OP_F_DW0 : OP_F_DW1, ns, 0);
+  if (ctx->zc == 0) run_ops(ctx, {OP_F_DU0, OP_F_DW0}, ns, 0);
+  else run_ops(ctx, {OP_F_DU1, OP_F_DW1}, ns, 0);
 }
 
 // Slot sy += sum_k c_k (slot sx[k]) over the core rows, as master and / or planes.
@@ -1580,12 +1588,20 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
       STCHK(run_fermi(ctx, mu, fermi_doublings(ctx, mu)));
       have_stage = true;
     }
-    back_transform(ctx, false);                                   // T1 = Z_c F, D_c
-    if (given) { done = true; break; }
-    launch_populations(ctx, ctx->d_dcoff, ctx->d_pop);             // N(mu)
+    if (given) {
+      back_transform(ctx, false);                                  // T1 = Z_c F, D_c
+      done = true;
+      break;
+    }
+    // the rows Z_c X of F, s and t, then D_c, D_s and D_t in one launch that reads Z once (9,000 atoms: 176 us,
+    // three launches 252 us)
+    run_op(ctx, ctx->zc == 0 ? OP_T1_0 : OP_T1_1, x_split_final(ctx), ns);
     STCHK(fermi_s_rows(ctx));
-    launch_populations(ctx, ctx->d_dcoff_d, pop_s);
     fermi_t_rows(ctx);
+    if (ctx->zc == 0) run_ops(ctx, {OP_DC0, OP_DDC0, OP_F_DT0}, ns, 0);
+    else run_ops(ctx, {OP_DC1, OP_DDC1, OP_F_DT1}, ns, 0);
+    launch_populations(ctx, ctx->d_dcoff, ctx->d_pop);
+    launch_populations(ctx, ctx->d_dcoff_d, pop_s);
     launch_populations(ctx, ctx->d_dcoff_t, pop_t);
     sum_pops(ctx, {ctx->d_pop, pop_s, pop_t}, {9, 10, 14});        // N(mu), sums of the D_s and D_t populations
     double sc[6];
@@ -1931,6 +1947,7 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
     run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);         // 2 dT1 Z
     launch_populations(ctx, ctx->d_dcoff_d, q);
     STCHK(fermi_s_rows(ctx));
+    run_op(ctx, ctx->zc == 0 ? OP_DDC0 : OP_DDC1, ns, 0);         // D_s = 2 dT1 Z
     launch_populations(ctx, ctx->d_dcoff_d, ps);
     sum_pops(ctx, {q, ps}, {9, 10});
     double sc[2];
