@@ -1092,12 +1092,15 @@ void back_transform(sedacs_ctx* ctx, bool with_w) {
   }
 }
 
-// Populations of the core rows at dc_off.
-void launch_populations(sedacs_ctx* ctx, const long long* dc_off, double* pop) {
+// Populations of n matrices' core rows.
+void launch_populations(sedacs_ctx* ctx, const CoreRows& rows, int n) {
   launch_observables(ctx->model, ctx->d_R, ctx->d_species, sk_geom(ctx), ctx->d_core_tab, ctx->n_core_total, ctx->d_pptr,
-                     ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, ctx->arena, dc_off,
-                     dc_off, pop, nullptr, ctx->d_dU, false, ctx->f64, ctx->stream);
+                     ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, rows, n, nullptr,
+                     nullptr, ctx->d_dU, false, ctx->f64, ctx->stream);
   ctx->launches += 1;
+}
+void launch_populations(sedacs_ctx* ctx, const long long* dc_off, double* pop) {
+  launch_populations(ctx, CoreRows{{dc_off}, {pop}}, 1);
 }
 
 // Populations / band energy (and forces) from the core rows; q = pop - Z.
@@ -1106,8 +1109,9 @@ void observe(sedacs_ctx* ctx, bool with_forces) {
   const SkGeom g = sk_geom(ctx);
   if (with_forces) cudaMemsetAsync(ctx->d_dU, 0, sizeof(double) * 3 * ctx->N, s);
   launch_observables(ctx->model, ctx->d_R, ctx->d_species, g, ctx->d_core_tab, ctx->n_core_total, ctx->d_pptr,
-                     ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena, ctx->arena,
-                     ctx->d_dcoff, ctx->d_wcoff, ctx->d_pop, ctx->d_eband, ctx->d_dU, with_forces, ctx->f64, s);
+                     ctx->d_pcol, ctx->d_pair_orb, ctx->d_h0b, ctx->d_sb, ctx->d_V, ctx->arena,
+                     CoreRows{{ctx->d_dcoff}, {ctx->d_pop}}, 1, ctx->d_wcoff, ctx->d_eband, ctx->d_dU, with_forces,
+                     ctx->f64, s);
   charges_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_pop, ctx->d_species, ctx->d_zval, ctx->d_q, ctx->N);
   ctx->launches += 2;
 }
@@ -1600,9 +1604,7 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
     fermi_t_rows(ctx);
     if (ctx->zc == 0) run_ops(ctx, {OP_DC0, OP_DDC0, OP_F_DT0}, ns, 0);
     else run_ops(ctx, {OP_DC1, OP_DDC1, OP_F_DT1}, ns, 0);
-    launch_populations(ctx, ctx->d_dcoff, ctx->d_pop);
-    launch_populations(ctx, ctx->d_dcoff_d, pop_s);
-    launch_populations(ctx, ctx->d_dcoff_t, pop_t);
+    launch_populations(ctx, CoreRows{{ctx->d_dcoff, ctx->d_dcoff_d, ctx->d_dcoff_t}, {ctx->d_pop, pop_s, pop_t}}, 3);
     sum_pops(ctx, {ctx->d_pop, pop_s, pop_t}, {9, 10, 14});        // N(mu), sums of the D_s and D_t populations
     double sc[6];
     CUCHK(cudaMemcpyAsync(sc, ctx->d_scal + 9, sizeof(sc), cudaMemcpyDeviceToHost, s));
@@ -1641,8 +1643,7 @@ sedacs_status fermi_density(sedacs_ctx* ctx, double* mu_io) {
       if (std::fabs(beta * d2) <= lin2) { dmu = d2; order = 2; done = true; break; }
       if (std::fabs(beta * d2) <= 1.5 * lin) {
         fermi_uw_rows(ctx);
-        launch_populations(ctx, ctx->d_dcoff_u, pop_u);
-        launch_populations(ctx, ctx->d_dcoff_w, pop_w);
+        launch_populations(ctx, CoreRows{{ctx->d_dcoff_u, ctx->d_dcoff_w}, {pop_u, pop_w}}, 2);
         sum_pops(ctx, {pop_u, pop_w}, {11, 12});
         double s34[2];
         CUCHK(cudaMemcpyAsync(s34, ctx->d_scal + 11, sizeof(s34), cudaMemcpyDeviceToHost, s));

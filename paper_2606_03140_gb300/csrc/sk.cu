@@ -267,7 +267,7 @@ template <typename T> struct __align__(16) Row4 { T v[4]; };
 
 // Collected observables, one warp per core atom (lanes split its neighbour list; sums are
 // combined by a fixed shuffle tree, the reaction on B by FP64 atomics).  Populations alone (FORCES false, the form
-// the chemical potential's passes use four to eight times a density; eband may be null) are bound by the FP64
+// the chemical potential's passes use for three matrices at a time, blockIdx.y; eband may be null) are bound by the FP64
 // additions and by the latency of the gathers, which the tables of pair_orbs_kernel cut from six to three levels;
 // without the force blocks' registers twice the warps fit.  Measured (GB300, 9,000 atoms): 82 us, 160 us with
 // one kernel for both that looked up every pair; with forces 267 us, 306 us.
@@ -276,16 +276,16 @@ __global__ void __launch_bounds__(128) observables_kernel(const ModelDev m, cons
                                                           SkGeom g, const int4* core_tab, int n_core_total,
                                                           const long long* pptr, const int* pcol, const int* pair_orb,
                                                           const T* h0b, const T* sb, const double* V,
-                                                          const uint8_t* dc, const uint8_t* wc, const long long* dc_off,
-                                                          const long long* wc_off, double* pop, double* eband,
-                                                          double* dU) {
+                                                          const uint8_t* arena, const CoreRows rows,
+                                                          const long long* wc_off, double* eband, double* dU) {
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= n_core_total) return;
   const int4 ct = core_tab[t];
   const int A = ct.x, na = ct.z & 7, oa = ct.z >> 3, ld = ct.w;
-  const T* D = reinterpret_cast<const T*>(dc + dc_off[ct.y]) + (long long)oa * ld;   // the core atom's rows
-  const T* W = FORCES ? reinterpret_cast<const T*>(wc + wc_off[ct.y]) + (long long)oa * ld : nullptr;
+  // the core atom's rows
+  const T* D = reinterpret_cast<const T*>(arena + rows.off[blockIdx.y][ct.y]) + (long long)oa * ld;
+  const T* W = FORCES ? reinterpret_cast<const T*>(arena + wc_off[ct.y]) + (long long)oa * ld : nullptr;
   const bool band = FORCES || eband != nullptr;
   const int sa = species[A];
   double p_acc = 0.0, e_acc = 0.0;
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(128) observables_kernel(const ModelDev m, cons
   if (FORCES)
     for (int c = 0; c < 3; ++c) fa[c] = warp_sum(fa[c]);
   if (lane == 0) {
-    pop[A] = p_acc;
+    rows.pop[blockIdx.y][A] = p_acc;
     if (band) eband[A] = e_acc;
     if (FORCES)
       for (int c = 0; c < 3; ++c) atomicAdd(&dU[3 * A + c], fa[c]);
@@ -497,14 +497,14 @@ void launch_pair_orbs(const ModelDev& m, const int* species, const long long* su
 
 void launch_observables(const ModelDev& m, const double* R, const int* species, const SkGeom& g, const int4* core_tab,
                         int n_core_total, const long long* pptr, const int* pcol, const int* pair_orb, const void* h0b,
-                        const void* sb, const double* V, const uint8_t* dc, const uint8_t* wc, const long long* dc_off,
-                        const long long* wc_off, double* pop, double* eband, double* dU, bool with_forces, bool f64,
+                        const void* sb, const double* V, const uint8_t* arena, const CoreRows& rows, int n_rows,
+                        const long long* wc_off, double* eband, double* dU, bool with_forces, bool f64,
                         cudaStream_t s) {
   const int TB = 128, nb = (int)((32LL * n_core_total + TB - 1) / TB);
   auto go = [&](auto kernel, auto type) {
     using T = decltype(type);
-    kernel<<<nb, TB, 0, s>>>(m, R, species, g, core_tab, n_core_total, pptr, pcol, pair_orb, (const T*)h0b,
-                             (const T*)sb, V, dc, wc, dc_off, wc_off, pop, eband, dU);
+    kernel<<<dim3(nb, n_rows), TB, 0, s>>>(m, R, species, g, core_tab, n_core_total, pptr, pcol, pair_orb,
+                                           (const T*)h0b, (const T*)sb, V, arena, rows, wc_off, eband, dU);
   };
   if (f64 && with_forces) go(observables_kernel<double, true>, double());
   else if (f64) go(observables_kernel<double, false>, double());

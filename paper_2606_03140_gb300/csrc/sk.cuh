@@ -26,10 +26,15 @@ void launch_pair_orbs(const ModelDev& m, const int* species, const long long* su
                       const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
                       const long long* pptr, const int* pcol, const int* loc, int N, const int* n_pad, int4* core_tab,
                       int* pair_orb, cudaStream_t s);
+// Matrices whose core rows (byte offsets in the arena per subgraph) are condensed, and their populations.
+struct CoreRows {
+  const long long* off[3];
+  double* pop[3];
+};
 void launch_observables(const ModelDev& m, const double* R, const int* species, const SkGeom& g, const int4* core_tab,
                         int n_core_total, const long long* pptr, const int* pcol, const int* pair_orb, const void* h0b,
-                        const void* sb, const double* V, const uint8_t* dc, const uint8_t* wc, const long long* dc_off,
-                        const long long* wc_off, double* pop, double* eband, double* dU, bool with_forces, bool f64,
+                        const void* sb, const double* V, const uint8_t* arena, const CoreRows& rows, int n_rows,
+                        const long long* wc_off, double* eband, double* dU, bool with_forces, bool f64,
                         cudaStream_t s);
 void launch_gd(const ModelDev& m, const long long* sub_ptr, const int* sub_atoms, const int* orb_off,
                const int* species, const int* core_list, const int* core_sub, const int* core_local, int n_core_total,
