@@ -87,9 +87,9 @@ struct GemmParams {
   double alpha, beta; // epilogue coefficients (FP64 in the FP64 path, rounded to FP32 on the tensor path)
   double g1, g2;
   // products of one launch with the same B and coefficients: task t is product t % n_batch of work item t / n_batch
-  // (so that the tiles of B are read together); bytes from the first product's A, C1 and output
+  // (so that the tiles of B are read together); bytes from the first product's A, C1 and outputs
   int n_batch;
-  long long batch_a[3], batch_c[3], batch_out[3];
+  long long batch_a[5], batch_c[5], batch_out[5], batch_outp[5];
   int ops_upper;      // generic mode: A and B are symmetric and may be stored as their upper 128x128 tiles
                       // only (blocks left of the diagonal read as transposes)
 };
@@ -112,6 +112,7 @@ __device__ __forceinline__ GemmMat gemm_mat(const GemmParams& p, int i, int b) {
     m.a_off += p.batch_a[b];
     m.c_off += p.batch_c[b];
     m.out_off += p.batch_out[b];
+    m.outp_off += p.batch_outp[b];
   }
   m.tr_off = s.tr_off;
   m.n_pad = s.n_pad;

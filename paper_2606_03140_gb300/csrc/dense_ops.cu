@@ -20,36 +20,60 @@ __global__ void split_planes_kernel(SlotViews views, uint8_t* arena, int nsplit)
   }
 }
 
-// Core rows y + sum_k a_k x_k over the terms, written as master and / or split planes.  One warp per row, 8 columns
-// per lane.  Sums of FP32 rows round like FP64 sums at the cost of FP32 ones: an unevaluated pair of floats holds the
-// sum to 2^-44 of its terms' magnitude; where the FP64 sum could round to another float (one element in about 10^5)
-// it is taken.  Memory bound (12 to 24 bytes an element), where FP64 sums were bound by the FP64 pipe.
-// Measured (GB300, 9,000 atoms, four terms): 68 us, 301 us with FP64 sums.
+// Core rows y + sum_k a_k x_k over the terms.  One warp per row, 8 columns per lane.  Sums of FP32 rows round like
+// FP64 ones at the cost of FP32 ones: a pair of floats holds the sum (EACH: every product, which is rounded and added
+// by itself) to 2^-44 of its terms' magnitude; where the FP64 sum could round to another float (one element in about
+// 10^5) it is taken.  Memory bound (12 to 24 bytes an element), where FP64 sums were bound by the FP64 pipe.
+// Measured (GB300, 9,000 atoms, four terms): 76 us, 301 us with FP64 sums; EACH 69 us, 328 us.
+__device__ __forceinline__ float pair_round(float hi, float lo, float mag, bool& sure) {
+  const float eps = mag * 0x1p-42f;
+  const float r0 = __fadd_rn(hi, __fsub_rn(lo, eps)), r1 = __fadd_rn(hi, __fadd_rn(lo, eps));
+  sure = r0 == r1;
+  return r0;
+}
+
+// The sum in FP64 (a call, so that it is not executed under a predicate for every element).
+template <bool EACH>
+__device__ __noinline__ float rows_sum_f64(float y, float x0, float x1, float x2, float x3, const double* a, int n) {
+  const float x[4] = {x0, x1, x2, x3};
+  double acc = 0.0;
+  float v = y;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (k < n) {
+      if (EACH) v += (float)(a[k] * (double)x[k]);
+      else acc += a[k] * (double)x[k];
+    }
+  return EACH ? v : (float)((double)y + acc);
+}
+
+template <bool EACH>
 __device__ __forceinline__ float rows_sum1(float y, const float (&x)[4], const float (&ah)[4], const float (&al)[4],
                                            const RowTerms& w) {
   float hi = y, lo = 0.0f, mag = fabsf(y);
+  bool sure, all = true;
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if (k < w.n) {
       const float p = __fmul_rn(ah[k], x[k]);
       const float r = __fmaf_rn(al[k], x[k], __fmaf_rn(ah[k], x[k], -p));      // a x = p + r
-      const float t = __fadd_rn(hi, p);
-      const float b = __fsub_rn(t, hi);
-      const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(p, b));
-      hi = t;
-      lo = __fadd_rn(lo, __fadd_rn(e, r));
-      mag += fabsf(p);
+      if (EACH) {
+        hi = __fadd_rn(hi, pair_round(p, r, fabsf(p), sure));
+        all = all && sure;
+      } else {
+        const float t = __fadd_rn(hi, p);
+        const float b = __fsub_rn(t, hi);
+        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(p, b));
+        hi = t;
+        lo = __fadd_rn(lo, __fadd_rn(e, r));
+        mag += fabsf(p);
+      }
     }
-  const float eps = mag * 0x1p-42f;
-  const float r0 = __fadd_rn(hi, __fsub_rn(lo, eps)), r1 = __fadd_rn(hi, __fadd_rn(lo, eps));
-  if (r0 == r1) return r0;
-  double acc = 0.0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (k < w.n) acc += w.a[k] * (double)x[k];
-  return (float)((double)y + acc);
+  if (!EACH) hi = pair_round(hi, lo, mag, all);
+  return all ? hi : rows_sum_f64<EACH>(y, x[0], x[1], x[2], x[3], w.a, w.n);
 }
 
+template <bool EACH>
 __device__ __forceinline__ void rows_sum8(uint8_t* m, const RowTerms& w, long long el, float (&y)[8]) {
   auto load = [&](const uint8_t* p, float (&v)[8]) {
     *reinterpret_cast<float4*>(v) = reinterpret_cast<const float4*>(p)[0];
@@ -68,21 +92,23 @@ __device__ __forceinline__ void rows_sum8(uint8_t* m, const RowTerms& w, long lo
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     const float xe[4] = {x[0][e], x[1][e], x[2][e], x[3][e]};
-    y[e] = rows_sum1(y[e], xe, ah, al, w);
+    y[e] = rows_sum1<EACH>(y[e], xe, ah, al, w);
   }
 }
 
+template <bool EACH>
 __device__ __forceinline__ void rows_sum8(uint8_t* m, const RowTerms& w, long long el, double (&y)[8]) {
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
-    double acc = 0.0;
+    y[e] = reinterpret_cast<const double*>(m)[el + e];
+    double acc = EACH ? y[e] : 0.0;
     for (int k = 0; k < w.n; ++k) acc += w.a[k] * reinterpret_cast<const double*>(m + w.delta[k])[el + e];
-    y[e] = reinterpret_cast<const double*>(m)[el + e] + acc;
+    y[e] = EACH ? acc : y[e] + acc;
   }
 }
 
-template <typename T>
-__global__ void rows_sum_kernel(SlotViews views, RowTerms w, int master, int nsplit, uint8_t* arena) {
+template <typename T, bool EACH>
+__global__ void rows_sum_kernel(SlotViews views, RowTerms w, uint8_t* arena) {
   const SubView v = views[blockIdx.y];
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= v.rows_pad) return;
@@ -90,17 +116,10 @@ __global__ void rows_sum_kernel(SlotViews views, RowTerms w, int master, int nsp
   for (int c8 = (threadIdx.x & 31) * 8; c8 < v.n_pad; c8 += 256) {
     const long long el = (long long)row * v.n_pad + c8;
     __align__(16) T y[8];
-    rows_sum8(m, w, el, y);
-    if (master)
+    rows_sum8<EACH>(m, w, el, y);
 #pragma unroll
-      for (int e = 0; e < 8; e += 16 / sizeof(T))
-        *reinterpret_cast<uint4*>(m + (el + e) * sizeof(T)) = *reinterpret_cast<const uint4*>(y + e);
-    if (nsplit) {
-      float f[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) f[e] = (float)y[e];
-      write_planes8(arena, v.planes + blocked_offset(row, c8, v.n_pad), v.plane_stride, nsplit, f);
-    }
+    for (int e = 0; e < 8; e += 16 / sizeof(T))
+      *reinterpret_cast<uint4*>(m + (el + e) * sizeof(T)) = *reinterpret_cast<const uint4*>(y + e);
   }
 }
 
@@ -434,12 +453,15 @@ void launch_split_planes(SlotViews views, int n_sub, int max_rows, uint8_t* aren
   else split_planes_kernel<float><<<g, 64, 0, s>>>(views, arena, nsplit);
 }
 
-void launch_rows_sum(SlotViews y, const RowTerms& w, int master, int nsplit, int n_sub, int max_rows, uint8_t* arena,
-                     bool f64, cudaStream_t s) {
+void launch_rows_sum(SlotViews y, const RowTerms& w, bool one_by_one, int n_sub, int max_rows, uint8_t* arena, bool f64,
+                     cudaStream_t s) {
   if (n_sub <= 0 || max_rows <= 0) return;
   dim3 g((max_rows + 7) / 8, n_sub);
-  if (f64) rows_sum_kernel<double><<<g, 256, 0, s>>>(y, w, 1, 0, arena);
-  else rows_sum_kernel<float><<<g, 256, 0, s>>>(y, w, master, nsplit, arena);
+  auto go = [&](auto kernel) { kernel<<<g, 256, 0, s>>>(y, w, arena); };
+  if (f64 && one_by_one) go(rows_sum_kernel<double, true>);
+  else if (f64) go(rows_sum_kernel<double, false>);
+  else if (one_by_one) go(rows_sum_kernel<float, true>);
+  else go(rows_sum_kernel<float, false>);
 }
 
 void launch_affine_planes(SlotViews in, SlotViews out1, double a1, double b1, int master1, int nsplit1,

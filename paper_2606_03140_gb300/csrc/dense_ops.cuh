@@ -54,8 +54,8 @@ struct RowTerms {
   double a[4];
   int n;
 };
-void launch_rows_sum(SlotViews y, const RowTerms& w, int master, int nsplit, int n_sub, int max_rows, uint8_t* arena,
-                     bool f64, cudaStream_t s);
+void launch_rows_sum(SlotViews y, const RowTerms& w, bool one_by_one, int n_sub, int max_rows, uint8_t* arena, bool f64,
+                     cudaStream_t s);
 void launch_affine_planes(SlotViews in, SlotViews out1, double a1, double b1, int master1, int nsplit1,
                           SlotViews out2, double a2, double b2, int master2, int nsplit2, int kind,
                           const double* bounds, int n_sub, int max_rows, uint8_t* arena, bool f64, cudaStream_t s);

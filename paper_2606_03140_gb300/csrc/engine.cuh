@@ -35,6 +35,7 @@ enum SlotId : int {
   kdT2, kdDt,          // core rows of t = s (I - 2F) (second-order mu term): Z_c t, 2 Z_c t Z
   kdT3, kdDu,          // core rows of the third-order term u: Z_c u, 2 Z_c u Z
   kdT4, kdDw,          // core rows of the fourth-order term w: Z_c w, 2 Z_c w Z
+  kT2s, kT2t, kT2u, kT2w,   // their rows Z_c X h~
   kNumSlots
 };
 
@@ -70,6 +71,9 @@ enum OpId : int {
   OP_F_UP_0, OP_F_UP_1, OP_F_FIN, OP_F_S,
   // core rows of F into the response slots (dT1 = Z_c F)
   OP_F_FT1_0, OP_F_FT1_1,
+  // W of the terms: T2 = dT h~, W = 2 T2 Z into the terms' D rows
+  OP_F_T2S, OP_F_T2T, OP_F_T2U, OP_F_T2W,
+  OP_F_WS0, OP_F_WT0, OP_F_WU0, OP_F_WW0, OP_F_WS1, OP_F_WT1, OP_F_WU1, OP_F_WW1,
   // second-order mu term: t = s - 2 s F (kR1 copy 1), its core rows (kdT2, kdDt)
   OP_F_T, OP_F_TT1_0, OP_F_TT1_1, OP_F_DT0, OP_F_DT1,
   // mu shift at a saved doubling stage: U' = U Q + tau Q, Q ~ (I + tau U)^-1 (U in kY0), into kX
