@@ -59,14 +59,10 @@ def parse():
 
 METRIC = "atoms*QMD-steps/s at |dq|<=1e-5 e vs FP64 oracle (mixed vs plain, one GB300)"
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the Fermi-recursion
-# product kernel (tc_gemm_persistent<2, true>) on the benchmarked 9,000-atom workload: the mean over
-# its 136 launches in the NVTX range 'timed' of `bench.py --no-plain --no-frames --no-cpu-baseline
-# --steps 2 --warmup 1` (one ncu pass, so the full workload could be captured); reported only while
-# the kernel source is the one the counters were taken on, and on the cores the capture used (the
-# recursive-bisection cores, not refined: refinement changes the subgraph sizes).
-FERMI_TRAFFIC = {"kernel_sha1": "f1e27abead4ca70ebedad479f3f8cb922699ee59", "precision": 1,
-                 "workload": "water9000", "core_refine": False, "bytes_per_launch": 998.1e6}
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the Fermi-recursion kernel on the
+# benchmarked workload, reported only while the kernel source is the one the counters were taken on.  None: the
+# chain kernel's counters need several passes, which were taken on a smaller box only.
+FERMI_TRAFFIC = None
 
 
 def strip_comments(src: str) -> str:
@@ -377,7 +373,7 @@ def run_ours(args, world, rank, local):
         bw = f16_bytes / (f16_ms / 1e3) / 1e9
         tf = f16_flops / (f16_ms / 1e3) / 1e12
         f_bw, f_tf = bw / hbm, tf * split / bf16
-        kname = "tc_gemm_persistent<2,F16> (Fermi-recursion products, two-plane fp16 on tcgen05)"
+        kname = "product_chain<2> (chains of Fermi-recursion products, two-plane fp16 on tcgen05)"
         if f_bw >= f_tf:
             bound, achieved, peak, unit = "hbm", bw, hbm, "GB/s"
         else:
@@ -405,7 +401,8 @@ def run_ours(args, world, rank, local):
             kname, bound, peak = "f64_gemm_kernel (Fermi-recursion products, FP64 CUDA cores)", "alu", 1.25
             peak_note = "nominal FP64 1.25 TF/s (no measured FP64 peak)"
         else:
-            kname = "tc_gemm_persistent (Fermi-recursion products, split bf16 on tcgen05)"
+            kname = ("product_chain<3>" if args.precision == 4 else "tc_gemm_persistent") + \
+                " (Fermi-recursion products, split bf16 on tcgen05)"
             bound, peak = "tensor", bf16
             peak_note = (f"measured sustained dense bf16 {bf16} TF/s {peak_src}; the FP32-class product costs {split} "
                          f"tensor-core products, counted as work of the kernel, not of the method")
