@@ -188,7 +188,8 @@ sedacs_status sedacs_charges(sedacs_ctx* ctx, double* q);
 /* Energies of the last density call: e[0] band Tr[D H0], e[1] Coulomb 1/2 (2q - n)^T gamma n,
  * e[2] repulsion, e[3] total shadow potential (Hartree). */
 sedacs_status sedacs_energy(sedacs_ctx* ctx, double* e);
-/* ---- a10: forces of the last density call at fixed n (Eq. NEQ), Hartree/Angstrom [N][3]. */
+/* ---- a10: forces of the last density call at fixed n (Eq. NEQ), Hartree/Angstrom [N][3].  Here and in the charge
+ * response the subgraphs have to be those of that call; after others have been set the numbers mean nothing. */
 sedacs_status sedacs_forces(sedacs_ctx* ctx, double* F);
 /* Density graph of the last density call: sizes, then rows (core atom I: G^D_IJ over its subgraph). */
 sedacs_status sedacs_density_graph_size(sedacs_ctx* ctx, int64_t* nnz);

@@ -313,6 +313,7 @@ sedacs_status prepare_geometry(sedacs_ctx* ctx) {
   if (ctx->geom_valid) return SEDACS_OK;
   const int N = ctx->N;
   cudaStream_t s = ctx->stream;
+  ctx->core_tab_valid = false;
   CUCHK(grow(&ctx->d_pptr, &ctx->rows_cap, (long long)N + 1) == cudaSuccess ? cudaSuccess : cudaErrorMemoryAllocation);
   long long pn = 0;
   // pair list of the Slater-Koster blocks: FP32 distance test (a pair at the cutoff carries a
@@ -711,6 +712,7 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   Layout& L = ctx->lay;
   L = Layout();
   L.n_sub = P;
+  ctx->core_tab_valid = false;
   const long long tot_rows = ctx->sub_ptr_h[P];
   ctx->stage_host.clear();              // (an earlier rebuild may have stopped half way)
   ctx->stage_recs.clear();
@@ -1102,6 +1104,21 @@ void back_transform(sedacs_ctx* ctx, bool with_w) {
     run_op(ctx, OP_T2, ns, ns);                                                          // T2 = T1 h~
     run_op(ctx, z == 0 ? OP_WC0 : OP_WC1, ns, 0);                                        // W_c = 2 T2 Z
   }
+}
+
+// Tables of the passes over core rows (launch_observables), for the current subgraphs and pair list.  Those
+// passes take offsets from the tables, so whoever launches one calls this first: the subgraphs may have
+// been replaced since the density.
+sedacs_status core_tables(sedacs_ctx* ctx) {
+  if (ctx->core_tab_valid) return SEDACS_OK;
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_tab), sizeof(int4) * std::max(1, ctx->n_core_total)));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_pair_orb), sizeof(int) * std::max(1LL, ctx->pnnz)));
+  launch_pair_orbs(ctx->model, ctx->d_species, ctx->d_sub_ptr, ctx->d_orb_off, ctx->part.perm, ctx->d_core_sub,
+                   ctx->d_core_local, ctx->n_core_total, ctx->d_pptr, ctx->d_pcol, ctx->d_loc, ctx->N, ctx->d_n_pad,
+                   ctx->d_core_tab, ctx->d_pair_orb, ctx->stream);
+  ctx->launches += 1;
+  ctx->core_tab_valid = true;
+  return SEDACS_OK;
 }
 
 // Populations of n matrices' core rows.
@@ -1731,15 +1748,8 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
   gather_hs(ctx);
   phase_end(ctx, 0, 2);
   phase_begin(ctx, 0);
-  if (!ctx->z_valid) {                  // new pairs or subgraphs
-    CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_tab), sizeof(int4) * std::max(1, ctx->n_core_total)));
-    CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_pair_orb), sizeof(int) * std::max(1LL, ctx->pnnz)));
-    launch_pair_orbs(ctx->model, ctx->d_species, ctx->d_sub_ptr, ctx->d_orb_off, ctx->part.perm, ctx->d_core_sub,
-                     ctx->d_core_local, ctx->n_core_total, ctx->d_pptr, ctx->d_pcol, ctx->d_loc, ctx->N, ctx->d_n_pad,
-                     ctx->d_core_tab, ctx->d_pair_orb, s);
-    ctx->launches += 1;
-    compute_z(ctx);
-  }
+  STCHK(core_tables(ctx));
+  if (!ctx->z_valid) compute_z(ctx);
   compute_ht(ctx);                      // h's planes were written by gather_hs
   CUCHK(cudaStreamSynchronize(s));
   ctx->ht_stale = false;
@@ -1795,7 +1805,10 @@ sedacs_status forces_core(sedacs_ctx* ctx) {
   if (!ctx->have_density) { ctx->err = "no density: call sedacs_subgraph_density first"; return SEDACS_EINVAL; }
   cudaStream_t s = ctx->stream;
   phase_begin(ctx, 0);
-  if (!ctx->du_ready) observe(ctx, true);   // else done with the density
+  if (!ctx->du_ready) {                     // else done with the density
+    STCHK(core_tables(ctx));
+    observe(ctx, true);
+  }
   ctx->du_ready = false;
   coul_a_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_q, ctx->d_n, ctx->d_tmp, ctx->N);
   CUCHK(ctx->ew.gradient(ctx->d_tmp, ctx->d_n, ctx->d_F, s, ctx->ew_tag));
@@ -1980,6 +1993,7 @@ sedacs_status response_fermi(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
 
 sedacs_status response_core(sedacs_ctx* ctx, const double* d_v, double* d_dq) {
   if (!ctx->have_density) { ctx->err = "no density: call sedacs_subgraph_density first"; return SEDACS_EINVAL; }
+  STCHK(core_tables(ctx));
   return ctx->prm.Te > 0.0 ? response_fermi(ctx, d_v, d_dq) : response_sp2(ctx, d_v, d_dq);
 }
 

@@ -202,8 +202,9 @@ struct sedacs_ctx {
   std::vector<long long> sub_ptr_h;
   int *d_orb_off = nullptr, *d_n_orb = nullptr;   // orbital offsets; orbitals per subgraph, then per core
   int* d_gd_len = nullptr;                          // density-graph row lengths
-  int4* d_core_tab = nullptr;     // tables of the passes over core rows (with z_valid)
+  int4* d_core_tab = nullptr;     // tables of the passes over core rows, see core_tables
   int* d_pair_orb = nullptr;
+  bool core_tab_valid = false;    // they are those of the current subgraphs and pairs
   int *d_sub_of_row = nullptr, *d_core_sub = nullptr, *d_core_local = nullptr, *d_loc = nullptr;
   long long loc_cap = 0, rows_cap = 0;
   int n_core_total = 0;

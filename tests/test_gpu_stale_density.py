@@ -1,0 +1,83 @@
+"""Calls on a density whose subgraphs have been rebuilt or replaced since.
+
+Rebuilt but the same: forces are those of the density.  Replaced by fewer: the rows in memory are not those of the
+new subgraphs, so the numbers mean nothing, but every index has to come from the new subgraphs (the tables of the core
+atoms and pairs once stayed those of the density and named subgraphs that were gone); the context stays usable, and its
+next density and forces are a new context's.  Both sides run the same kernels on the same inputs, so they differ by
+the FP64 atomics of the force scatter alone: 1e-10 Ha/A stands for 1e-16 of terms of order 1 over a few hundred pairs.
+"""
+import numpy as np
+import pytest
+
+from paper_2606_03140_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+MU = {300.0: float("nan"), 0.0: -0.03}                # Te = 0 takes it as given: in the gap of every partition here
+
+
+@pytest.fixture(scope="module")
+def S():
+    from paper_2606_03140_gb300 import sedacs
+    return sedacs
+
+
+def _cores(n, parts):
+    cut = np.linspace(0, n, parts + 1).astype(int)
+    return [np.arange(a, b, dtype=np.int32) for a, b in zip(cut[:-1], cut[1:])]
+
+
+def _ctx(S, s, precision, Te, cores):
+    ctx = S.sedacs_create(s.species, s.box, I.default_model(), S.sedacs_default_params(precision=precision, Te=Te))
+    S.sedacs_graph_build(ctx, np.ascontiguousarray(s.R))
+    S.sedacs_set_cores(ctx, cores)
+    return ctx
+
+
+def _density_forces(S, ctx, s, n, mu):
+    _, q, _, _ = S.sedacs_subgraph_density(ctx, np.ascontiguousarray(s.R), n, mu)
+    return q, S.sedacs_forces(ctx, s.n_atoms)
+
+
+@pytest.mark.parametrize("precision,Te", [(0, 300.0), (1, 300.0), (1, 0.0)])
+def test_same_subgraphs_rebuilt(S, precision, Te):
+    s = I.workload("water96")
+    n = np.ascontiguousarray(I.random_charges(96, 3, 0.05))
+    mu = MU[Te]
+    ctx = _ctx(S, s, precision, Te, _cores(96, 9))
+    try:
+        _, F = _density_forces(S, ctx, s, n, mu)
+        S.sedacs_subgraph_density(ctx, np.ascontiguousarray(s.R), n, mu)
+        S.sedacs_update_halos(ctx)
+        assert np.max(np.abs(S.sedacs_forces(ctx, 96) - F)) < 1e-10
+    finally:
+        S.sedacs_destroy(ctx)
+
+
+@pytest.mark.parametrize("call", ["forces", "energy", "response"])
+@pytest.mark.parametrize("precision,Te", [(0, 300.0), (1, 300.0), (1, 0.0)])
+def test_subgraphs_replaced(S, precision, Te, call):
+    s = I.workload("water96")
+    n = np.ascontiguousarray(I.random_charges(96, 3, 0.05))
+    mu = MU[Te]
+    ctx = _ctx(S, s, precision, Te, _cores(96, 16))
+    ref = _ctx(S, s, precision, Te, _cores(96, 3))
+    try:
+        S.sedacs_subgraph_density(ctx, np.ascontiguousarray(s.R), n, mu)
+        S.sedacs_set_cores(ctx, _cores(96, 3))
+        try:
+            if call == "forces":
+                S.sedacs_forces(ctx, 96)
+            elif call == "energy":
+                S.sedacs_energy(ctx)
+            else:
+                S.sedacs_charge_response(ctx, np.ascontiguousarray(n))
+        except S.SedacsError as e:
+            assert e.status == 6                      # SEDACS_ENUMERIC: the numbers may be anything
+        q, F = _density_forces(S, ctx, s, n, mu)
+        q2, F2 = _density_forces(S, ref, s, n, mu)
+        assert np.max(np.abs(q - q2)) < 1e-10
+        assert np.max(np.abs(F - F2)) < 1e-10
+    finally:
+        S.sedacs_destroy(ctx)
+        S.sedacs_destroy(ref)
