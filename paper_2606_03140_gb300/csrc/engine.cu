@@ -830,19 +830,18 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_sub), sizeof(int) * N));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_local), sizeof(int) * N));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_len), sizeof(int) * N));
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_ptr), sizeof(long long) * (N + 1)));
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gdl_ptr), sizeof(long long) * (N + 1)));
   launch_sub_tables(ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->part.leaves_d, ctx->d_loc, ctx->d_sub_of_row, ctx->d_core_sub,
                     ctx->d_core_local, ctx->d_gd_len, N, P, s);
-  launch_scan(ctx->d_gd_len, N, ctx->d_gd_ptr, s);
+  launch_scan(ctx->d_gd_len, N, ctx->d_gdl_ptr, s);
   CUCHK(cudaGetLastError());
   ctx->n_core_total = 0;
-  ctx->gd_nnz = 0;
+  ctx->gdl_nnz = 0;
   for (int i = 0; i < P; ++i) {
     ctx->n_core_total += ncore[i];
-    ctx->gd_nnz += (long long)ncore[i] * L.n_atoms[i];
+    ctx->gdl_nnz += (long long)ncore[i] * L.n_atoms[i];
   }
-  CUCHK(grow(&ctx->d_gd_col, &ctx->gd_cap, ctx->gd_nnz + 1) == cudaSuccess ? cudaSuccess : cudaErrorMemoryAllocation);
-  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_val), sizeof(double) * ctx->gd_cap));
+  ctx->gdl_new = true;
   // GEMM tables
   // S^-1/2 in deviation form: Y = I + E_y (kY*), Z = I + E_z (kZ*), T = I + E_t (kT);
   // only products of the small deviations go through the tensor cores.
@@ -1143,6 +1142,19 @@ void observe(sedacs_ctx* ctx, bool with_forces) {
                      ctx->f64, s);
   charges_kernel<<<nblk(ctx->N, 128), 128, 0, s>>>(ctx->d_pop, ctx->d_species, ctx->d_zval, ctx->d_q, ctx->N);
   ctx->launches += 2;
+}
+
+// Room for the density graph of the current subgraphs, whose rows they determine; the one of the last density
+// goes, which a graph build may have used until here, whatever subgraphs were set in between.
+sedacs_status density_graph_rows(sedacs_ctx* ctx) {
+  if (!ctx->gdl_new) return SEDACS_OK;
+  ctx->have_gd = false;
+  CUCHK(grow(&ctx->d_gd_col, &ctx->gd_cap, ctx->gdl_nnz + 1) == cudaSuccess ? cudaSuccess : cudaErrorMemoryAllocation);
+  CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_gd_val), sizeof(double) * ctx->gd_cap));
+  std::swap(ctx->d_gd_ptr, ctx->d_gdl_ptr);
+  ctx->gd_nnz = ctx->gdl_nnz;
+  ctx->gdl_new = false;
+  return SEDACS_OK;
 }
 
 // ---- finite-temperature Fermi operator (Eq. 2) and the chemical potential ------------------------
@@ -1768,6 +1780,7 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
   const bool fused = ctx->fuse_forces;
   observe(ctx, fused);
   ctx->du_ready = fused;
+  STCHK(density_graph_rows(ctx));
   launch_gd(ctx->model, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_species, ctx->part.perm,
             ctx->d_core_sub, ctx->d_core_local, ctx->n_core_total, ctx->arena, ctx->f64, ctx->d_dcoff, ctx->d_n_pad,
             ctx->d_gd_ptr, ctx->d_gd_col, ctx->d_gd_val, s);
@@ -2229,7 +2242,7 @@ void sedacs_destroy(sedacs_ctx* ctx) {
   void* ptrs[] = {ctx->d_err, ctx->d_species, ctx->d_R, ctx->d_n, ctx->d_q, ctx->d_V, ctx->d_pop, ctx->d_eband,
                   ctx->d_dU, ctx->d_F, ctx->d_erep, ctx->d_tmp, ctx->d_tmp2, ctx->d_scal, ctx->d_vel, ctx->d_hist,
                   ctx->d_mass, ctx->d_zval, ctx->d_vec, ctx->d_row_ptr, ctx->d_col, ctx->d_pptr, ctx->d_pcol,
-                  ctx->d_h0b, ctx->d_sb, ctx->d_gd_ptr, ctx->d_gd_col, ctx->d_gd_val, ctx->d_xgd_ptr, ctx->d_xgd_col,
+                  ctx->d_h0b, ctx->d_sb, ctx->d_gd_ptr, ctx->d_gdl_ptr, ctx->d_gd_col, ctx->d_gd_val, ctx->d_xgd_ptr, ctx->d_xgd_col,
                   ctx->d_xgd_val, ctx->d_sub_ptr, ctx->d_sub_atoms, ctx->d_orb_off, ctx->d_n_orb, ctx->d_sub_of_row,
                   ctx->d_core_sub, ctx->d_core_local, ctx->d_core_tab, ctx->d_pair_orb, ctx->d_loc, ctx->d_gd_len,
                   ctx->d_tables, ctx->arena, ctx->d_glo, ctx->d_ghi, ctx->d_bounds, ctx->d_slots, ctx->d_sp2,

@@ -187,6 +187,9 @@ struct sedacs_ctx {
   int* d_gd_col = nullptr;
   double* d_gd_val = nullptr;
   long long gd_cap = 0, gd_nnz = 0;
+  long long* d_gdl_ptr = nullptr;      // row pointers of the current subgraphs' density graph until a density has them
+  long long gdl_nnz = 0;
+  bool gdl_new = false;
   bool have_gd = false;
   // external density graph uploaded by the caller
   long long* d_xgd_ptr = nullptr;

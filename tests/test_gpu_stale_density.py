@@ -81,3 +81,25 @@ def test_subgraphs_replaced(S, precision, Te, call):
     finally:
         S.sedacs_destroy(ctx)
         S.sedacs_destroy(ref)
+
+
+@pytest.mark.parametrize("parts", [3, 40])             # more entries than the density graph has, and fewer
+def test_density_graph_outlives_its_subgraphs(S, parts):
+    s = I.workload("water96")
+    R = np.ascontiguousarray(s.R)
+    n = np.ascontiguousarray(I.random_charges(96, 3, 0.05))
+    ctx = _ctx(S, s, 1, 300.0, _cores(96, 16))
+    ref = _ctx(S, s, 1, 300.0, _cores(96, 16))
+    try:
+        S.sedacs_subgraph_density(ctx, R, n)
+        gd = S.sedacs_density_graph_get(ctx, 96)
+        S.sedacs_set_cores(ctx, _cores(96, parts))
+        for a, b in zip(S.sedacs_density_graph_get(ctx, 96), gd):
+            assert np.array_equal(a, b)
+        nnz = S.sedacs_graph_build(ctx, R, use_prev_D=True)
+        nnz_ref = S.sedacs_graph_build(ref, R, gd=gd)
+        for a, b in zip(S.sedacs_graph_get(ctx, 96, nnz), S.sedacs_graph_get(ref, 96, nnz_ref)):
+            assert np.array_equal(a, b)
+    finally:
+        S.sedacs_destroy(ctx)
+        S.sedacs_destroy(ref)
