@@ -61,7 +61,7 @@ __global__ void embed_kernel(const double* y, const int* species, const float* P
 // The per-atom work is a sum over about 30 edges with ten loads each (latency) and two 64 x 64 mixes, so a
 // block gathers its atoms' sums warp by warp into shared memory and mixes them from there, with both
 // matrices in shared memory: one launch and one pass over the activations per layer and direction.
-// Measured (GB300, 9,000 atoms, 27 edges each), an application and a parameter gradient: 0.82 ms in all, against
+// Measured (GB300, 9,000 atoms, 27 edges each), an application and a parameter gradient: 0.83 ms in all, against
 // 2.44 ms with one kernel per step, of which 1.75 ms went to the filter gradient on 141 blocks of two warps and
 // 0.35 ms to mixes that read the matrices by columns.
 constexpr int kTile = 32, kWarps = 8;
@@ -135,7 +135,8 @@ __device__ __forceinline__ void mix8(const float* M, const float* x, float (&acc
   }
 }
 
-// One layer: a_i = sum_j phi(r_ij) * h_j (kept for the backward pass), out = h + A a + B h.
+// One layer: a_i = sum_j phi(r_ij) * h_j (kept for the backward pass), out = h + A a + B h.  The two mixes are summed
+// from zero and h comes last: they are a tenth of h, and 128 sums on top of h would round at its size each.
 __global__ void __launch_bounds__(256) layer_fwd_kernel(const float* h, const float* P, int l, const long long* row_ptr,
                                                         const int* col, const float* ebas, int N, float* a, float* out) {
   extern __shared__ float sm[];
@@ -164,16 +165,16 @@ __global__ void __launch_bounds__(256) layer_fwd_kernel(const float* h, const fl
   }
   __syncthreads();
   const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
-  float acc[8];
+  float ma[8], mb[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = sh[(8 * g + q) * W + c];
-  mix8(sA, sa, acc);
-  mix8(sB, sh, acc);
+  for (int q = 0; q < 8; ++q) ma[q] = mb[q] = 0.f;
+  mix8(sA, sa, ma);
+  mix8(sB, sh, mb);
   for (int q = 0; q < 8; ++q)
-    if (i0 + 8 * g + q < N) out[(long long)(i0 + 8 * g + q) * W + c] = acc[q];
+    if (i0 + 8 * g + q < N) out[(long long)(i0 + 8 * g + q) * W + c] = sh[(8 * g + q) * W + c] + (ma[q] + mb[q]);
 }
 
-// Backward through the mixes of a layer: ga = A^T gh, base = gh + B^T gh, and this block's part of
+// Backward through the mixes of a layer: ga = A^T gh, base = gh + B^T gh (gh last, as h above), and this block's part of
 // dA = sum gh a^T, dB = sum gh h^T (part[blk][0 .. W W) and [W W .. 2 W W)).
 __global__ void __launch_bounds__(256) mix_bwd_kernel(const float* gh, const float* a, const float* h, const float* P, int l,
                                                       int N, float* ga, float* base, float* part) {
@@ -193,16 +194,13 @@ __global__ void __launch_bounds__(256) mix_bwd_kernel(const float* gh, const flo
   const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
   float acc[8], bas[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    acc[q] = 0.f;
-    bas[q] = sg[(8 * g + q) * W + c];
-  }
+  for (int q = 0; q < 8; ++q) acc[q] = bas[q] = 0.f;
   mix8(sA, sg, acc);
   mix8(sB, sg, bas);
   for (int q = 0; q < 8; ++q)
     if (8 * g + q < n) {
       ga[(long long)(i0 + 8 * g + q) * W + c] = acc[q];
-      base[(long long)(i0 + 8 * g + q) * W + c] = bas[q];
+      base[(long long)(i0 + 8 * g + q) * W + c] = sg[(8 * g + q) * W + c] + bas[q];
     }
   // outer products: thread (row block of four channels, column block of four) over both matrices
   const int r4 = (threadIdx.x >> 4) * 4, k4 = (threadIdx.x & 15) * 4;
