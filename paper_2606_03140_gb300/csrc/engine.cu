@@ -757,7 +757,9 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
     ctx->sum_n3 += (double)L.n_real[i] * L.n_real[i] * L.n_real[i];
     ctx->sum_tri += 0.5 * (double)L.n_real[i] * (L.n_real[i] + 1);
   }
-  // arena slots
+  // arena slots; the rows of the mu step's terms (kT2s ..) lie in square slots whose matrices are done with by then,
+  // each at least as large (m_pad <= n_pad)
+  const int rows_in[4] = {kT, kY0, kY1, kP};
   const int esz = ctx->f64 ? 8 : 4;
   const bool planes = !ctx->f64;
   long long off = 0;
@@ -771,8 +773,9 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
     S.master_bytes = (el * esz + 1023) / 1024 * 1024;
     S.plane_stride = el * 2;
     S.copy_stride = S.master_bytes + (S.planes ? (3 * el * 2 + 1023) / 1024 * 1024 : 0);
-    S.base = off;
-    off += S.copy_stride * S.copies;
+    const bool inside = k >= kT2s && k <= kT2w;
+    S.base = inside ? ctx->slot[rows_in[k - kT2s]].base : off;
+    if (!inside) off += S.copy_stride * S.copies;
   }
   if ((size_t)off > ctx->arena_cap) {
     if (ctx->arena) cudaFree(ctx->arena);

@@ -35,7 +35,7 @@ enum SlotId : int {
   kdT2, kdDt,          // core rows of t = s (I - 2F) (second-order mu term): Z_c t, 2 Z_c t Z
   kdT3, kdDu,          // core rows of the third-order term u: Z_c u, 2 Z_c u Z
   kdT4, kdDw,          // core rows of the fourth-order term w: Z_c w, 2 Z_c w Z
-  kT2s, kT2t, kT2u, kT2w,   // their rows Z_c X h~
+  kT2s, kT2t, kT2u, kT2w,   // their rows Z_c X h~, in the place of kT, kY0, kY1 and kP (see rebuild_layout)
   kNumSlots
 };
 
