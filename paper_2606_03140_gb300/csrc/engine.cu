@@ -230,6 +230,7 @@ void dev_dot_into(sedacs_ctx* ctx, const double* a, const double* b, double* out
     cudaError_t e__ = (x);                                                        \
     if (e__ != cudaSuccess) {                                                     \
       ctx->err = std::string(#x) + ": " + cudaGetErrorString(e__);                 \
+      cudaGetLastError();   /* reported here, not by the next call */              \
       return e__ == cudaErrorMemoryAllocation ? SEDACS_ENOMEM : SEDACS_ECUDA;       \
     }                                                                             \
   } while (0)
@@ -325,9 +326,12 @@ sedacs_status prepare_geometry(sedacs_ctx* ctx) {
   if (pn * 16 > ctx->blk_cap) {
     if (ctx->d_h0b) cudaFree(ctx->d_h0b);
     if (ctx->d_sb) cudaFree(ctx->d_sb);
-    ctx->blk_cap = pn * 16 + pn * 4 + 1024;
-    CUCHK(cudaMalloc(&ctx->d_h0b, esz * ctx->blk_cap));
-    CUCHK(cudaMalloc(&ctx->d_sb, esz * ctx->blk_cap));
+    ctx->d_h0b = ctx->d_sb = nullptr;
+    ctx->blk_cap = 0;
+    const long long want = pn * 16 + pn * 4 + 1024;
+    CUCHK(cudaMalloc(&ctx->d_h0b, esz * want));
+    CUCHK(cudaMalloc(&ctx->d_sb, esz * want));
+    ctx->blk_cap = want;
   }
   SkGeom g;
   for (int a = 0; a < 3; ++a) {
@@ -712,7 +716,7 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   Layout& L = ctx->lay;
   L = Layout();
   L.n_sub = P;
-  ctx->core_tab_valid = false;
+  ctx->core_tab_valid = ctx->layout_valid = false;
   const long long tot_rows = ctx->sub_ptr_h[P];
   ctx->stage_host.clear();              // (an earlier rebuild may have stopped half way)
   ctx->stage_recs.clear();
@@ -780,6 +784,7 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   if ((size_t)off > ctx->arena_cap) {
     if (ctx->arena) cudaFree(ctx->arena);
     ctx->arena = nullptr;
+    ctx->arena_cap = 0;
     const size_t want = (size_t)off + (size_t)off / 4;
     CUCHK(cudaMalloc(&ctx->arena, want));
     ctx->arena_cap = want;
@@ -887,7 +892,7 @@ sedacs_status rebuild_layout(sedacs_ctx* ctx) {
   CUCHK(cudaGetLastError());
   STCHK(flush_staged(ctx));
   CUCHK(cudaGetLastError());
-  ctx->have_subs = true;
+  ctx->have_subs = ctx->layout_valid = true;
   ctx->z_valid = false;
   ctx->sp2_iters_h.assign(P, 0);
   return SEDACS_OK;
@@ -1108,10 +1113,18 @@ void back_transform(sedacs_ctx* ctx, bool with_w) {
   }
 }
 
+// A rebuild that did not fit leaves no arena or tables to work on (halos and lists stay readable).
+sedacs_status need_layout(sedacs_ctx* ctx) {
+  if (ctx->layout_valid) return SEDACS_OK;
+  ctx->err = "the current subgraphs did not fit the device";
+  return SEDACS_EINVAL;
+}
+
 // Tables of the passes over core rows (launch_observables), for the current subgraphs and pair list.  Those
 // passes take offsets from the tables, so whoever launches one calls this first: the subgraphs may have
 // been replaced since the density.
 sedacs_status core_tables(sedacs_ctx* ctx) {
+  STCHK(need_layout(ctx));
   if (ctx->core_tab_valid) return SEDACS_OK;
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_core_tab), sizeof(int4) * std::max(1, ctx->n_core_total)));
   CUCHK(ensure(ctx, reinterpret_cast<void**>(&ctx->d_pair_orb), sizeof(int) * std::max(1LL, ctx->pnnz)));
@@ -1752,6 +1765,7 @@ sedacs_status density_core(sedacs_ctx* ctx, double* mu_io) {
     ctx->err = "Te = 0 (T -> 0 SP2) needs a chemical potential";
     return SEDACS_EINVAL;
   }
+  STCHK(need_layout(ctx));
   cudaStream_t s = ctx->stream;
   STCHK(prepare_geometry(ctx));
   phase_begin(ctx, 0);
@@ -2589,6 +2603,7 @@ sedacs_status sedacs_density_graph_get(sedacs_ctx* ctx, int64_t* ptr, int32_t* c
 sedacs_status sedacs_subgraph_matrix(sedacs_ctx* ctx, int32_t part, int32_t which, double* out, int32_t* n,
                                      int32_t* n_core_orb) {
   if (!ctx || !ctx->have_density || part < 0 || part >= ctx->lay.n_sub || which < 0 || which > 5) return SEDACS_EINVAL;
+  STCHK(need_layout(ctx));
   const int nr = ctx->lay.n_real[part], nc = ctx->lay.n_core_orb[part];
   if (n) *n = nr;
   if (n_core_orb) *n_core_orb = nc;

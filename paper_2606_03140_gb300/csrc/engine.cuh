@@ -207,6 +207,7 @@ struct sedacs_ctx {
   int* d_gd_len = nullptr;                          // density-graph row lengths
   int4* d_core_tab = nullptr;     // tables of the passes over core rows, see core_tables
   int* d_pair_orb = nullptr;
+  bool layout_valid = false;      // the last rebuild of the arena and its tables went through
   bool core_tab_valid = false;    // they are those of the current subgraphs and pairs
   int *d_sub_of_row = nullptr, *d_core_sub = nullptr, *d_core_local = nullptr, *d_loc = nullptr;
   long long loc_cap = 0, rows_cap = 0;
