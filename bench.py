@@ -59,11 +59,6 @@ def parse():
 
 METRIC = "atoms*QMD-steps/s at |dq|<=1e-5 e vs FP64 oracle (mixed vs plain, one GB300)"
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the Fermi-recursion kernel on the
-# benchmarked workload, reported only while the kernel source is the one the counters were taken on.  None: the
-# chain kernel's counters need several passes, which were taken on a smaller box only.
-FERMI_TRAFFIC = None
-
 
 def strip_comments(src: str) -> str:
     """C/C++ source without comments and blank lines (string literals kept)."""
@@ -89,10 +84,10 @@ def strip_comments(src: str) -> str:
 
 
 def kernel_sha1() -> str:
-    """sha1 of the GEMM kernel's source (dense_gemm.cu, dense.cuh, common.cuh), comments stripped."""
+    """sha1 of the product kernels' source, comments stripped: a roofline line names the code it was measured on."""
     import hashlib
     h = hashlib.sha1()
-    for f in ("dense_gemm.cu", "dense.cuh", "common.cuh"):
+    for f in ("chain.cu", "chain.cuh", "dense_gemm.cu", "dense.cuh", "common.cuh"):
         with open(os.path.join(ROOT, "paper_2606_03140_gb300", "csrc", f), encoding="utf-8") as fh:
             h.update(strip_comments(fh.read()).encode())
     return h.hexdigest()
@@ -361,34 +356,30 @@ def run_ours(args, world, rank, local):
     split = {1: 3, 2: 3, 3: 1, 4: 6}.get(args.precision, 6)
     hbm = peaks.get("hbm_gbs", 6800.0)
     hbm_src = "of measured" if "hbm_gbs" in peaks else "of fallback"
-    traffic = None
-    if FERMI_TRAFFIC and kernel_sha1() == FERMI_TRAFFIC["kernel_sha1"] and args.precision == FERMI_TRAFFIC["precision"] \
-            and args.workload == FERMI_TRAFFIC["workload"] and args.refine_cores == FERMI_TRAFFIC["core_refine"]:
-        traffic = FERMI_TRAFFIC["bytes_per_launch"]
     if args.precision == 1 and f16_ms > 0:
-        # the dominant kernel: the products in two fp16 planes.  Roofline: its algorithmic bytes
+        # the dominant kernels: the products in two fp16 planes, most of them in the chains.  Roofline: their algorithmic bytes
         # (operands once, FP32 addends, output planes and master, over the upper triangles) against
-        # the measured HBM copy bandwidth, and its algorithmic flops (n^3 per symmetric product) x 3
+        # the measured HBM copy bandwidth, and their algorithmic flops (n^3 per symmetric product) x 3
         # tensor-core products against the measured bf16 rate; the larger fraction is the bound
         bw = f16_bytes / (f16_ms / 1e3) / 1e9
         tf = f16_flops / (f16_ms / 1e3) / 1e12
         f_bw, f_tf = bw / hbm, tf * split / bf16
-        kname = "product_chain<2> (chains of Fermi-recursion products, two-plane fp16 on tcgen05)"
+        kname = ("product_chain<2> (chains of about 60 products of the Fermi recursion, and G by itself) and "
+                 "tc_gemm_persistent<2,F16> (F and s, one product a launch), two-plane fp16 on tcgen05")
         if f_bw >= f_tf:
             bound, achieved, peak, unit = "hbm", bw, hbm, "GB/s"
         else:
             bound, achieved, peak, unit = "tensor", tf, bf16, "TFLOP/s"
         roof = {"kernel": kname, "bound": bound, "achieved": achieved, "peak": peak, "unit": unit,
-                "frac": achieved / peak, "traffic": traffic,
-                "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
-                "algorithmic_bytes_per_launch": f16_bytes / f16_launch,
+                "frac": achieved / peak, "algorithmic_bytes": f16_bytes, "algorithmic_flops": f16_flops,
+                "kernel_source_sha1": kernel_sha1(),
                 "hbm": {"achieved_gbs": bw, "peak_gbs": hbm, "frac": f_bw, "peak_note": f"STREAM copy {hbm_src}"},
                 "tensor": {"achieved_tflops": tf, "peak_tflops": bf16, "frac": tf / bf16,
                            "frac_with_split_products": f_tf, "split_products": split,
                            "peak_note": f"dense bf16 sustained {peak_src} (fp16 runs at the bf16 rate); the FP32-class "
                                         f"product costs {split} tensor-core products"},
                 "launches": f16_launch, "kernel_ms": f16_ms,
-                "work_note": "bytes: per launch, over the upper triangle of every subgraph (n (n+1)/2 elements), operands "
+                "work_note": "sums over all products of the launches; bytes: over the upper triangle of every subgraph (n (n+1)/2 elements), operands "
                              "read once (4 B an element in two fp16 planes; once when A = B), each FP32 addend (4 B), "
                              "output planes (4 B, 6 B in three bf16 planes), FP32 master (4 B) unless planes-only, second "
                              "output (4 B); flops: n^3 per symmetric product",
@@ -401,18 +392,17 @@ def run_ours(args, world, rank, local):
             kname, bound, peak = "f64_gemm_kernel (Fermi-recursion products, FP64 CUDA cores)", "alu", 1.25
             peak_note = "nominal FP64 1.25 TF/s (no measured FP64 peak)"
         else:
-            kname = ("product_chain<3>" if args.precision == 4 else "tc_gemm_persistent") + \
-                " (Fermi-recursion products, split bf16 on tcgen05)"
+            kname = ("product_chain<3> (chains of the Fermi recursion) and " if args.precision == 4 else "") + \
+                "tc_gemm_persistent (single Fermi products), split bf16 on tcgen05"
             bound, peak = "tensor", bf16
             peak_note = (f"measured sustained dense bf16 {bf16} TF/s {peak_src}; the FP32-class product costs {split} "
                          f"tensor-core products, counted as work of the kernel, not of the method")
         roof = {"kernel": kname, "bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": (achieved / peak) if achieved else None, "traffic": traffic,
-                "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
+                "frac": (achieved / peak) if achieved else None, "kernel_source_sha1": kernel_sha1(),
                 "split_products": split,
                 "tensor_frac_with_split_products": (achieved * split / peak) if achieved else None,
                 "peak_note": peak_note, "launches": k_launch, "kernel_ms": k_ms,
-                "work_note": "flops = sum over launches of sum_i n_i^3 (one symmetric product per subgraph, upper "
+                "work_note": "flops = sum over products of sum_i n_i^3 (one symmetric product per subgraph, upper "
                              "triangle, n_i the orbital count)"}
     plain = None
     if not args.no_plain and args.precision != 0 and rank == 0:
