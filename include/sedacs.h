@@ -270,8 +270,9 @@ sedacs_status sedacs_density_info(sedacs_ctx* ctx, double* info, int32_t n_info)
 sedacs_status sedacs_phase_times(sedacs_ctx* ctx, double* t, int64_t* launches);
 sedacs_status sedacs_reset_counters(sedacs_ctx* ctx);
 /* Per-launch timing of the Fermi-operator products (Te > 0: the tanh-doubling recursion; Te = 0:
- * the SP2 squares): on != 0 records CUDA events around every launch on the context stream (in
- * forms 1 and 4 a launch is a chain of products).
+ * the SP2 squares): on != 0 records CUDA events around every launch on the context stream.  In
+ * forms 1 and 4 most products of a pass are one launch (a chain), the others a launch each, so that
+ * only the sums over the launches have a meaning.
  * Returns the accumulated kernel time (ms), number of launches and the algorithmic work of
  * those launches in flops, counting a symmetric product of two n x n matrices (upper triangle)
  * as n^3 (n the orbital count of the subgraph), since the last reset. */

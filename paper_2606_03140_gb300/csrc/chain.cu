@@ -38,16 +38,15 @@ constexpr int kThreads = 32 * (kEW + 2);
 constexpr int kSlabBytes = 4096;                    // 32 rows x 64 columns of one plane
 constexpr int kReady = 16;                          // ring of tasks (more than can be in flight)
 
-// Operand ring: a unit holds the planes of one operand's 128 x 64 block (32 or 48 KB).  Slabs: for each
-// of the eight warp pairs kSlabs x 4 KB, first the landing place of the leading addend columns, then the
+// Operand ring: a unit holds the planes of one operand's 128 x 64 block (32 or 48 KB), two units a k-block.  Slabs:
+// for each of the eight warp pairs 4 KB, first the landing place of the leading addend columns, then the
 // source of the planes' bulk stores.
 template <int P>
 struct Cfg {
   static constexpr int kUnits = P == 2 ? 6 : 4;
   static constexpr int kUnitBytes = P * kBlkBytes;
-  static constexpr int kBars = (kUnits + 1) / 2;    // k-blocks in the ring, each with a full and an empty barrier
-  static constexpr int kSlabs = 1;
-  static constexpr int kSlabTotal = 8 * kSlabs * kSlabBytes;
+  static constexpr int kBars = kUnits / 2;          // k-blocks in the ring, each with a full and an empty barrier
+  static constexpr int kSlabTotal = 8 * kSlabBytes;
   static constexpr int kPre = 2;       // float4 columns of each addend landing in the slabs
   static constexpr int kSmem = kUnits * kUnitBytes + kSlabTotal + 1024 + 1024;
 };
@@ -271,18 +270,13 @@ __global__ void __launch_bounds__(kThreads, 1) product_chain(const __grid_consta
         const int s = k % C::kBars;
         uint8_t* ua = smem + (2 * k) % C::kUnits * C::kUnitBytes + my_dst;
         uint8_t* ub = smem + (2 * k + 1) % C::kUnits * C::kUnitBytes + my_dst;
-        // the unit of A was last used by k-block k - kBars
+        // both units were last used by k-block k - kBars
         if (k >= C::kBars) ok = mbar_wait(&empty[s], (uint32_t)((k / C::kBars - 1) & 1));
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         if (lane == 0) mbar_arrive_expect_tx(&full[s], one ? C::kUnitBytes : 2 * C::kUnitBytes);
         __syncwarp();
         copy(ua, A, t.tm, kb, &full[s]);
         if (one) continue;
-        if ((C::kUnits & 1) && k >= 2) {                // that of B by k-block k - 2
-          const int s2 = (k - 2) % C::kBars;
-          ok = mbar_wait(&empty[s2], (uint32_t)(((k - 2) / C::kBars) & 1));
-          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-        }
         copy(ub, B, t.tn, kb, &full[s]);
       }
       if (!ok) break;
@@ -349,12 +343,12 @@ __global__ void __launch_bounds__(kThreads, 1) product_chain(const __grid_consta
     // ---- epilogue warps: lane = row of the quadrant, 32 columns --------------------------------
     const int qd = warp & 3, cq = warp >> 2;
     const int pair = qd * 2 + (cq >> 1);
-    uint8_t* slab = slabs + pair * C::kSlabs * kSlabBytes;
+    uint8_t* slab = slabs + pair * kSlabBytes;
     const bool elect = (cq & 1) == 0 && lane == 0;      // issues the pair's copies
     const int row_sw = lane & 7, ch0 = (cq & 1) * 4;
     const uint32_t t_row = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cq * 32);
     // this warp's leading addend columns in the slab: kPre x 512 bytes of C1, then of C2
-    const float4* pre = reinterpret_cast<const float4*>(slab + (cq & 1) * (C::kSlabs * kSlabBytes / 2)) + lane;
+    const float4* pre = reinterpret_cast<const float4*>(slab + (cq & 1) * (kSlabBytes / 2)) + lane;
     int ti = 0, n_add = 0, n_meet = 0;
     auto meet = [&] {
       __syncwarp();
@@ -382,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_chain(const __grid_consta
           constexpr uint32_t nb = C::kPre * 512;
           mbar_arrive_expect_tx(&addf[pair], (has2 ? 4 : 2) * nb);
           for (int h = 0; h < 2; ++h) {                 // this warp and its neighbour (warp + 4)
-            uint8_t* d = slab + h * (C::kSlabs * kSlabBytes / 2);
+            uint8_t* d = slab + h * (kSlabBytes / 2);
             const long long at = mt + h * (4 * 8 * 512);
             bulk_g2s(d, p.arena + o.c1 + at, nb, &addf[pair]);
             if (has2) bulk_g2s(d + nb, p.arena + o.c2 + at, nb, &addf[pair]);
@@ -433,21 +427,17 @@ __global__ void __launch_bounds__(kThreads, 1) product_chain(const __grid_consta
       const long long pt = t.el * 2 + ((long long)t.tm * (t.n_pad >> 6) + t.tn * 2 + (cq >> 1)) * kBlkBytes + qd * kSlabBytes;
       auto put = [&](long long dst, bool first) {
 #pragma unroll
-        for (int p0 = 0; p0 < P; p0 += C::kSlabs) {
+        for (int p0 = 0; p0 < P; ++p0) {
           if (elect && (p0 > 0 || !first)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           meet();
 #pragma unroll
-          for (int k = 0; k < C::kSlabs; ++k)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              *reinterpret_cast<uint4*>(slab + k * kSlabBytes + lane * 128 + (((ch0 + i) ^ row_sw) << 4)) =
-                  make_uint4(u[p0 + k][4 * i], u[p0 + k][4 * i + 1], u[p0 + k][4 * i + 2], u[p0 + k][4 * i + 3]);
+          for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<uint4*>(slab + lane * 128 + (((ch0 + i) ^ row_sw) << 4)) =
+                make_uint4(u[p0][4 * i], u[p0][4 * i + 1], u[p0][4 * i + 2], u[p0][4 * i + 3]);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           meet();
           if (elect) {
-#pragma unroll
-            for (int k = 0; k < C::kSlabs; ++k)
-              bulk_s2g(p.arena + dst + (p0 + k) * p.plane + pt, slab + k * kSlabBytes, kSlabBytes);
+            bulk_s2g(p.arena + dst + p0 * p.plane + pt, slab, kSlabBytes);
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
         }
@@ -555,12 +545,17 @@ __global__ void __launch_bounds__(kThreads, 1) product_chain(const __grid_consta
   if (!ok) atomicOr(p.err, kErrTimeout);
 }
 
+cudaError_t sm_count(int* sms) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
 template <int P>
 cudaError_t launch(const ChainParams& p, int n_work, cudaStream_t s) {
   cudaError_t e;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev))) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
+  int sms = 0;
+  if ((e = sm_count(&sms))) return e;
   if ((e = cudaFuncSetAttribute(product_chain<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<P>::kSmem))) return e;
   void* args[] = {const_cast<ChainParams*>(&p)};
   const dim3 grid(n_work < sms ? n_work : sms);
@@ -573,7 +568,12 @@ cudaError_t launch(const ChainParams& p, int n_work, cudaStream_t s) {
 // Three tiles per SM: a subgraph's next product then starts when the last one's tiles have been two rounds in
 // flight, and the window's matrices (about 260 MB) are partly still in L2.  Measured for 3,415 tiles: windows of
 // 152 tiles 319 us a product, 228: 249, 304: 202, 380: 196, 456: 198, 608: 206, one window: 222.
-int chain_window_tiles() { return 456; }
+cudaError_t chain_window_tiles(int* tiles) {
+  int sms = 0;
+  const cudaError_t e = sm_count(&sms);
+  *tiles = 3 * sms;
+  return e;
+}
 
 cudaError_t launch_chain(const ChainParams& p, int planes, int n_work, int n_sub, cudaStream_t s) {
   if (n_work <= 0 || p.n_ops <= 0) return cudaSuccess;

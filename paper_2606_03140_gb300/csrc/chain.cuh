@@ -39,7 +39,7 @@ struct ChainParams {
 // (n_sub words) when the chain holds more than one product.
 cudaError_t launch_chain(const ChainParams& p, int planes, int n_work, int n_sub, cudaStream_t s);
 
-// Window boundaries for the tiles of subgraphs with tile counts tiles[i] (see chain.cu).
-int chain_window_tiles();
+// About how many tiles a window of subgraphs holds on this device (see chain.cu).
+cudaError_t chain_window_tiles(int* tiles);
 
 }  // namespace sedacs

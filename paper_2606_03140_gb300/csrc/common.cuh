@@ -26,8 +26,9 @@ struct ModelDev {
 constexpr double kBohrA = 0.529177210903;
 constexpr double kAccHaAAmu = 0.2625499639;   // (Ha/A)/amu expressed in A/fs^2
 
-// Bounded spin limit for every device-side wait (cycles; ~0.2 s at 2 GHz).  Legitimate
-// waits of the pipelines here last microseconds.
+// Bounded spin limit for every device-side wait (cycles; ~0.2 s at 2 GHz).  Legitimate waits of the pipelines here
+// last microseconds; those of a chain (chain.cu) for the product before, up to a few times as long as a product of
+// one subgraph takes: well below a millisecond at six tiles a side.
 constexpr long long kWaitLimitCycles = 400000000LL;
 
 // Error flags raised by kernels (OR-ed into a device word, read by the host).

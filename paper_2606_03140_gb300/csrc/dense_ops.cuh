@@ -45,17 +45,18 @@ void launch_split_planes(SlotViews views, int n_sub, int max_rows, uint8_t* aren
 // 128x128 tiles, as the full matrix in three bf16 planes (two launches).
 void launch_f16x2_to_bf16x3(SlotViews views, const Sp2State* st, long long copy_stride, int n_sub, int max_rows,
                             uint8_t* arena, cudaStream_t s);
-// out1 = a1 in + b1 I (kind 0), the SP2 start (kind 1) or its first-order change (kind 2) from
-// the subgraph bounds; optional out2 = a2 in + b2 I.  Each output: master and / or planes
-// (format nsplit).
 // Terms of a sum over core rows: byte distance of a term's master from the result's, and its factor.
 struct RowTerms {
   long long delta[4];
   double a[4];
   int n;
 };
+// y += sum_k a_k x_k over core rows; one_by_one: each term is rounded and added by itself.
 void launch_rows_sum(SlotViews y, const RowTerms& w, bool one_by_one, int n_sub, int max_rows, uint8_t* arena, bool f64,
                      cudaStream_t s);
+// out1 = a1 in + b1 I (kind 0), the SP2 start (kind 1) or its first-order change (kind 2) from
+// the subgraph bounds; optional out2 = a2 in + b2 I.  Each output: master and / or planes
+// (format nsplit).
 void launch_affine_planes(SlotViews in, SlotViews out1, double a1, double b1, int master1, int nsplit1,
                           SlotViews out2, double a2, double b2, int master2, int nsplit2, int kind,
                           const double* bounds, int n_sub, int max_rows, uint8_t* arena, bool f64, cudaStream_t s);

@@ -693,7 +693,9 @@ sedacs_status build_chain_tables(sedacs_ctx* ctx) {
   }
   // windows of whole subgraphs with about equal tile counts
   const int n = (int)tiles.size();
-  const int nw = std::max(1, (n + chain_window_tiles() / 2) / chain_window_tiles());
+  int window = 0;
+  CUCHK(chain_window_tiles(&window));
+  const int nw = std::max(1, (n + window / 2) / window);
   std::vector<int> win(1, 0);
   for (int i = 0; i < L.n_sub; ++i)
     if ((int)win.size() < nw && first[i + 1] > win.back() &&

@@ -12,9 +12,9 @@
 //
 // Cores (Fig. 1b): recursive coordinate bisection of the wrapped coordinates
 // w = x - L * floor(x / L).  The split sizes follow from integers only
-// (floor(c * floor(p/2) / p) atoms take floor(p/2) cores), so the host knows the tree;
-// each level sorts every segment by (w_axis, atom index) along its widest axis (first
-// axis on ties) in one CTA.  Halo (Fig. 1c): graph neighbours of core atoms outside the
+// (floor(c * floor(p/2) / p) atoms take floor(p/2) cores), so the host knows the tree; on each
+// level a CTA per segment selects the atoms that come first by (w_axis, atom index) along its
+// widest axis (first axis on ties), and sorts where too many coincide.  Halo (Fig. 1c): graph neighbours of core atoms outside the
 // core, ascending, from a per-core bitmap.
 #include "graph.cuh"
 
